@@ -135,6 +135,7 @@ static wis::SweepArgs sweep_args(weno_ctx* c, int dir)
     a.dx1 = c->dx[1];
     a.acc_scale = 1.0;
     a.acc_scale_f = 1.0f;
+    a.fx = c->prec == WENO_FP64 && wis::use_fx((long long)interior_cells(c)) ? 1 : 0;
     // a stage sweeps the directions from the last to x: the first one
     // computes and stores the primitives, the others read them
     if (c->use_prims) {

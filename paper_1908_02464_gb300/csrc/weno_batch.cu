@@ -33,7 +33,7 @@ template <> struct BatchTile<1> { static constexpr int SEG = 63, NT = 64; };
 template <> struct BatchTile<2> { static constexpr int SEG = 255, NT = 256; };
 constexpr int kBatchVariants = 3;
 
-template <typename T, int SEG, int NT, bool EXACTDET>
+template <typename T, int SEG, int NT, bool EXACTDET, bool FX>
 __global__ void __launch_bounds__(NT) k_batch(BatchArgs b)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs b)
         a.gamma = b.gamma; a.eps = b.eps; a.c_lambda = b.c_lambda; a.hybrid = b.hybrid;
         a.wmode = b.wmode; a.split = b.split; a.alpha_g = nullptr;
         a.inv_dx_f = (float)(a.inv_dx * (1.0 / 60.0)); a.gamma_f = (float)b.gamma; a.eps_f = (float)b.eps;
+        a.fx = FX && use_fx(n);
         a.slim = sqrt(3600.0 * eps_h);
         a.slim_f = (float)a.slim; a.lam_scale_f = (float)(b.c_lambda * (1.0 / 3600.0));
         const T inv_dx_t[1] = {T(a.inv_dx)};
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs b)
                 a.rk_a = ra[st]; a.rk_b = rb[st];
                 a.rk_a_f = (float)ra[st]; a.rk_b_f = (float)rb[st];
                 for (int tile = 0; tile < ntiles; ++tile)
-                    sbad |= sweep_tile<T, 1, 0, 1, SEG, NT, EXACTDET>(a, tile, 0, 0, dtt, smem_raw);
+                    sbad |= sweep_tile<T, 1, 0, 1, SEG, NT, EXACTDET, false, FX>(a, tile, 0, 0, dtt, smem_raw);
             }
             if (__syncthreads_or(sbad)) { status = WENO_ERR_NONPHYSICAL; break; }
             const int tmp = cur;
@@ -151,12 +152,12 @@ __global__ void __launch_bounds__(NT) k_batch(BatchArgs b)
     }
 }
 
-template <typename T, bool EXACTDET, int V>
+template <typename T, bool EXACTDET, int V, bool FX>
 cudaError_t batch_config(int* blocks_per_sm, size_t* smem)
 {
     using BT = BatchTile<V>;
     using SM = SweepSmem<T, 1, 1, BT::SEG>;
-    auto kern = k_batch<T, BT::SEG, BT::NT, EXACTDET>;
+    auto kern = k_batch<T, BT::SEG, BT::NT, EXACTDET, FX>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -165,12 +166,12 @@ cudaError_t batch_config(int* blocks_per_sm, size_t* smem)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, BT::NT, SM::bytes);
 }
 
-template <typename T, bool EXACTDET, int V>
+template <typename T, bool EXACTDET, int V, bool FX>
 cudaError_t batch_launch(const BatchArgs& b, int blocks, cudaStream_t s)
 {
     using BT = BatchTile<V>;
     using SM = SweepSmem<T, 1, 1, BT::SEG>;
-    k_batch<T, BT::SEG, BT::NT, EXACTDET><<<blocks, BT::NT, SM::bytes, s>>>(b);
+    k_batch<T, BT::SEG, BT::NT, EXACTDET, FX><<<blocks, BT::NT, SM::bytes, s>>>(b);
     return cudaGetLastError();
 }
 
@@ -204,6 +205,7 @@ struct weno_batch {
     unsigned long long* wcount = nullptr;
     int* trial_caps = nullptr;
     std::vector<int> n_host;      // steps grow with this size: n (1D), max(nx, ny) (2D)
+    bool fx = false;              // an FP64 instance takes the integer six-point sums
     int variant = 0;
     int blocks = 0;
     cudaGraphExec_t graph = nullptr;
@@ -222,34 +224,44 @@ static std::string g_batch_err;
         }                                                                                   \
     } while (0)
 
-static cudaError_t batch_dispatch_config(int dim, int prec, int v, int* bps, size_t* smem)
+// fx: an FP64 batch with an instance large enough for the integer six-point
+// sums (use_fx); other batches keep the leaner kernel
+template <typename T, bool EXACTDET, bool FX>
+static cudaError_t batch_config_v(int v, int* bps, size_t* smem)
 {
     using namespace wis;
-    if (dim == 2) return batch2d_config(prec, v, bps, smem);
-    if (prec == WENO_FP64) {
-        if (v == 1) return batch_config<double, false, 1>(bps, smem);
-        if (v == 2) return batch_config<double, false, 2>(bps, smem);
-        return batch_config<double, false, 0>(bps, smem);
-    }
-    const bool ex = prec == WENO_MIXED;
-    if (v == 1) return ex ? batch_config<float, true, 1>(bps, smem) : batch_config<float, false, 1>(bps, smem);
-    if (v == 2) return ex ? batch_config<float, true, 2>(bps, smem) : batch_config<float, false, 2>(bps, smem);
-    return ex ? batch_config<float, true, 0>(bps, smem) : batch_config<float, false, 0>(bps, smem);
+    if (v == 1) return batch_config<T, EXACTDET, 1, FX>(bps, smem);
+    if (v == 2) return batch_config<T, EXACTDET, 2, FX>(bps, smem);
+    return batch_config<T, EXACTDET, 0, FX>(bps, smem);
 }
 
-static cudaError_t batch_dispatch_launch(int dim, int prec, int v, const BatchArgs& b, int blocks, cudaStream_t s)
+template <typename T, bool EXACTDET, bool FX>
+static cudaError_t batch_launch_v(int v, const BatchArgs& b, int blocks, cudaStream_t s)
 {
     using namespace wis;
-    if (dim == 2) return batch2d_launch(prec, v, b, blocks, s);
-    if (prec == WENO_FP64) {
-        if (v == 1) return batch_launch<double, false, 1>(b, blocks, s);
-        if (v == 2) return batch_launch<double, false, 2>(b, blocks, s);
-        return batch_launch<double, false, 0>(b, blocks, s);
-    }
-    const bool ex = prec == WENO_MIXED;
-    if (v == 1) return ex ? batch_launch<float, true, 1>(b, blocks, s) : batch_launch<float, false, 1>(b, blocks, s);
-    if (v == 2) return ex ? batch_launch<float, true, 2>(b, blocks, s) : batch_launch<float, false, 2>(b, blocks, s);
-    return ex ? batch_launch<float, true, 0>(b, blocks, s) : batch_launch<float, false, 0>(b, blocks, s);
+    if (v == 1) return batch_launch<T, EXACTDET, 1, FX>(b, blocks, s);
+    if (v == 2) return batch_launch<T, EXACTDET, 2, FX>(b, blocks, s);
+    return batch_launch<T, EXACTDET, 0, FX>(b, blocks, s);
+}
+
+static cudaError_t batch_dispatch_config(int dim, int prec, bool fx, int v, int* bps, size_t* smem)
+{
+    if (dim == 2) return wis::batch2d_config(prec, fx, v, bps, smem);
+    if (prec == WENO_FP64)
+        return fx ? batch_config_v<double, false, true>(v, bps, smem) : batch_config_v<double, false, false>(v, bps, smem);
+    return prec == WENO_MIXED ? batch_config_v<float, true, false>(v, bps, smem)
+                              : batch_config_v<float, false, false>(v, bps, smem);
+}
+
+static cudaError_t batch_dispatch_launch(int dim, int prec, bool fx, int v, const BatchArgs& b, int blocks,
+                                         cudaStream_t s)
+{
+    if (dim == 2) return wis::batch2d_launch(prec, fx, v, b, blocks, s);
+    if (prec == WENO_FP64)
+        return fx ? batch_launch_v<double, false, true>(v, b, blocks, s)
+                  : batch_launch_v<double, false, false>(v, b, blocks, s);
+    return prec == WENO_MIXED ? batch_launch_v<float, true, false>(v, b, blocks, s)
+                              : batch_launch_v<float, false, false>(v, b, blocks, s);
 }
 
 static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_back)
@@ -280,7 +292,7 @@ static weno_status set_variant(weno_batch* bt, int v, int blocks_per_sm_cap)
 {
     int bps = 0;
     size_t smem = 0;
-    BCK(batch_dispatch_config(bt->dim, bt->prec, v, &bps, &smem));
+    BCK(batch_dispatch_config(bt->dim, bt->prec, bt->fx, v, &bps, &smem));
     if (bps < 1) { bt->err = "batch kernel cannot be resident"; return WENO_ERR_CUDA; }
     if (blocks_per_sm_cap > 0 && bps > blocks_per_sm_cap) bps = blocks_per_sm_cap;
     bt->variant = v;
@@ -300,7 +312,7 @@ static cudaError_t enqueue_run(weno_batch* bt, void* U, int max_steps, int write
     if (e != cudaSuccess) return e;
     BatchArgs b = batch_args(bt, U, max_steps, write_back);
     b.trial_caps = trial_caps;
-    return batch_dispatch_launch(bt->dim, bt->prec, bt->variant, b, bt->blocks, s);
+    return batch_dispatch_launch(bt->dim, bt->prec, bt->fx, bt->variant, b, bt->blocks, s);
 }
 
 static void batch_free(weno_batch* bt)
@@ -395,6 +407,7 @@ weno_status weno_batch_create(const weno_batch_desc* d, const weno_params* param
     alloc((void**)&bt->wcount, sizeof(unsigned long long));
     alloc((void**)&bt->trial_caps, sizeof(int) * cnt);
     bt->n_host.assign(d->n, d->n + cnt);
+    for (int i = 0; i < cnt; ++i) bt->fx = bt->fx || (bt->prec == WENO_FP64 && wis::use_fx(d->n[i]));
     if (e == cudaSuccess) e = cudaMemcpy(bt->order, order.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(bt->n, d->n, sizeof(int) * cnt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(bt->off, off.data(), sizeof(long long) * cnt, cudaMemcpyHostToDevice);
@@ -512,6 +525,8 @@ weno_status weno_batch2d_create(const weno_batch2d_desc* d, const weno_params* p
     alloc((void**)&bt->wcount, sizeof(unsigned long long));
     alloc((void**)&bt->trial_caps, sizeof(int) * cnt);
     bt->n_host = lin;
+    for (int i = 0; i < cnt; ++i)
+        bt->fx = bt->fx || (bt->prec == WENO_FP64 && wis::use_fx((long long)d->nx[i] * d->ny[i]));
     if (e == cudaSuccess) e = cudaMemcpy(bt->order, order.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(bt->n, d->nx, sizeof(int) * cnt, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(bt->ny, d->ny, sizeof(int) * cnt, cudaMemcpyHostToDevice);
@@ -654,7 +669,7 @@ weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_ste
     if (ce == cudaSuccess) {
         BatchArgs b = batch_args(bt, Us, bt->max_steps, 1);
         b.t_end = t_half;
-        ce = batch_dispatch_launch(bt->dim, bt->prec, bt->variant, b, bt->blocks, bt->stream);
+        ce = batch_dispatch_launch(bt->dim, bt->prec, bt->fx, bt->variant, b, bt->blocks, bt->stream);
     }
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(bt->stream);
     cudaFree(t_half);

@@ -38,7 +38,7 @@ struct BatchArgs {
 
 // 2D batch kernel variants (weno_batch2d.cu); v in [0, kBatch2Variants)
 constexpr int kBatch2Variants = 3;
-cudaError_t batch2d_config(int prec, int v, int* blocks_per_sm, size_t* smem);
-cudaError_t batch2d_launch(int prec, int v, const BatchArgs& b, int blocks, cudaStream_t s);
+cudaError_t batch2d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem);
+cudaError_t batch2d_launch(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s);
 
 }  // namespace wis

@@ -66,7 +66,7 @@ __device__ __forceinline__ void batch2d_dir_args(const BatchArgs& b, int d, int 
     a.xs_fixed = 0.0;
 }
 
-template <typename T, int V, bool EXACTDET>
+template <typename T, int V, bool EXACTDET, bool FX>
 __global__ void __launch_bounds__(Batch2Tile<V>::NT) k_batch2d(BatchArgs b)
 {
     using BT = Batch2Tile<V>;
@@ -96,6 +96,7 @@ __global__ void __launch_bounds__(Batch2Tile<V>::NT) k_batch2d(BatchArgs b)
         SweepArgs ax, ay;
         batch2d_dir_args(b, 0, nx, ny, dx, ax);
         batch2d_dir_args(b, 1, nx, ny, dy, ay);
+        ax.fx = ay.fx = FX && use_fx(cells);
         ay.mode = MODE_ACC_SET;
         ay.acc = acc;
         ax.mode = MODE_COMBINE;
@@ -149,7 +150,7 @@ __global__ void __launch_bounds__(Batch2Tile<V>::NT) k_batch2d(BatchArgs b)
                 ay.U = W[in_[st]];
                 for (int tile = 0; tile < nsy * nly; ++tile) {
                     const int seg = tile % nsy, lg = tile / nsy;
-                    sweep_tile<T, 2, 1, BT::YL, BT::YS, NT, EXACTDET>(ay, seg, lg * BT::YL, 0, dtt, smem_raw);
+                    sweep_tile<T, 2, 1, BT::YL, BT::YS, NT, EXACTDET, false, FX>(ay, seg, lg * BT::YL, 0, dtt, smem_raw);
                 }
                 ax.U = W[in_[st]];
                 ax.Un = W[cur];
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(Batch2Tile<V>::NT) k_batch2d(BatchArgs b)
                 ax.rk_a_f = (float)ra[st]; ax.rk_b_f = (float)rb[st];
                 for (int tile = 0; tile < nsx * nlx; ++tile) {
                     const int seg = tile % nsx, lg = tile / nsx;
-                    sbad |= sweep_tile<T, 2, 0, BT::XL, BT::XS, NT, EXACTDET>(ax, seg, lg * BT::XL, 0, dtt,
+                    sbad |= sweep_tile<T, 2, 0, BT::XL, BT::XS, NT, EXACTDET, false, FX>(ax, seg, lg * BT::XL, 0, dtt,
                                                                               smem_raw);
                 }
             }
@@ -180,11 +181,11 @@ __global__ void __launch_bounds__(Batch2Tile<V>::NT) k_batch2d(BatchArgs b)
     }
 }
 
-template <typename T, bool EXACTDET, int V>
+template <typename T, bool EXACTDET, bool FX, int V>
 static cudaError_t config_v(int* blocks_per_sm, size_t* smem)
 {
     using SM = Batch2Smem<T, V>;
-    auto kern = k_batch2d<T, V, EXACTDET>;
+    auto kern = k_batch2d<T, V, EXACTDET, FX>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
@@ -193,41 +194,44 @@ static cudaError_t config_v(int* blocks_per_sm, size_t* smem)
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, Batch2Tile<V>::NT, SM::bytes);
 }
 
-template <typename T, bool EXACTDET, int V>
+template <typename T, bool EXACTDET, bool FX, int V>
 static cudaError_t launch_v(const BatchArgs& b, int blocks, cudaStream_t s)
 {
-    k_batch2d<T, V, EXACTDET><<<blocks, Batch2Tile<V>::NT, Batch2Smem<T, V>::bytes, s>>>(b);
+    k_batch2d<T, V, EXACTDET, FX><<<blocks, Batch2Tile<V>::NT, Batch2Smem<T, V>::bytes, s>>>(b);
     return cudaGetLastError();
 }
 
-template <typename T, bool EXACTDET>
+template <typename T, bool EXACTDET, bool FX>
 static cudaError_t config_t(int v, int* bps, size_t* smem)
 {
-    if (v == 1) return config_v<T, EXACTDET, 1>(bps, smem);
-    if (v == 2) return config_v<T, EXACTDET, 2>(bps, smem);
-    return config_v<T, EXACTDET, 0>(bps, smem);
+    if (v == 1) return config_v<T, EXACTDET, FX, 1>(bps, smem);
+    if (v == 2) return config_v<T, EXACTDET, FX, 2>(bps, smem);
+    return config_v<T, EXACTDET, FX, 0>(bps, smem);
 }
 
-template <typename T, bool EXACTDET>
+template <typename T, bool EXACTDET, bool FX>
 static cudaError_t launch_t(int v, const BatchArgs& b, int blocks, cudaStream_t s)
 {
-    if (v == 1) return launch_v<T, EXACTDET, 1>(b, blocks, s);
-    if (v == 2) return launch_v<T, EXACTDET, 2>(b, blocks, s);
-    return launch_v<T, EXACTDET, 0>(b, blocks, s);
+    if (v == 1) return launch_v<T, EXACTDET, FX, 1>(b, blocks, s);
+    if (v == 2) return launch_v<T, EXACTDET, FX, 2>(b, blocks, s);
+    return launch_v<T, EXACTDET, FX, 0>(b, blocks, s);
 }
 
-cudaError_t batch2d_config(int prec, int v, int* blocks_per_sm, size_t* smem)
+cudaError_t batch2d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem)
 {
-    if (prec == WENO_FP64) return config_t<double, false>(v, blocks_per_sm, smem);
-    if (prec == WENO_MIXED) return config_t<float, true>(v, blocks_per_sm, smem);
-    return config_t<float, false>(v, blocks_per_sm, smem);
+    if (prec == WENO_FP64)
+        return fx ? config_t<double, false, true>(v, blocks_per_sm, smem)
+                  : config_t<double, false, false>(v, blocks_per_sm, smem);
+    if (prec == WENO_MIXED) return config_t<float, true, false>(v, blocks_per_sm, smem);
+    return config_t<float, false, false>(v, blocks_per_sm, smem);
 }
 
-cudaError_t batch2d_launch(int prec, int v, const BatchArgs& b, int blocks, cudaStream_t s)
+cudaError_t batch2d_launch(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s)
 {
-    if (prec == WENO_FP64) return launch_t<double, false>(v, b, blocks, s);
-    if (prec == WENO_MIXED) return launch_t<float, true>(v, b, blocks, s);
-    return launch_t<float, false>(v, b, blocks, s);
+    if (prec == WENO_FP64)
+        return fx ? launch_t<double, false, true>(v, b, blocks, s) : launch_t<double, false, false>(v, b, blocks, s);
+    if (prec == WENO_MIXED) return launch_t<float, true, false>(v, b, blocks, s);
+    return launch_t<float, false, false>(v, b, blocks, s);
 }
 
 }  // namespace wis

@@ -100,6 +100,93 @@ template <> struct Ar<float> {
     static __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 };
 
+// ------------------------------------------- six-point sums on the integer pipes
+// The two fixed linear combinations of a face's six stencil values, the
+// detector difference (Eq. eq28) and the central flux (Eq. linearupwind), take
+// 5 FP64 instructions per variable each.  GB300 issues 2 FP64 lanes per SM and
+// clock but 64 integer lanes, and the FP64 sweeps leave 90% of the issue slots
+// idle, so in FP64 both sums are formed in 64-bit integers instead: the six
+// significands are aligned to the largest exponent with G guard bits and the
+// integer sum is exact, then rounded once to double.  A value whose exponent
+// lies up to G below the largest keeps every bit (the whole sum is then exact
+// before its one rounding); beyond that, bits below 2^-(52+G) of the largest
+// value are dropped, which bounds the error by 2^-52 of the largest value.  The FP64 form
+// rounds four times.  Alignment, sum and rounding act on magnitudes, so a
+// mirrored or negated stencil gives the mirrored or negated sum exactly.
+template <int G>
+__device__ __forceinline__ void fx_align(const double* x, long long* v, int& eh)
+{
+    int hi[6];
+    int m = 0;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        hi[i] = __double2hiint(x[i]);
+        m = max(m, hi[i] & 0x7fffffff);
+    }
+    eh = m | 0x000fffff;   // the largest exponent field, ones below it
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        // eh - |hi| = (difference of the exponent fields) * 2^20 + non-negative rest
+        const int s = min((eh - (hi[i] & 0x7fffffff)) >> 20, 63);
+        const unsigned mh = ((unsigned)hi[i] & 0x000fffffu) | 0x00100000u;
+        const unsigned long long mag =
+            ((((unsigned long long)mh << 32) | (unsigned)__double2loint(x[i])) << G) >> s;
+        const long long sg = hi[i] >> 31;
+        v[i] = ((long long)mag ^ sg) - sg;
+    }
+}
+
+// r 2^(E - 1075 - G) rounded to nearest, E the exponent field in eh.  Zero for
+// a zero sum, for stencils of zeros and subnormals (E = 0) and for results
+// below the smallest normal number; NaN if a value is infinite or NaN;
+// infinity on overflow.
+template <int G>
+__device__ __forceinline__ double fx_round(long long r, int eh)
+{
+    const int sg = (int)(r >> 63);
+    unsigned long long a = (unsigned long long)((r ^ (long long)sg) - (long long)sg);
+    const int E = eh >> 20;
+    const int n = __clzll((long long)a) - 1;   // |r| < 2^63
+    const int field = E - n + (10 - G);
+    const bool none = a == 0ull || E == 0 || field <= 0;
+    a = ((a << (n & 63)) + 0x200ull) >> 10;
+    int h = (int)(a >> 32) + ((field - 1) << 20);
+    int l = (int)a;
+    if (field >= 0x7ff) { h = 0x7ff00000; l = 0; }
+    if (none) { h = 0; l = 0; }
+    if (E == 0x7ff) { h = 0x7ff80000; l = 0; }
+    return __hiloint2double(h | (sg & (int)0x80000000), l);
+}
+
+// guard bits of the two sums: sum |coefficients| = 32 and 92, so that
+// 53 + G bits and the growth of the sum stay below 63
+constexpr int FX_GD = 5, FX_GC = 3;
+
+// x0 - 5 x1 + 10 x2 - 10 x3 + 5 x4 - x5
+__device__ __forceinline__ long long fx_fifth(const long long* v)
+{
+    return (v[0] - v[5]) + 5 * ((v[4] - v[1]) + 2 * (v[2] - v[3]));
+}
+// x0 - 8 x1 + 37 x2 + 37 x3 - 8 x4 + x5
+__device__ __forceinline__ long long fx_central(const long long* v)
+{
+    return (v[0] + v[5]) - 8 * (v[1] + v[4]) + 37 * (v[2] + v[3]);
+}
+__device__ __forceinline__ double fx_detector(const double* x)
+{
+    long long v[6];
+    int eh;
+    fx_align<FX_GD>(x, v, eh);
+    return fx_round<FX_GD>(fx_fifth(v), eh);
+}
+__device__ __forceinline__ double fx_central_flux(const double* x)
+{
+    long long v[6];
+    int eh;
+    fx_align<FX_GC>(x, v, eh);
+    return fx_round<FX_GC>(fx_central(v), eh);
+}
+
 // ------------------------------------------------------------- cell records
 // Per-cell quantities kept in shared memory for a sweep along direction DIR.
 // Record layout (NQ entries): U[NV], F[NV], sqrt(rho) u[DIM], sqrt(rho) H,

@@ -116,7 +116,19 @@ struct SweepArgs {
     // an ACC_ADD accumulator is already scaled (1).
     double acc_scale = 1.0;
     float acc_scale_f = 1.0f;
+    int fx = 0;   // FP64: the six-point sums in 64-bit integers (use_fx)
 };
+
+// FP64 problems of at least this many cells form their six-point sums on the
+// integer pipes (fx_detector, fx_central_flux), in the grid solver and in the
+// batches alike, so that both give the same bits.  There the FP64 pipe bounds
+// the sweeps: double Mach 2048 x 512 RK3 step 2.21 -> 1.72 ms, 512 x 128 (the
+// next smaller size measured) 0.346 -> 0.304 ms.  A few thousand cells do not
+// fill the pipe, the longer integer sequence gains little (Sod, 200 cells:
+// 5%), and the whole runs of thousands of such instances in one batch keep
+// the FP64 form.
+constexpr long long kFxMinCells = 32768;
+__host__ __device__ inline bool use_fx(long long cells) { return cells >= kFxMinCells; }
 
 template <typename T> __device__ __forceinline__ T pick(double d, float f);
 template <> __device__ __forceinline__ double pick<double>(double d, float) { return d; }
@@ -301,7 +313,9 @@ __device__ __forceinline__ T fifth_difference(T u0, T u1, T u2, T u3, T u4, T u5
 // nd + 1 faces each), starting at face seg_blk * SEG: every tile computes a
 // full set of faces, and a tile that reaches the end of a line continues on
 // the next one, each piece with its own halo.  line0 and pb are unused then.
-template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false>
+// FX: a.fx may ask for the integer six-point sums (FP64).
+template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false,
+          bool FX = sizeof(T) == 8>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int line0, int pb, T dt,
                                            unsigned char* smem_raw)
 {
@@ -481,7 +495,10 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
                 const T u3 = cq[k * NCELL + cidx(l, p + 3)];
                 const T u4 = cq[k * NCELL + cidx(l, p + 4)];
                 const T u5 = cq[k * NCELL + cidx(l, p + 5)];
-                if (EXACTDET) dU[v] = -fifth_difference(u0, u1, u2, u3, u4, u5);
+                if (FX && a.fx) {
+                    const double x[6] = {u0, u1, u2, u3, u4, u5};
+                    dU[v] = T(fx_detector(x));
+                } else if (EXACTDET) dU[v] = -fifth_difference(u0, u1, u2, u3, u4, u5);
                 else dU[v] = fmaT(T(10), u2 - u3, fmaT(T(5), u4 - u1, u0 - u5));
             }
             T w[NV];
@@ -519,10 +536,17 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     const int k = CL::F + v;
-                    const T f05 = cq[k * NCELL + cidx(l, p + 0)] + cq[k * NCELL + cidx(l, p + 5)];
-                    const T f14 = cq[k * NCELL + cidx(l, p + 1)] + cq[k * NCELL + cidx(l, p + 4)];
-                    const T f23 = cq[k * NCELL + cidx(l, p + 2)] + cq[k * NCELL + cidx(l, p + 3)];
-                    Fo[v] = fmaT(T(37), f23, fmaT(T(-8), f14, f05));
+                    if (FX && a.fx) {
+                        double x[6];
+#pragma unroll
+                        for (int m = 0; m < 6; ++m) x[m] = cq[k * NCELL + cidx(l, p + m)];
+                        Fo[v] = T(fx_central_flux(x));
+                    } else {
+                        const T f05 = cq[k * NCELL + cidx(l, p + 0)] + cq[k * NCELL + cidx(l, p + 5)];
+                        const T f14 = cq[k * NCELL + cidx(l, p + 1)] + cq[k * NCELL + cidx(l, p + 4)];
+                        const T f23 = cq[k * NCELL + cidx(l, p + 2)] + cq[k * NCELL + cidx(l, p + 3)];
+                        Fo[v] = fmaT(T(37), f23, fmaT(T(-8), f14, f05));
+                    }
                 }
                 ups_dissipation_add<T, DIM, DIR>(r, dU, w, am, a0, ap, Fo);
                 // face fluxes are kept times 60; the divergence scales by dx/60
