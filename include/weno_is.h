@@ -241,8 +241,8 @@ weno_status weno_conserved_totals(weno_ctx* ctx, double* totals);
  * Each instance i is a 1D Euler problem on [lo[i], hi[i]] with n[i] cells,
  * advanced from t = 0 to t_end[i] with its own CFL step (same scheme and
  * constants as weno_params), in one persistent launch replayed from a CUDA
- * graph: every CTA takes the next instance from a work queue ordered
- * largest first and runs its whole RK3 loop (Sec. 4) on its own.
+ * graph: the CTAs take runs of tiles of the instances' sweeps from a work
+ * queue, each instance's next sweep entering it when its last one is done.
  * ---------------------------------------------------------------------- */
 typedef struct {
     int count;              /* number of instances (>= 1)                      */
@@ -257,7 +257,7 @@ typedef struct {
 typedef struct weno_batch weno_batch;
 
 /* Create a batch: copies the description, orders the instances largest
- * first, allocates three ghosted work arrays per instance.  States are passed
+ * first, allocates three work arrays per instance and the task queue.  States are passed
  * to weno_batch_run as one device array holding the instances back to back,
  * instance i as [3][n[i]] (rho, rho u, E) starting at element 3 sum_{j<i} n[j]
  * (double for WENO_FP64, float otherwise).  Errors: WENO_ERR_INVALID_ARG for
@@ -274,11 +274,13 @@ weno_status weno_batch_run(weno_batch* batch, void* U_dev);
 /* Per-instance results of the last run (host arrays of count entries, each
  * may be NULL): status (0 ok, WENO_ERR_NONPHYSICAL: the instance stopped at
  * its last admissible step), completed steps and reached time.
- * Synchronizes; returns WENO_ERR_NONPHYSICAL if any instance failed. */
+ * Synchronizes; returns WENO_ERR_NONPHYSICAL if any instance failed,
+ * WENO_ERR_TIMEOUT if a CTA's bounded wait for its next task ran out (the
+ * run's states are then not valid). */
 weno_status weno_batch_results(weno_batch* batch, int* status, long long* steps, double* t);
 
 /* Autotuner (no counterpart in the paper): times trial runs for each CTA
- * size (64, 128, 256 threads: tiles of 63, 127, 255 faces) and residency
+ * size (64, 128, 256 threads: tiles of 59, 123, 251 faces) and residency
  * (all that fit, 4 or 2 CTAs per SM) and keeps the fastest.  U_dev is not
  * modified.  The trials start from a scratch copy of U_dev advanced with
  * the current configuration to half of each instance's end time: the cost
@@ -289,15 +291,16 @@ weno_status weno_batch_results(weno_batch* batch, int* status, long long* steps,
  * one): a full run's step count grows with the cell count, so the trial
  * keeps the full run's work per instance, growing like N_i^2, and with it
  * the load balance of the schedule.  choice[0] = tile variant, choice[1] =
- * CTAs launched.  The per-instance results afterwards are those of the last
+ * the number weno_batch_set_config reports.  The per-instance results afterwards are those of the last
  * trial.  Synchronizes. */
 weno_status weno_batch_autotune(weno_batch* batch, const void* U_dev, int trial_steps, int* choice);
 
 /* Fixes the configuration without timing (no counterpart in the paper):
- * variant 0, 1, 2 = 128-, 64-, 256-thread CTAs (tiles of 127, 63, 255
+ * variant 0, 1, 2 = 128-, 64-, 256-thread CTAs (tiles of 123, 59, 251
  * faces); blocks_per_sm = resident CTAs per SM, 0 = as many as fit (values
- * above that are lowered to it).  *blocks (may be NULL) receives the CTAs a
- * run launches: min(count, residency x SMs).  WENO_ERR_INVALID_ARG for a
+ * above that are lowered to it).  *blocks (may be NULL) receives min(count,
+ * residency x SMs), the instances that can have a task in work at once at
+ * the most; a run launches min(tiles, residency x SMs) CTAs.  WENO_ERR_INVALID_ARG for a
  * variant outside 0..2 or a negative blocks_per_sm. */
 weno_status weno_batch_set_config(weno_batch* batch, int variant, int blocks_per_sm, int* blocks);
 
@@ -315,9 +318,9 @@ const char* weno_batch_last_error(const weno_batch* batch);
  * with nx[i] x ny[i] cells, advanced from t = 0 to t_end[i] with its own CFL
  * step (dt = CFL / max (|u| + c)/dx + (|v| + c)/dy, Sec. 4) by the same
  * dimension-by-dimension scheme as weno_step (Sec. 2.4, Eq. goveq5), in one
- * persistent launch replayed from a CUDA graph: every CTA takes the next
- * instance from a work queue ordered by nx ny max(nx, ny) (cells x steps),
- * largest first, and runs its whole RK3 loop on its own.  Each stage is the
+ * persistent launch replayed from a CUDA graph: the CTAs take runs of tiles
+ * of the instances' sweeps from a work queue, which the instances enter by
+ * nx ny max(nx, ny) (cells x steps), largest first.  Each stage is the
  * y sweep (flux divergence into an accumulator) followed by the x sweep
  * (its divergence plus the RK3 combination), as in the grid solver, whose
  * results the batch reproduces bit for bit.

@@ -1,19 +1,9 @@
-// Batched solver: many independent Euler problems of uneven sizes, each
-// advanced to its own end time with its own CFL step, in one persistent
-// launch replayed from a CUDA graph.  This file holds the 1D kernel and the
-// host object shared with the 2D kernel of weno_batch2d.cu.
-//
-// Each CTA pulls an instance from a work queue (instances ordered largest
-// first, so the tail of the schedule holds the small ones), copies it into
-// three work arrays that stay L2-resident while it is being solved, and runs
-// the whole RK3 loop (Sec. 4 of the paper) with block-level barriers only:
-// CFL max-reduction, then per stage a chain of sweep tiles (the same
-// per-tile code as the grid solver, which takes the ghost cells from the
-// boundary conditions while staging, so every face is computed by identical
-// arithmetic).  No CTA ever waits on another.
+// Batched solver: the host object of the persistent batch kernel
+// (weno_batch.cuh) for 1D and 2D instances, and the 1D instantiations.
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -23,156 +13,39 @@
 
 #include "../../include/weno_is.h"
 #include "weno_batch.cuh"
-#include "weno_kernels.cuh"
 
 namespace wis {
 
-template <int V> struct BatchTile;
-template <> struct BatchTile<0> { static constexpr int SEG = 127, NT = 128; };
-template <> struct BatchTile<1> { static constexpr int SEG = 63, NT = 64; };
-template <> struct BatchTile<2> { static constexpr int SEG = 255, NT = 256; };
-constexpr int kBatchVariants = 3;
+// Line tiles on 128, 64 and 256 threads (LineTile).  1024 Riemann problems of
+// 100 to 2000 cells in FP64: 64, 68 and 65 ms, with the FP64 pipe 85% busy
+// over the first steps (one CTA per instance: 125, 192 and 75 ms, the
+// heaviest instance alone 80 ms against 12 ms here); 4096 of 100 to 4000
+// cells in FP32: 147, 146 and 167 ms (231, 380 and 146 ms), issue 56% of the
+// cycles and the shared-memory data path 67%.  128 threads are the default.
+// Runs of 8 tiles: with single-tile tasks and a lane-by-lane queue the FP32
+// batch took 202 ms.
+template <int V>
+struct Batch1Cfg {
+    static constexpr int NT = V == 0 ? 128 : (V == 1 ? 64 : 256);
+    static constexpr int XS = NT - 6, XL = 1, YL = 1, YS = 1;
+    static constexpr int RUN = 8;
+    template <typename T> static constexpr size_t smem_bytes() { return LineTile<T, NT>::bytes; }
+    template <typename T> static constexpr int min_blocks() { return (sizeof(T) == 8 ? 640 : 1024) / NT; }
+};
 
-template <typename T, int SEG, int NT, bool EXACTDET, bool FX>
-__global__ void __launch_bounds__(NT) k_batch(BatchArgs b)
+cudaError_t batch1d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ int s_inst;
-    __shared__ double s_red[NT / 32];
-    __shared__ double s_dt;
-    __shared__ int s_flag;
-    const T gamma = T(b.gamma);
-    for (;;) {
-        if (threadIdx.x == 0) {
-            const unsigned int k = atomicAdd(b.head, 1u);
-            s_inst = k < (unsigned int)b.count ? b.order[k] : -1;
-        }
-        __syncthreads();
-        const int inst = s_inst;
-        if (inst < 0) return;
-        const int n = b.n[inst];
-        const long long sv = n + 6;
-        T* W[3] = {reinterpret_cast<T*>(b.work0) + b.goff[inst], reinterpret_cast<T*>(b.work1) + b.goff[inst],
-                   reinterpret_cast<T*>(b.work2) + b.goff[inst]};
-        T* Ui = reinterpret_cast<T*>(b.U) + b.off[inst];
-        for (int i = threadIdx.x; i < n; i += NT)
-#pragma unroll
-            for (int v = 0; v < 3; ++v) W[0][3 + v * sv + i] = Ui[(long long)v * n + i];
-        const double dx = b.dx[inst], t_end = b.t_end[inst];
-        // Eq. eq31
-        double eps_h = b.C_thr;
-        for (int k = 0; k < b.alpha_thr; ++k) eps_h *= dx / b.L_char;
-
-        SweepArgs a;
-        a.bc_lo = b.bc_lo;   // the tiles take their ghost cells from these
-        a.bc_hi = b.bc_hi;
-        a.acc = nullptr;
-        a.mode = MODE_COMBINE;
-        a.tm = nullptr;
-        a.weno_count = b.weno_count;
-        a.flags = nullptr;
-        a.n[0] = n; a.n[1] = 1; a.n[2] = 1;
-        a.sy = sv; a.sz = sv; a.sv = sv; a.off0 = 3;
-        a.inv_dx = 1.0 / dx;
-        a.eps_h = eps_h;
-        a.gamma = b.gamma; a.eps = b.eps; a.c_lambda = b.c_lambda; a.hybrid = b.hybrid;
-        a.wmode = b.wmode; a.split = b.split; a.alpha_g = nullptr;
-        a.inv_dx_f = (float)(a.inv_dx * (1.0 / 60.0)); a.gamma_f = (float)b.gamma; a.eps_f = (float)b.eps;
-        a.fx = FX && use_fx(n);
-        a.slim = sqrt(3600.0 * eps_h);
-        a.slim_f = (float)a.slim; a.lam_scale_f = (float)(b.c_lambda * (1.0 / 3600.0));
-        const T inv_dx_t[1] = {T(a.inv_dx)};
-        const int ntiles = (n + SEG - 1) / SEG;
-
-        int cur = 0, x = 1, y = 2;
-        double t = 0.0;
-        long long steps = 0;
-        int status = 0;
-        __syncthreads();
-        const long long max_steps = b.trial_caps != nullptr ? (long long)b.trial_caps[inst] : (long long)b.max_steps;
-        while (steps < max_steps) {
-            // CFL max-reduction (same per-cell arithmetic as the grid solver)
-            double smax = 0.0;
-            bool bad = false;
-            for (int i = threadIdx.x; i < n; i += NT) {
-                T u[3];
-#pragma unroll
-                for (int v = 0; v < 3; ++v) u[v] = W[cur][3 + v * sv + i];
-                T s;
-                if (!cell_speed<T, 1>(u, gamma, inv_dx_t, s)) bad = true;
-                else smax = maxT(smax, (double)s);
-            }
-            smax = warp_max(smax);
-            if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = smax;
-            const int anybad = __syncthreads_or(bad);
-            if (threadIdx.x == 0) {
-                double m = 0.0;
-                for (int w = 0; w < NT / 32; ++w) m = maxT(m, s_red[w]);
-                int clipped = 0;
-                s_dt = anybad ? 0.0 : cfl_step(b.cfl, m, t, t_end, &clipped);
-                s_flag = clipped;
-            }
-            __syncthreads();
-            const double dt = s_dt;
-            const int clipped = s_flag;
-            if (anybad) { status = WENO_ERR_NONPHYSICAL; break; }
-            if (!(dt > 0.0)) break;
-            const T dtt = T(dt);
-            // three stages: x = cur + dt L(cur); y = 3/4 cur + 1/4 (x + dt L(x));
-            // x = 1/3 cur + 2/3 (y + dt L(y))
-            const int in_[3] = {cur, x, y}, out_[3] = {x, y, x};
-            const double ra[3] = {0.0, 0.75, 1.0 / 3.0}, rb[3] = {1.0, 0.25, 2.0 / 3.0};
-            bool sbad = false;
-            for (int st = 0; st < 3; ++st) {
-                a.U = W[in_[st]];
-                a.Un = W[cur];
-                a.out = W[out_[st]];
-                a.rk_a = ra[st]; a.rk_b = rb[st];
-                a.rk_a_f = (float)ra[st]; a.rk_b_f = (float)rb[st];
-                for (int tile = 0; tile < ntiles; ++tile)
-                    sbad |= sweep_tile<T, 1, 0, 1, SEG, NT, EXACTDET, false, FX>(a, tile, 0, 0, dtt, smem_raw);
-            }
-            if (__syncthreads_or(sbad)) { status = WENO_ERR_NONPHYSICAL; break; }
-            const int tmp = cur;
-            cur = x;
-            x = tmp;
-            t = clipped ? t_end : t + dt;
-            ++steps;
-        }
-        if (b.write_back)
-            for (int i = threadIdx.x; i < n; i += NT)
-#pragma unroll
-                for (int v = 0; v < 3; ++v) Ui[(long long)v * n + i] = W[cur][3 + v * sv + i];
-        if (threadIdx.x == 0) {
-            b.status[inst] = status;
-            b.steps[inst] = steps;
-            b.t_out[inst] = t;
-        }
-        __syncthreads();
-    }
+    return batch_config_p<1, Batch1Cfg>(prec, fx, v, blocks_per_sm, smem);
 }
-
-template <typename T, bool EXACTDET, int V, bool FX>
-cudaError_t batch_config(int* blocks_per_sm, size_t* smem)
+cudaError_t batch1d_launch(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s)
 {
-    using BT = BatchTile<V>;
-    using SM = SweepSmem<T, 1, 1, BT::SEG>;
-    auto kern = k_batch<T, BT::SEG, BT::NT, EXACTDET, FX>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    if (e != cudaSuccess) return e;
-    *smem = SM::bytes;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, BT::NT, SM::bytes);
+    return batch_launch_p<1, Batch1Cfg>(prec, fx, v, b, blocks, s);
 }
-
-template <typename T, bool EXACTDET, int V, bool FX>
-cudaError_t batch_launch(const BatchArgs& b, int blocks, cudaStream_t s)
+int batch1d_tiles(int v, int nx)
 {
-    using BT = BatchTile<V>;
-    using SM = SweepSmem<T, 1, 1, BT::SEG>;
-    k_batch<T, BT::SEG, BT::NT, EXACTDET, FX><<<blocks, BT::NT, SM::bytes, s>>>(b);
-    return cudaGetLastError();
+    if (v == 1) return batch_tiles<Batch1Cfg<1>>(1, nx, 1, 0);
+    if (v == 2) return batch_tiles<Batch1Cfg<2>>(1, nx, 1, 0);
+    return batch_tiles<Batch1Cfg<0>>(1, nx, 1, 0);
 }
 
 }  // namespace wis
@@ -180,38 +53,40 @@ cudaError_t batch_launch(const BatchArgs& b, int blocks, cudaStream_t s)
 using wis::BatchArgs;
 
 struct weno_batch {
-    int dim = 1;   // 1: [3][n] instances (k_batch); 2: [4][ny][nx] instances (k_batch2d)
+    int dim = 1;   // 1: [3][n] instances, 2: [4][ny][nx] instances
     int count = 0, prec = 0, dev = 0, nsm = 1;
     size_t esz = 8;
     weno_params p;
-    int bc_lo = 0, bc_hi = 0, max_steps = 0;
+    int bc_lo[2] = {0, 0}, bc_hi[2] = {0, 0}, max_steps = 0;
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;
-    long long total_cells = 0, total_ghosted = 0;
+    long long total = 0;          // elements of the states of all instances
     int* order = nullptr;
-    int* n = nullptr;
-    long long* off = nullptr;
-    long long* goff = nullptr;
-    double* dx = nullptr;
+    wis::BatchInst* inst = nullptr;
     double* t_end = nullptr;
-    int* ny = nullptr;        // 2D
-    double* dy = nullptr;     // 2D
-    int bc_lo_y = 0, bc_hi_y = 0;
     void* work[4] = {nullptr, nullptr, nullptr, nullptr};   // the fourth: 2D accumulator
+    unsigned char* run = nullptr;   // BatchCtrl, the BatchState of every instance, the task queue
+    size_t run_bytes = 0;
+    long long places = 0;           // of the queue: the tiles of all instances
+    long long tiles_of[wis::kBatchVariants] = {};    // tiles of the longer direction, per variant
     int* status = nullptr;
     long long* steps = nullptr;
     double* t_out = nullptr;
-    unsigned int* head = nullptr;
     unsigned long long* wcount = nullptr;
     int* trial_caps = nullptr;
     std::vector<int> n_host;      // steps grow with this size: n (1D), max(nx, ny) (2D)
     bool fx = false;              // an FP64 instance takes the integer six-point sums
     int variant = 0;
-    int blocks = 0;
+    int blocks = 0;               // reported: min(count, residency x SMs)
+    int grid = 0;                 // CTAs launched: min(tiles, residency x SMs)
     cudaGraphExec_t graph = nullptr;
     void* graph_U = nullptr;
     std::string err;
 };
+
+// the BatchState array starts here in weno_batch::run
+constexpr size_t kCtrlBytes = 256;
+static_assert(sizeof(wis::BatchCtrl) <= kCtrlBytes, "control block");
 
 static std::string g_batch_err;
 
@@ -224,44 +99,10 @@ static std::string g_batch_err;
         }                                                                                   \
     } while (0)
 
-// fx: an FP64 batch with an instance large enough for the integer six-point
-// sums (use_fx); other batches keep the leaner kernel
-template <typename T, bool EXACTDET, bool FX>
-static cudaError_t batch_config_v(int v, int* bps, size_t* smem)
+static cudaError_t dispatch_config(weno_batch* bt, int v, int* bps, size_t* smem)
 {
-    using namespace wis;
-    if (v == 1) return batch_config<T, EXACTDET, 1, FX>(bps, smem);
-    if (v == 2) return batch_config<T, EXACTDET, 2, FX>(bps, smem);
-    return batch_config<T, EXACTDET, 0, FX>(bps, smem);
-}
-
-template <typename T, bool EXACTDET, bool FX>
-static cudaError_t batch_launch_v(int v, const BatchArgs& b, int blocks, cudaStream_t s)
-{
-    using namespace wis;
-    if (v == 1) return batch_launch<T, EXACTDET, 1, FX>(b, blocks, s);
-    if (v == 2) return batch_launch<T, EXACTDET, 2, FX>(b, blocks, s);
-    return batch_launch<T, EXACTDET, 0, FX>(b, blocks, s);
-}
-
-static cudaError_t batch_dispatch_config(int dim, int prec, bool fx, int v, int* bps, size_t* smem)
-{
-    if (dim == 2) return wis::batch2d_config(prec, fx, v, bps, smem);
-    if (prec == WENO_FP64)
-        return fx ? batch_config_v<double, false, true>(v, bps, smem) : batch_config_v<double, false, false>(v, bps, smem);
-    return prec == WENO_MIXED ? batch_config_v<float, true, false>(v, bps, smem)
-                              : batch_config_v<float, false, false>(v, bps, smem);
-}
-
-static cudaError_t batch_dispatch_launch(int dim, int prec, bool fx, int v, const BatchArgs& b, int blocks,
-                                         cudaStream_t s)
-{
-    if (dim == 2) return wis::batch2d_launch(prec, fx, v, b, blocks, s);
-    if (prec == WENO_FP64)
-        return fx ? batch_launch_v<double, false, true>(v, b, blocks, s)
-                  : batch_launch_v<double, false, false>(v, b, blocks, s);
-    return prec == WENO_MIXED ? batch_launch_v<float, true, false>(v, b, blocks, s)
-                              : batch_launch_v<float, false, false>(v, b, blocks, s);
+    return bt->dim == 2 ? wis::batch2d_config(bt->prec, bt->fx, v, bps, smem)
+                        : wis::batch1d_config(bt->prec, bt->fx, v, bps, smem);
 }
 
 static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_back)
@@ -269,22 +110,28 @@ static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_ba
     BatchArgs b;
     std::memset(&b, 0, sizeof(b));
     b.count = bt->count;
-    b.order = bt->order; b.n = bt->n; b.off = bt->off; b.goff = bt->goff;
-    b.dx = bt->dx; b.t_end = bt->t_end;
+    b.order = bt->order;
+    b.inst = bt->inst;
+    b.ctrl = reinterpret_cast<wis::BatchCtrl*>(bt->run);
+    b.state = reinterpret_cast<wis::BatchState*>(bt->run + kCtrlBytes);
+    b.queue = reinterpret_cast<wis::BatchTask*>(bt->run + kCtrlBytes + sizeof(wis::BatchState) * (size_t)bt->count);
+    b.places = bt->places;
+    b.total_tiles = bt->tiles_of[bt->variant];
+    b.t_end = bt->t_end;
     b.U = U;
-    b.work0 = bt->work[0]; b.work1 = bt->work[1]; b.work2 = bt->work[2];
+    for (int k = 0; k < 3; ++k) b.work[k] = bt->work[k];
+    b.acc = bt->work[3];
     b.status = bt->status; b.steps = bt->steps; b.t_out = bt->t_out;
-    b.head = bt->head;
     b.weno_count = bt->wcount;
     b.max_steps = max_steps;
     b.write_back = write_back;
     b.gamma = bt->p.gamma; b.cfl = bt->p.cfl; b.eps = bt->p.eps; b.c_lambda = bt->p.c_lambda;
-    b.C_thr = bt->p.C_thr; b.L_char = bt->p.L_char; b.alpha_thr = bt->p.alpha_thr; b.hybrid = bt->p.hybrid;
-    b.bc_lo = bt->bc_lo; b.bc_hi = bt->bc_hi;
+    b.gamma_f = (float)bt->p.gamma;
+    b.eps_f = (float)bt->p.eps;
+    b.lam_scale_f = (float)(bt->p.c_lambda * (1.0 / 3600.0));
+    b.hybrid = bt->p.hybrid;
     b.wmode = bt->p.weights; b.split = bt->p.splitting;
-    b.ny = bt->ny; b.dy = bt->dy;
-    b.bc_lo_y = bt->bc_lo_y; b.bc_hi_y = bt->bc_hi_y;
-    b.work3 = bt->work[3];
+    for (int d = 0; d < 2; ++d) { b.bc_lo[d] = bt->bc_lo[d]; b.bc_hi[d] = bt->bc_hi[d]; }
     return b;
 }
 
@@ -292,38 +139,128 @@ static weno_status set_variant(weno_batch* bt, int v, int blocks_per_sm_cap)
 {
     int bps = 0;
     size_t smem = 0;
-    BCK(batch_dispatch_config(bt->dim, bt->prec, bt->fx, v, &bps, &smem));
+    BCK(dispatch_config(bt, v, &bps, &smem));
     if (bps < 1) { bt->err = "batch kernel cannot be resident"; return WENO_ERR_CUDA; }
     if (blocks_per_sm_cap > 0 && bps > blocks_per_sm_cap) bps = blocks_per_sm_cap;
     bt->variant = v;
-    long long blocks = (long long)bps * bt->nsm;
-    if (blocks > bt->count) blocks = bt->count;
-    bt->blocks = (int)blocks;
+    const long long resident = (long long)bps * bt->nsm;
+    bt->blocks = (int)std::min<long long>(resident, bt->count);
+    bt->grid = (int)std::min<long long>(resident, bt->tiles_of[v]);
     if (bt->graph) cudaGraphExecDestroy(bt->graph);
     bt->graph = nullptr;
     return WENO_OK;
 }
 
-// reset the queue and launch once (on stream s, optionally under capture)
+// one run on stream s (optionally under capture): counters and progress
+// zeroed, then the kernel
+static cudaError_t launch_run(weno_batch* bt, const BatchArgs& b, cudaStream_t s)
+{
+    cudaError_t e = cudaMemsetAsync(bt->run, 0, bt->run_bytes, s);
+    if (e != cudaSuccess) return e;
+    return bt->dim == 2 ? wis::batch2d_launch(bt->prec, bt->fx, bt->variant, b, bt->grid, s)
+                        : wis::batch1d_launch(bt->prec, bt->fx, bt->variant, b, bt->grid, s);
+}
+
 static cudaError_t enqueue_run(weno_batch* bt, void* U, int max_steps, int write_back, cudaStream_t s,
                                const int* trial_caps = nullptr)
 {
-    cudaError_t e = cudaMemsetAsync(bt->head, 0, sizeof(unsigned int), s);
-    if (e != cudaSuccess) return e;
     BatchArgs b = batch_args(bt, U, max_steps, write_back);
     b.trial_caps = trial_caps;
-    return batch_dispatch_launch(bt->dim, bt->prec, bt->fx, bt->variant, b, bt->blocks, s);
+    return launch_run(bt, b, s);
 }
 
 static void batch_free(weno_batch* bt)
 {
     if (bt->graph) cudaGraphExecDestroy(bt->graph);
-    void* ptrs[] = {bt->order, bt->n, bt->off, bt->goff, bt->dx, bt->t_end, bt->work[0], bt->work[1],
-                    bt->work[2], bt->work[3], bt->status, bt->steps, bt->t_out, bt->head, bt->wcount,
-                    bt->trial_caps, bt->ny, bt->dy};
+    void* ptrs[] = {bt->order, bt->inst, bt->t_end, bt->work[0], bt->work[1], bt->work[2], bt->work[3], bt->run,
+                    bt->status, bt->steps, bt->t_out, bt->wcount, bt->trial_caps};
     for (void* q : ptrs)
         if (q) cudaFree(q);
     if (bt->cap) cudaStreamDestroy(bt->cap);
+}
+
+// Allocations and device tables of a batch whose dim, count, prec, p, bc_*,
+// max_steps, stream and n_host are set: nx, ny (null in 1D), the spacings and
+// end times per instance, and the schedule (most work first).
+static cudaError_t batch_setup(weno_batch* bt, const int* nx, const int* ny, const std::vector<double>& dx,
+                               const std::vector<double>& dy, const double* t_end, const std::vector<int>& order)
+{
+    const int cnt = bt->count, nv = bt->dim + 2;
+    bt->esz = bt->prec == WENO_FP64 ? sizeof(double) : sizeof(float);
+    std::vector<wis::BatchInst> inst(cnt);
+    std::memset(inst.data(), 0, sizeof(wis::BatchInst) * cnt);
+    long long off = 0;
+    for (int i = 0; i < cnt; ++i) {
+        wis::BatchInst& q = inst[i];
+        q.nx = nx[i];
+        q.ny = ny ? ny[i] : 1;
+        q.off = off;
+        const long long cells = (long long)q.nx * q.ny;
+        off += nv * cells;
+        for (int d = 0; d < bt->dim; ++d) {
+            const double h = d == 0 ? dx[i] : dy[i];
+            // Eq. eq31 with the spacing of the direction
+            double eps_h = bt->p.C_thr;
+            for (int k = 0; k < bt->p.alpha_thr; ++k) eps_h *= h / bt->p.L_char;
+            q.inv_dx[d] = 1.0 / h;
+            q.inv_dx_f[d] = (float)q.inv_dx[d];
+            q.inv_dx60_f[d] = (float)(q.inv_dx[d] * (1.0 / 60.0));
+            q.slim[d] = std::sqrt(3600.0 * eps_h);
+            q.slim_f[d] = (float)q.slim[d];
+        }
+        bt->fx = bt->fx || (bt->prec == WENO_FP64 && wis::use_fx(cells));
+        for (int v = 0; v < wis::kBatchVariants; ++v)
+            bt->tiles_of[v] += bt->dim == 1 ? wis::batch1d_tiles(v, q.nx)
+                                            : std::max(wis::batch2d_tiles(v, q.nx, q.ny, 0),
+                                                       wis::batch2d_tiles(v, q.nx, q.ny, 1));
+    }
+    bt->total = off;
+    for (int v = 0; v < wis::kBatchVariants; ++v) bt->places = std::max(bt->places, bt->tiles_of[v]);
+    if (bt->places > INT_MAX) return cudaErrorInvalidValue;
+
+    cudaError_t e = cudaGetDevice(&bt->dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bt->nsm, cudaDevAttrMultiProcessorCount, bt->dev);
+    auto alloc = [&](void** p, size_t bytes) {
+        if (e == cudaSuccess) e = cudaMalloc(p, bytes);
+    };
+    bt->run_bytes = kCtrlBytes + sizeof(wis::BatchState) * (size_t)cnt + sizeof(wis::BatchTask) * (size_t)bt->places;
+    alloc((void**)&bt->order, sizeof(int) * cnt);
+    alloc((void**)&bt->inst, sizeof(wis::BatchInst) * cnt);
+    alloc((void**)&bt->t_end, sizeof(double) * cnt);
+    for (int k = 0; k < (bt->dim == 2 ? 4 : 3); ++k) alloc(&bt->work[k], bt->esz * (size_t)bt->total);
+    alloc((void**)&bt->run, bt->run_bytes);
+    alloc((void**)&bt->status, sizeof(int) * cnt);
+    alloc((void**)&bt->steps, sizeof(long long) * cnt);
+    alloc((void**)&bt->t_out, sizeof(double) * cnt);
+    alloc((void**)&bt->wcount, sizeof(unsigned long long));
+    alloc((void**)&bt->trial_caps, sizeof(int) * cnt);
+    if (e == cudaSuccess) e = cudaMemcpy(bt->order, order.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(bt->inst, inst.data(), sizeof(wis::BatchInst) * cnt, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(bt->t_end, t_end, sizeof(double) * cnt, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(bt->wcount, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMemset(bt->run, 0, bt->run_bytes);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking);
+    return e;
+}
+
+// the last part of both create calls
+static weno_status finish_create(weno_batch* bt, cudaError_t e, const char* what, weno_batch** out)
+{
+    weno_status st = WENO_OK;
+    if (e != cudaSuccess) {
+        bt->err = std::string(what) + ": " + cudaGetErrorString(e);
+        st = WENO_ERR_CUDA;
+    } else {
+        st = set_variant(bt, 0, 0);
+    }
+    if (st != WENO_OK) {
+        g_batch_err = bt->err;
+        batch_free(bt);
+        delete bt;
+        return st;
+    }
+    *out = bt;
+    return WENO_OK;
 }
 
 extern "C" {
@@ -356,22 +293,14 @@ weno_status weno_batch_create(const weno_batch_desc* d, const weno_params* param
         return WENO_ERR_INVALID_ARG;
     }
     const int cnt = d->count;
-    std::vector<long long> off(cnt), goff(cnt);
-    std::vector<double> dx(cnt), tend(cnt);
-    long long tc = 0, tg = 0;
+    std::vector<double> dx(cnt);
     for (int i = 0; i < cnt; ++i) {
         if (d->n[i] < 3 || !(d->hi[i] > d->lo[i]) || !(d->t_end[i] >= 0.0)) {
             g_batch_err = "instance with n < 3, hi <= lo or negative t_end";
             return WENO_ERR_INVALID_ARG;
         }
-        off[i] = tc;
-        goff[i] = tg;
-        tc += 3LL * d->n[i];
-        tg += 3LL * (d->n[i] + 6);
         dx[i] = (d->hi[i] - d->lo[i]) / d->n[i];
-        tend[i] = d->t_end[i];
     }
-    // schedule: largest instances first
     std::vector<int> order(cnt);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return d->n[a] > d->n[b]; });
@@ -381,56 +310,12 @@ weno_status weno_batch_create(const weno_batch_desc* d, const weno_params* param
     bt->count = cnt;
     bt->p = *params;
     bt->prec = params->precision;
-    bt->esz = bt->prec == WENO_FP64 ? sizeof(double) : sizeof(float);
-    bt->bc_lo = d->bc_lo;
-    bt->bc_hi = d->bc_hi;
+    bt->bc_lo[0] = d->bc_lo;
+    bt->bc_hi[0] = d->bc_hi;
     bt->max_steps = d->max_steps > 0 ? d->max_steps : 0x7fffffff;
     bt->stream = (cudaStream_t)stream;
-    bt->total_cells = tc / 3;
-    bt->total_ghosted = tg;
-    cudaError_t e = cudaGetDevice(&bt->dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bt->nsm, cudaDevAttrMultiProcessorCount, bt->dev);
-    auto alloc = [&](void** p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-    };
-    alloc((void**)&bt->order, sizeof(int) * cnt);
-    alloc((void**)&bt->n, sizeof(int) * cnt);
-    alloc((void**)&bt->off, sizeof(long long) * cnt);
-    alloc((void**)&bt->goff, sizeof(long long) * cnt);
-    alloc((void**)&bt->dx, sizeof(double) * cnt);
-    alloc((void**)&bt->t_end, sizeof(double) * cnt);
-    for (int k = 0; k < 3; ++k) alloc(&bt->work[k], bt->esz * (size_t)tg);
-    alloc((void**)&bt->status, sizeof(int) * cnt);
-    alloc((void**)&bt->steps, sizeof(long long) * cnt);
-    alloc((void**)&bt->t_out, sizeof(double) * cnt);
-    alloc((void**)&bt->head, sizeof(unsigned int));
-    alloc((void**)&bt->wcount, sizeof(unsigned long long));
-    alloc((void**)&bt->trial_caps, sizeof(int) * cnt);
     bt->n_host.assign(d->n, d->n + cnt);
-    for (int i = 0; i < cnt; ++i) bt->fx = bt->fx || (bt->prec == WENO_FP64 && wis::use_fx(d->n[i]));
-    if (e == cudaSuccess) e = cudaMemcpy(bt->order, order.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->n, d->n, sizeof(int) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->off, off.data(), sizeof(long long) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->goff, goff.data(), sizeof(long long) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->dx, dx.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->t_end, tend.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(bt->wcount, 0, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-        g_batch_err = std::string("weno_batch_create: ") + cudaGetErrorString(e);
-        batch_free(bt);
-        delete bt;
-        return WENO_ERR_CUDA;
-    }
-    weno_status st = set_variant(bt, 0, 0);
-    if (st != WENO_OK) {
-        g_batch_err = bt->err;
-        batch_free(bt);
-        delete bt;
-        return st;
-    }
-    *out = bt;
-    return WENO_OK;
+    return finish_create(bt, batch_setup(bt, d->n, nullptr, dx, dx, d->t_end, order), "weno_batch_create", out);
 }
 
 weno_status weno_batch2d_create(const weno_batch2d_desc* d, const weno_params* params, void* stream,
@@ -465,26 +350,20 @@ weno_status weno_batch2d_create(const weno_batch2d_desc* d, const weno_params* p
         }
     }
     const int cnt = d->count;
-    std::vector<long long> off(cnt);
-    std::vector<double> dx(cnt), dy(cnt), tend(cnt), work(cnt);
+    std::vector<double> dx(cnt), dy(cnt), work(cnt);
     std::vector<int> lin(cnt);
-    long long tc = 0;
     for (int i = 0; i < cnt; ++i) {
         if (d->nx[i] < 3 || d->ny[i] < 3 || !(d->hi_x[i] > d->lo_x[i]) || !(d->hi_y[i] > d->lo_y[i]) ||
             !(d->t_end[i] >= 0.0)) {
             g_batch_err = "instance with nx or ny < 3, hi <= lo or negative t_end";
             return WENO_ERR_INVALID_ARG;
         }
-        off[i] = tc;
-        tc += 4LL * d->nx[i] * d->ny[i];
         dx[i] = (d->hi_x[i] - d->lo_x[i]) / d->nx[i];
         dy[i] = (d->hi_y[i] - d->lo_y[i]) / d->ny[i];
-        tend[i] = d->t_end[i];
         lin[i] = std::max(d->nx[i], d->ny[i]);
         // work of a run ~ cells x steps, and the steps grow with the finer spacing
         work[i] = (double)d->nx[i] * d->ny[i] * lin[i];
     }
-    // schedule: most work first
     std::vector<int> order(cnt);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return work[a] > work[b]; });
@@ -495,63 +374,11 @@ weno_status weno_batch2d_create(const weno_batch2d_desc* d, const weno_params* p
     bt->count = cnt;
     bt->p = *params;
     bt->prec = params->precision;
-    bt->esz = bt->prec == WENO_FP64 ? sizeof(double) : sizeof(float);
-    bt->bc_lo = d->bc_lo[0];
-    bt->bc_hi = d->bc_hi[0];
-    bt->bc_lo_y = d->bc_lo[1];
-    bt->bc_hi_y = d->bc_hi[1];
+    for (int k = 0; k < 2; ++k) { bt->bc_lo[k] = d->bc_lo[k]; bt->bc_hi[k] = d->bc_hi[k]; }
     bt->max_steps = d->max_steps > 0 ? d->max_steps : 0x7fffffff;
     bt->stream = (cudaStream_t)stream;
-    bt->total_cells = tc / 4;
-    bt->total_ghosted = tc;
-    cudaError_t e = cudaGetDevice(&bt->dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bt->nsm, cudaDevAttrMultiProcessorCount, bt->dev);
-    auto alloc = [&](void** p, size_t bytes) {
-        if (e == cudaSuccess) e = cudaMalloc(p, bytes);
-    };
-    alloc((void**)&bt->order, sizeof(int) * cnt);
-    alloc((void**)&bt->n, sizeof(int) * cnt);
-    alloc((void**)&bt->ny, sizeof(int) * cnt);
-    alloc((void**)&bt->off, sizeof(long long) * cnt);
-    alloc((void**)&bt->goff, sizeof(long long) * cnt);
-    alloc((void**)&bt->dx, sizeof(double) * cnt);
-    alloc((void**)&bt->dy, sizeof(double) * cnt);
-    alloc((void**)&bt->t_end, sizeof(double) * cnt);
-    for (int k = 0; k < 4; ++k) alloc(&bt->work[k], bt->esz * (size_t)tc);
-    alloc((void**)&bt->status, sizeof(int) * cnt);
-    alloc((void**)&bt->steps, sizeof(long long) * cnt);
-    alloc((void**)&bt->t_out, sizeof(double) * cnt);
-    alloc((void**)&bt->head, sizeof(unsigned int));
-    alloc((void**)&bt->wcount, sizeof(unsigned long long));
-    alloc((void**)&bt->trial_caps, sizeof(int) * cnt);
     bt->n_host = lin;
-    for (int i = 0; i < cnt; ++i)
-        bt->fx = bt->fx || (bt->prec == WENO_FP64 && wis::use_fx((long long)d->nx[i] * d->ny[i]));
-    if (e == cudaSuccess) e = cudaMemcpy(bt->order, order.data(), sizeof(int) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->n, d->nx, sizeof(int) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->ny, d->ny, sizeof(int) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->off, off.data(), sizeof(long long) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->goff, off.data(), sizeof(long long) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->dx, dx.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->dy, dy.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(bt->t_end, tend.data(), sizeof(double) * cnt, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(bt->wcount, 0, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&bt->cap, cudaStreamNonBlocking);
-    if (e != cudaSuccess) {
-        g_batch_err = std::string("weno_batch2d_create: ") + cudaGetErrorString(e);
-        batch_free(bt);
-        delete bt;
-        return WENO_ERR_CUDA;
-    }
-    weno_status st = set_variant(bt, 0, 0);
-    if (st != WENO_OK) {
-        g_batch_err = bt->err;
-        batch_free(bt);
-        delete bt;
-        return st;
-    }
-    *out = bt;
-    return WENO_OK;
+    return finish_create(bt, batch_setup(bt, d->nx, d->ny, dx, dy, d->t_end, order), "weno_batch2d_create", out);
 }
 
 void weno_batch_destroy(weno_batch* bt)
@@ -598,7 +425,14 @@ weno_status weno_batch_results(weno_batch* bt, int* status, long long* steps, do
     if (status) BCK(cudaMemcpyAsync(status, bt->status, sizeof(int) * bt->count, cudaMemcpyDeviceToHost, bt->stream));
     if (steps) BCK(cudaMemcpyAsync(steps, bt->steps, sizeof(long long) * bt->count, cudaMemcpyDeviceToHost, bt->stream));
     if (t) BCK(cudaMemcpyAsync(t, bt->t_out, sizeof(double) * bt->count, cudaMemcpyDeviceToHost, bt->stream));
+    int abort = 0;
+    BCK(cudaMemcpyAsync(&abort, &reinterpret_cast<wis::BatchCtrl*>(bt->run)->abort, sizeof(int),
+                        cudaMemcpyDeviceToHost, bt->stream));
     BCK(cudaStreamSynchronize(bt->stream));
+    if (abort) {
+        bt->err = "a wait of the batch kernel for its next task ran out; the states are not valid";
+        return WENO_ERR_TIMEOUT;
+    }
     if (status)
         for (int i = 0; i < bt->count; ++i)
             if (status[i] != WENO_OK) {
@@ -625,7 +459,7 @@ weno_status weno_batch_weno_face_count(weno_batch* bt, unsigned long long* count
 weno_status weno_batch_set_config(weno_batch* bt, int variant, int blocks_per_sm, int* blocks)
 {
     if (!bt) return WENO_ERR_INVALID_ARG;
-    if (variant < 0 || variant >= (bt->dim == 2 ? wis::kBatch2Variants : wis::kBatchVariants) || blocks_per_sm < 0) {
+    if (variant < 0 || variant >= wis::kBatchVariants || blocks_per_sm < 0) {
         bt->err = "set_config: variant must be 0, 1 or 2 and blocks_per_sm >= 0";
         return WENO_ERR_INVALID_ARG;
     }
@@ -650,7 +484,7 @@ weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_ste
     // have spread, and trials from the initial jumps rank the configurations
     // unlike full runs do (they favour small tiles that lose on developed
     // solutions)
-    const size_t sbytes = (size_t)bt->total_cells * (bt->dim + 2) * bt->esz;
+    const size_t sbytes = (size_t)bt->total * bt->esz;
     void* Us = nullptr;
     double* t_half = nullptr;
     BCK(cudaMalloc(&Us, sbytes));
@@ -665,11 +499,10 @@ weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_ste
     if (ce == cudaSuccess)
         ce = cudaMemcpy(t_half, th.data(), sizeof(double) * bt->count, cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(Us, U_dev, sbytes, cudaMemcpyDeviceToDevice, bt->stream);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(bt->head, 0, sizeof(unsigned int), bt->stream);
     if (ce == cudaSuccess) {
         BatchArgs b = batch_args(bt, Us, bt->max_steps, 1);
         b.t_end = t_half;
-        ce = batch_dispatch_launch(bt->dim, bt->prec, bt->fx, bt->variant, b, bt->blocks, bt->stream);
+        ce = launch_run(bt, b, bt->stream);
     }
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(bt->stream);
     cudaFree(t_half);
@@ -687,8 +520,7 @@ weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_ste
     int best_v = bt->variant, best_cap = 0;
     const int caps[3] = {0, 4, 2};   // 0 = as many CTAs per SM as fit
     weno_status st = WENO_OK;
-    const int nvariants = bt->dim == 2 ? wis::kBatch2Variants : wis::kBatchVariants;
-    for (int v = 0; v < nvariants && st == WENO_OK; ++v) {
+    for (int v = 0; v < wis::kBatchVariants && st == WENO_OK; ++v) {
         for (int c = 0; c < 3 && st == WENO_OK; ++c) {
             st = set_variant(bt, v, caps[c]);
             if (st != WENO_OK) break;

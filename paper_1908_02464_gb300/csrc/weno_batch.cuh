@@ -1,44 +1,473 @@
-// Arguments of the persistent batched solvers (weno_batch.cu: 1D instances,
-// weno_batch2d.cu: 2D instances) and the 2D kernel's host entry points.
+// Persistent batched solver (1D instances: weno_batch.cu, 2D instances:
+// weno_batch2d.cu): many independent Euler problems of uneven sizes, each
+// advanced to its own end time with its own CFL step.
+//
+// One launch of resident CTAs works through a queue of tasks.  A task is a
+// run of consecutive tiles of one sweep of one instance.  The CTA that
+// finishes the last run of a sweep puts the instance's next sweep into the
+// queue, and after the last sweep of a step (Sec. 4 of the paper) it also
+// advances the instance's time and takes the next CFL step.  Instances wait
+// only for their own previous sweep.  A CTA without a task polls its place in
+// the queue; it holds nothing that another CTA waits for, so the polls end
+// whichever CTAs are resident.
+//
+// What bounds it: the FP64 pipe (FP64), instruction issue and shared-memory
+// loads (FP32).  In the first form of this solver one CTA integrated one
+// instance from start to end.  The steps of an instance vary by a factor of
+// twenty, and a CTA alone uses a third of its SM, so the heaviest of 1024
+// Riemann problems (1913 cells, 224 steps, 0.7% of the work) took 80 of 125
+// ms.  The figures stand beside the launch shapes in weno_batch.cu and
+// weno_batch2d.cu.
+//
+// The tiles are the grid solver's (sweep_tile, line_tile), so every face is
+// computed by identical arithmetic; maxima and flags do not depend on the
+// order in which tiles finish.
 #pragma once
 
 #include <cuda_runtime.h>
 
+#include "../../include/weno_is.h"
+#include "weno_kernels.cuh"
+#include "weno_line.cuh"
+
 namespace wis {
+
+// constants of one instance (written by the host)
+struct BatchInst {
+    int nx, ny;                  // ny = 1 in 1D
+    long long off;               // its states [nvar][ny][nx] start here in U and in the work arrays
+    double inv_dx[2], slim[2];   // per direction: 1 / dx, 60 sqrt(eps_h)
+    float inv_dx_f[2], inv_dx60_f[2], slim_f[2];
+};
+
+// progress of one instance (zeroed before each run)
+struct BatchState {
+    double t, dt;                // dt = 0: finished
+    unsigned long long smax;     // CFL wave speed of the current state (bits)
+    long long steps;
+    int left;                    // runs of the current sweep not yet finished
+    int run;                     // tiles per run of the current sweep
+    int phase;                   // sweep of the step: 1D the stage, 2D 2 stage + (0 y, 1 x)
+    int cur;                     // work array (0 or 1) of the current state
+    int clipped;                 // the step in progress ends at t_end
+    int bad;                     // BAD_STAGE, BAD_CFL
+    float dt_f;
+    int pad;
+};
+enum { BAD_STAGE = 1, BAD_CFL = 2 };
+
+// one place of the task queue
+struct BatchTask {
+    int inst, run;
+    unsigned int turn;           // how often the place has been filled
+    int pad;
+};
+
+// counters of one run (zeroed before each run)
+struct BatchCtrl {
+    unsigned long long head;           // places taken by CTAs
+    unsigned long long tail;           // tasks put into the queue
+    unsigned long long finished_tiles; // tiles of finished instances
+    int finished;                      // instances
+    int abort;                         // a wait for a task ran out
+};
 
 struct BatchArgs {
     int count;
-    const int* order;        // instance ids, largest first
-    const int* n;            // cells per instance (2D: columns nx)
-    const long long* off;    // offset of instance i in U (1D [3][n_i], 2D [4][ny_i][nx_i])
-    const long long* goff;   // offset of instance i in each work array (1D [3][n_i + 6], 2D as U)
-    const double* dx;
+    const int* order;            // instance ids, most work first
+    const BatchInst* inst;
+    BatchCtrl* ctrl;
+    BatchState* state;
+    BatchTask* queue;            // one place per tile of the batch
+    long long places, total_tiles;
     const double* t_end;
     void* U;
-    void* work0;
-    void* work1;
-    void* work2;
-    int* status;             // per instance: 0 ok, WENO_ERR_NONPHYSICAL
+    void* work[3];               // two rotating states and the second stage
+    void* acc;                   // 2D: divergence of the y sweep
+    int* status;                 // per instance: 0 ok, WENO_ERR_NONPHYSICAL
     long long* steps;
     double* t_out;
-    unsigned int* head;      // work-queue counter (reset before each launch)
     unsigned long long* weno_count;
     int max_steps;
-    const int* trial_caps;   // autotuner trial runs: step cap per instance (null otherwise)
-    int write_back;          // 0: trial run, the caller's states are not touched
-    double gamma, cfl, eps, c_lambda, C_thr, L_char;
-    int alpha_thr, hybrid, bc_lo, bc_hi;
-    int wmode, split;
-    // 2D instances only
-    const int* ny;           // rows per instance
-    const double* dy;
-    int bc_lo_y, bc_hi_y;
-    void* work3;             // divergence of the y sweep (accumulator)
+    const int* trial_caps;       // autotuner trial runs: step cap per instance (null otherwise)
+    int write_back;              // 0: trial run, the caller's states are not touched
+    double gamma, cfl, eps, c_lambda;
+    float gamma_f, eps_f, lam_scale_f;
+    int hybrid, wmode, split;
+    int bc_lo[2], bc_hi[2];
 };
 
-// 2D batch kernel variants (weno_batch2d.cu); v in [0, kBatch2Variants)
-constexpr int kBatch2Variants = 3;
+// polls of a CTA for its next task before it gives up (about 100 ns each: some
+// seconds, where the longest sweep of a batch takes milliseconds)
+constexpr int kTaskPolls = 1 << 26;
+
+// tiles of nx x ny cells along direction d
+template <typename CFG>
+__host__ __device__ inline int batch_tiles(int dim, int nx, int ny, int d)
+{
+    if (dim == 1) return (nx + CFG::XS - 1) / CFG::XS;
+    return d == 0 ? ((nx + CFG::XS - 1) / CFG::XS) * ((ny + CFG::XL - 1) / CFG::XL)
+                  : ((ny + CFG::YS - 1) / CFG::YS) * ((nx + CFG::YL - 1) / CFG::YL);
+}
+
+// sweep arguments of one instance along direction d
+template <int DIM, bool FX>
+__device__ __forceinline__ SweepArgs batch_sweep_args(const BatchArgs& b, const BatchInst& q, int d)
+{
+    SweepArgs a;
+    const long long cells = (long long)q.nx * q.ny;
+    a.n[0] = q.nx; a.n[1] = q.ny; a.n[2] = 1;
+    a.sy = q.nx; a.sz = cells; a.sv = cells; a.off0 = 0;
+    a.acc = nullptr; a.Un = nullptr; a.out = nullptr;
+    a.tm = nullptr;
+    a.weno_count = b.weno_count;
+    a.flags = nullptr;
+    a.alpha_g = nullptr;
+    a.inv_dx = q.inv_dx[d];
+    a.slim = q.slim[d];
+    a.gamma = b.gamma; a.eps = b.eps; a.c_lambda = b.c_lambda; a.hybrid = b.hybrid;
+    a.wmode = b.wmode; a.split = b.split;
+    a.inv_dx_f = q.inv_dx60_f[d];
+    a.slim_f = q.slim_f[d];
+    a.gamma_f = b.gamma_f; a.eps_f = b.eps_f; a.lam_scale_f = b.lam_scale_f;
+    a.bc_lo = b.bc_lo[d]; a.bc_hi = b.bc_hi[d];
+    a.stage = 0;
+    a.xs_fixed = 0.0;
+    a.fx = FX && use_fx(cells);
+    return a;
+}
+
+// Time bookkeeping of one instance between two steps (first: before the
+// first one): takes over the step just made, then the next CFL step.
+__device__ __forceinline__ void batch_next_step(const BatchArgs& b, int inst, bool first)
+{
+    BatchState& s = b.state[inst];
+    const double t_end = b.t_end[inst];
+    const long long max_steps = b.trial_caps != nullptr ? (long long)b.trial_caps[inst] : (long long)b.max_steps;
+    int status = 0;
+    double t = s.t, dt = 0.0;
+    long long steps = s.steps;
+    int clipped = s.clipped;
+    const int bad = s.bad;
+    if (!first) {
+        if (bad & BAD_STAGE) {
+            status = WENO_ERR_NONPHYSICAL;   // the state before the step stays
+        } else {
+            s.cur = 1 - s.cur;
+            t = clipped ? t_end : t + s.dt;
+            ++steps;
+        }
+    }
+    if (status == 0 && steps < max_steps) {
+        if (bad & BAD_CFL) status = WENO_ERR_NONPHYSICAL;
+        else dt = cfl_step(b.cfl, __longlong_as_double((long long)s.smax), t, t_end, &clipped);
+    }
+    s.t = t;
+    s.steps = steps;
+    s.clipped = clipped;
+    s.dt = dt;
+    s.dt_f = (float)dt;
+    s.smax = 0ull;
+    s.bad = 0;
+    if (!(dt > 0.0)) {
+        b.status[inst] = status;
+        b.steps[inst] = steps;
+        b.t_out[inst] = t;
+    }
+}
+
+// One thread: moves an instance to its next sweep and reserves its places in
+// the queue: nr runs from place number `at` on.  Returns true when the
+// instance has finished instead.
+template <int DIM, typename CFG>
+__device__ bool batch_next_sweep(const BatchArgs& b, int inst, bool first, int& nr, unsigned long long& at)
+{
+    BatchState& s = b.state[inst];
+    const int nx = b.inst[inst].nx, ny = b.inst[inst].ny;
+    if (!first && s.phase + 1 < 3 * DIM) {
+        s.phase += 1;
+    } else {
+        batch_next_step(b, inst, first);
+        s.phase = 0;
+        if (!(s.dt > 0.0)) {
+            atomicAdd(&b.ctrl->finished_tiles, (unsigned long long)batch_tiles<CFG>(DIM, nx, ny, 0));
+            nr = 0;
+            return true;
+        }
+    }
+    const int nt = batch_tiles<CFG>(DIM, nx, ny, DIM == 2 && (s.phase & 1) == 0 ? 1 : 0);
+    // Long runs save the fixed work per task (queue, arguments, the first
+    // loads), short ones share the work evenly: CFG::RUN tiles while every CTA
+    // has several such runs, fewer when instances have finished
+    const long long per = (b.total_tiles - (long long)*(volatile unsigned long long*)&b.ctrl->finished_tiles) /
+                          ((long long)gridDim.x * 4);
+    const int run = per < 1 ? 1 : (per > CFG::RUN ? CFG::RUN : (int)per);
+    nr = (nt + run - 1) / run;
+    s.run = run;
+    s.left = nr;
+    at = atomicAdd(&b.ctrl->tail, (unsigned long long)nr);
+    return false;
+}
+
+// One warp: fills the places reserved by batch_next_sweep (its stores, and
+// those the block made before, are visible to the CTAs that take the tasks).
+__device__ __forceinline__ void batch_put(const BatchArgs& b, int inst, int nr, unsigned long long at)
+{
+    const unsigned long long places = (unsigned long long)b.places;
+    for (int r = threadIdx.x & 31; r < nr; r += 32) {
+        const unsigned long long k = at + (unsigned long long)r, turn = k / places;
+        BatchTask* q = b.queue + (long long)(k - turn * places);
+        q->inst = inst;
+        q->run = r;
+        __threadfence();
+        *(volatile unsigned int*)&q->turn = (unsigned int)turn + 1u;
+    }
+}
+
+// One thread: the next task; false when every instance has finished (or a
+// wait ran out).
+__device__ __forceinline__ bool batch_take(const BatchArgs& b, int& inst, int& run)
+{
+    const unsigned long long at = atomicAdd(&b.ctrl->head, 1ull);
+    const unsigned long long turn = at / (unsigned long long)b.places;
+    const BatchTask* q = b.queue + (long long)(at - turn * (unsigned long long)b.places);
+    for (int k = 0;; ++k) {
+        unsigned int v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&q->turn) : "memory");
+        if (v == (unsigned int)turn + 1u) break;
+        if ((k & 7) == 7) {
+            if (*(volatile int*)&b.ctrl->finished >= b.count || *(volatile int*)&b.ctrl->abort != 0) return false;
+            if (k >= kTaskPolls) {
+                atomicExch(&b.ctrl->abort, 1);
+                return false;
+            }
+        }
+        if (k > 32) __nanosleep(40);
+    }
+    inst = q->inst;
+    run = q->run;
+    return true;
+}
+
+template <typename T, int DIM, typename CFG, bool EXACTDET, bool FX>
+__global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batch(BatchArgs b)
+{
+    constexpr int NT = CFG::NT, NV = DIM + 2;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int s_inst, s_run, s_done;
+    unsigned int wenos = 0;
+    const int lane = threadIdx.x & 31;
+    const T gamma = pick<T>(b.gamma, b.gamma_f);
+    T* W[3] = {reinterpret_cast<T*>(b.work[0]), reinterpret_cast<T*>(b.work[1]), reinterpret_cast<T*>(b.work[2])};
+    T* U = reinterpret_cast<T*>(b.U);
+    // CFL wave speeds and flags of cells of one instance into its progress
+    auto note_cfl = [&](BatchState& s, T smax, bool bad) {
+        const T m = warp_max_nn(smax);
+        if (lane == 0 && m > T(0)) atomicMax(&s.smax, (unsigned long long)__double_as_longlong((double)m));
+        if (bad) atomicOr(&s.bad, BAD_CFL);
+    };
+    // the first warp queues the instance's next sweep; the states of a finished
+    // instance go back to the caller.  Every thread calls it; the sweep's (or
+    // the preparation's) stores come before.
+    auto next_sweep = [&](int inst, bool first) {
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            int done = 0, nr = 0;
+            unsigned long long at = 0ull;
+            if (threadIdx.x == 0) {
+                __threadfence();
+                if (first || atomicSub(&b.state[inst].left, 1) == 1) {
+                    __threadfence();
+                    done = batch_next_sweep<DIM, CFG>(b, inst, first, nr, at) ? 1 : 0;
+                    __threadfence();
+                }
+                s_done = done;
+            }
+            nr = __shfl_sync(0xffffffffu, nr, 0);
+            at = __shfl_sync(0xffffffffu, at, 0);
+            if (nr > 0) batch_put(b, inst, nr, at);
+        }
+        __syncthreads();
+        if (s_done != 0) {
+            if (b.write_back) {
+                const BatchInst q = b.inst[inst];
+                const T* w = W[b.state[inst].cur] + q.off;
+                for (long long c = threadIdx.x; c < (long long)NV * q.nx * q.ny; c += NT) U[q.off + c] = w[c];
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) atomicAdd(&b.ctrl->finished, 1);
+        }
+    };
+
+    // initial states, and their CFL wave speeds
+    for (int k = blockIdx.x; k < b.count; k += gridDim.x) {
+        const int inst = b.order[k];
+        const BatchInst q = b.inst[inst];
+        const long long cells = (long long)q.nx * q.ny;
+        T ih[DIM];
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) ih[d] = pick<T>(q.inv_dx[d], q.inv_dx_f[d]);
+        T m = T(0);
+        bool bad = false;
+        for (long long c = threadIdx.x; c < cells; c += NT) {
+            T u[NV], sp;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                u[v] = U[q.off + v * cells + c];
+                W[0][q.off + v * cells + c] = u[v];
+            }
+            if (!cell_speed<T, DIM>(u, gamma, ih, sp)) bad = true;
+            else m = max_nn(m, sp);
+        }
+        note_cfl(b.state[inst], m, bad);
+        next_sweep(inst, true);
+    }
+
+    for (;;) {
+        if (threadIdx.x == 0) {
+            int inst = -1, run = 0;
+            if (!batch_take(b, inst, run)) inst = -1;
+            s_inst = inst;
+            s_run = run;
+        }
+        __syncthreads();
+        const int inst = s_inst, run = s_run;
+        if (inst < 0) break;
+        BatchState& s = b.state[inst];
+        const BatchInst q = b.inst[inst];
+        const int phase = s.phase, cur = s.cur, len = s.run;
+        const T dt = pick<T>(s.dt, s.dt_f);
+        const int t0 = run * len;
+        // three stages: x = cur + dt L(cur); y = 3/4 cur + 1/4 (x + dt L(x));
+        // x = 1/3 cur + 2/3 (y + dt L(y)), x the other one of work arrays 0
+        // and 1, y work array 2
+        const int st = DIM == 2 ? phase >> 1 : phase;
+        const int in = st == 0 ? cur : (st == 1 ? 1 - cur : 2), out = st == 1 ? 2 : 1 - cur;
+        if (DIM == 2 && (phase & 1) == 0) {
+            SweepArgs a = batch_sweep_args<DIM, FX>(b, q, 1);
+            a.mode = MODE_ACC_SET;
+            a.U = W[in] + q.off;
+            a.acc = reinterpret_cast<T*>(b.acc) + q.off;
+            const int t1 = min(t0 + len, batch_tiles<CFG>(DIM, q.nx, q.ny, 1)), ns = (q.ny + CFG::YS - 1) / CFG::YS;
+            if constexpr (DIM == 2) {
+                for (int t = t0; t < t1; ++t) {
+                    const int lg = t / ns;
+                    sweep_tile<T, DIM, 1, CFG::YL, CFG::YS, NT, EXACTDET, false, FX>(a, t - lg * ns, lg * CFG::YL, 0,
+                                                                                     T(0), smem_raw);
+                }
+            }
+        } else {
+            SweepArgs a = batch_sweep_args<DIM, FX>(b, q, 0);
+            a.mode = MODE_COMBINE;
+            a.U = W[in] + q.off;
+            a.Un = W[cur] + q.off;
+            a.out = W[out] + q.off;
+            a.rk_a = st == 0 ? 0.0 : (st == 1 ? 0.75 : 1.0 / 3.0);
+            a.rk_b = st == 0 ? 1.0 : (st == 1 ? 0.25 : 2.0 / 3.0);
+            a.rk_a_f = st == 0 ? 0.0f : (st == 1 ? 0.75f : (float)(1.0 / 3.0));
+            a.rk_b_f = st == 0 ? 1.0f : (st == 1 ? 0.25f : (float)(2.0 / 3.0));
+            TileCfl<T, DIM> cfl;
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) cfl.inv_dx[d] = pick<T>(q.inv_dx[d], q.inv_dx_f[d]);
+            cfl.smax = T(0);
+            cfl.bad = false;
+            TileCfl<T, DIM>* const cp = st == 2 ? &cfl : nullptr;
+            const int t1 = min(t0 + len, batch_tiles<CFG>(DIM, q.nx, q.ny, 0));
+            bool bad = false;
+            if constexpr (DIM == 1) {
+                T u[3];
+                line_load(a, t0 * CFG::XS, u);
+                for (int t = t0; t < t1; ++t)
+                    bad |= line_tile<T, NT, EXACTDET, FX>(a, t * CFG::XS, t + 1 < t1 ? (t + 1) * CFG::XS : -1, dt, u,
+                                                          smem_raw, cp, wenos);
+            } else {
+                a.acc = reinterpret_cast<T*>(b.acc) + q.off;
+                a.acc_scale = q.inv_dx[1] * (1.0 / 60.0);   // the y sweep stores unscaled flux differences
+                a.acc_scale_f = q.inv_dx60_f[1];
+                const int ns = (q.nx + CFG::XS - 1) / CFG::XS;
+                for (int t = t0; t < t1; ++t) {
+                    const int lg = t / ns;
+                    bad |= sweep_tile<T, DIM, 0, CFG::XL, CFG::XS, NT, EXACTDET, false, FX>(a, t - lg * ns, lg * CFG::XL,
+                                                                                            0, dt, smem_raw, cp);
+                }
+            }
+            if (bad) atomicOr(&s.bad, BAD_STAGE);
+            if (st == 2) note_cfl(s, cfl.smax, cfl.bad);
+        }
+        next_sweep(inst, false);
+    }
+
+    if (DIM == 1 && b.weno_count != nullptr) {   // the 2D tiles count their own
+        const unsigned int w = __reduce_add_sync(0xffffffffu, wenos);
+        if (lane == 0 && w != 0u) atomicAdd(b.weno_count, (unsigned long long)w);
+    }
+}
+
+// CTAs per SM and shared memory of a configuration
+template <typename T, int DIM, typename CFG, bool EXACTDET, bool FX>
+cudaError_t batch_config(int* blocks_per_sm, size_t* smem)
+{
+    auto kern = k_batch<T, DIM, CFG, EXACTDET, FX>;
+    constexpr size_t bytes = CFG::template smem_bytes<T>();
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    if (e != cudaSuccess) return e;
+    *smem = bytes;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, kern, CFG::NT, bytes);
+}
+
+template <typename T, int DIM, typename CFG, bool EXACTDET, bool FX>
+cudaError_t batch_launch(const BatchArgs& b, int blocks, cudaStream_t s)
+{
+    k_batch<T, DIM, CFG, EXACTDET, FX><<<blocks, CFG::NT, CFG::template smem_bytes<T>(), s>>>(b);
+    return cudaGetLastError();
+}
+
+// Host entry points of the two kernels; variant v in [0, kBatchVariants), fx:
+// an FP64 instance of the batch takes the integer six-point sums (use_fx).
+// batch*_tiles: tiles of one instance along direction d.
+constexpr int kBatchVariants = 3;
+cudaError_t batch1d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem);
+cudaError_t batch1d_launch(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s);
+int batch1d_tiles(int v, int nx);
 cudaError_t batch2d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem);
 cudaError_t batch2d_launch(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s);
+int batch2d_tiles(int v, int nx, int ny, int d);
+
+// the dispatch over precision and variant, shared by the two translation
+// units; CFG<V> is the unit's configuration template
+template <int DIM, template <int> class CFG, typename T, bool EXACTDET, bool FX>
+cudaError_t batch_config_v(int v, int* bps, size_t* smem)
+{
+    if (v == 1) return batch_config<T, DIM, CFG<1>, EXACTDET, FX>(bps, smem);
+    if (v == 2) return batch_config<T, DIM, CFG<2>, EXACTDET, FX>(bps, smem);
+    return batch_config<T, DIM, CFG<0>, EXACTDET, FX>(bps, smem);
+}
+template <int DIM, template <int> class CFG>
+cudaError_t batch_config_p(int prec, bool fx, int v, int* bps, size_t* smem)
+{
+    if (prec == WENO_FP64)
+        return fx ? batch_config_v<DIM, CFG, double, false, true>(v, bps, smem)
+                  : batch_config_v<DIM, CFG, double, false, false>(v, bps, smem);
+    return prec == WENO_MIXED ? batch_config_v<DIM, CFG, float, true, false>(v, bps, smem)
+                              : batch_config_v<DIM, CFG, float, false, false>(v, bps, smem);
+}
+template <int DIM, template <int> class CFG, typename T, bool EXACTDET, bool FX>
+cudaError_t batch_launch_v(int v, const BatchArgs& b, int blocks, cudaStream_t s)
+{
+    if (v == 1) return batch_launch<T, DIM, CFG<1>, EXACTDET, FX>(b, blocks, s);
+    if (v == 2) return batch_launch<T, DIM, CFG<2>, EXACTDET, FX>(b, blocks, s);
+    return batch_launch<T, DIM, CFG<0>, EXACTDET, FX>(b, blocks, s);
+}
+template <int DIM, template <int> class CFG>
+cudaError_t batch_launch_p(int prec, bool fx, int v, const BatchArgs& b, int blocks, cudaStream_t s)
+{
+    if (prec == WENO_FP64)
+        return fx ? batch_launch_v<DIM, CFG, double, false, true>(v, b, blocks, s)
+                  : batch_launch_v<DIM, CFG, double, false, false>(v, b, blocks, s);
+    return prec == WENO_MIXED ? batch_launch_v<DIM, CFG, float, true, false>(v, b, blocks, s)
+                              : batch_launch_v<DIM, CFG, float, false, false>(v, b, blocks, s);
+}
 
 }  // namespace wis

@@ -300,6 +300,130 @@ __device__ __forceinline__ T fifth_difference(T u0, T u1, T u2, T u3, T u4, T u5
     return d1 - d0;
 }
 
+// CFL wave-speed sum sum_d (|u_d| + c) / dx_d of one cell; false if the cell
+// is not admissible (rho <= 0, p <= 0 or non-finite).  Shared by the grid
+// reduction and the batched solver so both take identical time steps.
+template <typename T, int DIM>
+__device__ __forceinline__ bool cell_speed(const T* u, T gamma, const T* inv_dx, T& s)
+{
+    const T gm1 = gamma - T(1);
+    const T irho = Ar<T>::rcp_f(u[0]);
+    T ke2 = T(0);
+    T vel[DIM];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) { vel[d] = u[1 + d] * irho; ke2 = fmaT(u[1 + d], vel[d], ke2); }
+    const T p = gm1 * fmaT(T(-0.5), ke2, u[DIM + 1]);
+    const T c2 = gamma * p * irho;
+    const T c = c2 * Ar<T>::rsqrt_(c2);   // NaN for p <= 0, rejected below
+    s = T(0);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) s = fmaT(absT(vel[d]) + c, inv_dx[d], s);
+    return (u[0] > T(0)) && (p > T(0)) && isfinite(s);
+}
+
+// dt = CFL / smax clipped to t_end (the clipped step lands exactly on t_end)
+__device__ __forceinline__ double cfl_step(double cfl, double smax, double t, double t_end, int* clipped)
+{
+    double dt = 0.0;
+    *clipped = 0;
+    if (t < t_end) {
+        if (smax > 0.0) dt = cfl / smax;
+        if (t + dt >= t_end) { dt = t_end - t; *clipped = 1; }
+        if (!(dt > 0.0)) { dt = 0.0; *clipped = 0; }
+    }
+    return dt;
+}
+
+// Characteristic regularized WENO-IS flux of the nq queued faces of a tile, in
+// chunks of QC faces: cq the tile's cell records, fr the face records, fh the
+// face fluxes (written, times 60), fpm and res scratch of one chunk.
+// cell(f, m): index of stencil cell m of face f.  Starts and ends without a
+// barrier (the queue is visible to the block; the caller synchronizes before
+// it reads fh).
+template <typename T, int DIM, int DIR, int NCELL, int NFACE, int QC, int NT, typename CELL>
+__device__ __forceinline__ void weno_queue(const SweepArgs& a, int nq, const T* cq, T* fh, const T* fr, T* fpm, T* res,
+                                           const int* queue, CELL cell)
+{
+    using CL = CellLayout<DIM>;
+    using FR = FaceRec<T, DIM>;
+    constexpr int NV = DIM + 2;
+    const T lam_scale = pick<T>(a.c_lambda * (1.0 / 3600.0), a.lam_scale_f);
+    const T eps = pick<T>(a.eps, a.eps_f);
+    for (int q0 = 0; q0 < nq; q0 += QC) {
+        const int qc = nq - q0 < QC ? nq - q0 : QC;
+        // 2a: project U_m and F_m of the six stencil cells (Eq. eqchara) and
+        //     split them (Eq. flxuspliting); one work item per (face, cell)
+        for (int it = threadIdx.x; it < qc * 6; it += NT) {
+            const int q = it / 6, m = it - (it / 6) * 6;
+            const int f = queue[q0 + q];
+            Roe<T, DIM> r;
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) r.u[k] = fr[(FR::U + k) * NFACE + f];
+            r.ic = fr[FR::IC * NFACE + f];
+            r.b1 = fr[FR::B1 * NFACE + f];
+            r.hq2 = fr[FR::HQ2 * NFACE + f];
+            const T am = fr[FR::AM * NFACE + f];
+            const T a0 = fr[FR::A0 * NFACE + f];
+            const T ap = fr[FR::AP * NFACE + f];
+            const int ci = cell(f, m);
+            T xu[NV], xf[NV], wv[NV], wg[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                xu[v] = cq[(CL::U + v) * NCELL + ci];
+                xf[v] = cq[(CL::F + v) * NCELL + ci];
+            }
+            proj_all<T, DIM, DIR>(r, xu, wv);
+            proj_all<T, DIM, DIR>(r, xf, wg);
+#pragma unroll
+            for (int s = 0; s < NV; ++s) {
+                const T al = s == 0 ? am : (s == NV - 1 ? ap : a0);
+                const T h = halve(wg[s]);
+                const T k = al * wv[s];   // al holds alpha / 2
+                // f+ in stencil order j-2 .. j+3, f- mirrored (j+3 .. j-2), so
+                // that both signs take the same call in 2b (neighbouring lanes
+                // hold the two signs and would otherwise diverge)
+                fpm[((q * NV + s) * 2 + 0) * 6 + m] = h + k;
+                fpm[((q * NV + s) * 2 + 1) * 6 + (5 - m)] = h - k;
+            }
+        }
+        __syncthreads();
+        // 2b: one reconstruction per (face, field, sign): Eq. eq6, eq11, eq18,
+        //     eq8-r; the minus part on the mirrored stencil j+3 .. j-1 (stored
+        //     mirrored by 2a)
+        for (int it = threadIdx.x; it < qc * NV * 2; it += NT) {
+            const int q = it / (2 * NV);
+            const int rem = it - q * (2 * NV);
+            const int s = rem >> 1, sg = rem & 1;
+            const int f = queue[q0 + q];
+            // Eq. eq27, eq29: lambda^s = c (dv^s / rho~)^2 = c w_s^2 / (3600 rho~^2)
+            const T ws = fr[(FR::W + s) * NFACE + f];
+            const T lam = lam_scale * (ws * ws) * fr[FR::IRT2 * NFACE + f];
+            // per-field hybrid: the linear scheme for a smooth field
+            const int fm_bits = (int)fr[FR::MASK * NFACE + f];
+            const int wm = (fm_bits >> s) & 1 ? W_LINEAR : a.wmode;
+            const T* v = fpm + ((q * NV + s) * 2 + sg) * 6;
+            res[(q * NV + s) * 2 + sg] = recon<T>(v[0], v[1], v[2], v[3], v[4], lam, eps, wm);
+        }
+        __syncthreads();
+        // 2c: Eq. reconstruction1 and the back-projection Eq. reconstruction2,
+        //     one work item per (face, conserved variable)
+        for (int it = threadIdx.x; it < qc * NV; it += NT) {
+            const int q = it / NV, v = it - (it / NV) * NV;
+            const int f = queue[q0 + q];
+            Roe<T, DIM> r;
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) r.u[k] = fr[(FR::U + k) * NFACE + f];
+            r.c = fr[FR::C * NFACE + f];
+            r.H = fr[FR::H * NFACE + f];
+            r.hq2 = fr[FR::HQ2 * NFACE + f];
+            T wch[NV];
+#pragma unroll
+            for (int s = 0; s < NV; ++s) wch[s] = res[(q * NV + s) * 2] + res[(q * NV + s) * 2 + 1];
+            fh[v * NFACE + f] = T(60) * back_proj_row<T, DIM, DIR>(r, wch, v);
+        }
+    }
+}
+
 // One tile of the sweep: stage, faces, WENO queue, divergence and output.
 // EXACTDET: detector difference by nested differences (mixed precision);
 // otherwise the direct six-term combination.  dt is the RK step (COMBINE
@@ -314,10 +438,18 @@ __device__ __forceinline__ T fifth_difference(T u0, T u1, T u2, T u3, T u4, T u5
 // full set of faces, and a tile that reaches the end of a line continues on
 // the next one, each piece with its own halo.  line0 and pb are unused then.
 // FX: a.fx may ask for the integer six-point sums (FP64).
+// cfl (COMBINE mode, may be null): the CFL wave speeds of the cells written
+// (cell_speed), for the step that follows.
+template <typename T, int DIM>
+struct TileCfl {
+    T inv_dx[DIM];   // 1 / dx per direction
+    T smax;          // running maximum over the cells this thread wrote
+    bool bad;        // a cell this thread wrote is not admissible
+};
 template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false,
           bool FX = sizeof(T) == 8>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int line0, int pb, T dt,
-                                           unsigned char* smem_raw)
+                                           unsigned char* smem_raw, TileCfl<T, DIM>* cfl = nullptr)
 {
     static_assert(!FLAT || LINES == 1, "flat tiles hold one line piece at a time");
     using CL = CellLayout<DIM>;
@@ -465,7 +597,6 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
 
     // sigma^s < eps_h  <=>  |60 dv^s| < 60 sqrt(eps_h) rho~ (both sides >= 0)
     const T slim = pick<T>(a.slim, a.slim_f);
-    const T lam_scale = pick<T>(a.c_lambda * (1.0 / 3600.0), a.lam_scale_f);
     const int lane = threadIdx.x & 31;
     unsigned int my_weno = 0;
 
@@ -610,83 +741,12 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     __syncthreads();
 
     // ---- phase 2: characteristic regularized WENO-IS flux of queued faces --
-    const int nq = qcount;
-    const T eps = pick<T>(a.eps, a.eps_f);
-    for (int q0 = 0; q0 < nq; q0 += QC) {
-        const int qc = nq - q0 < QC ? nq - q0 : QC;
-        // 2a: project U_m and F_m of the six stencil cells (Eq. eqchara) and
-        //     split them (Eq. flxuspliting); one work item per (face, cell)
-        for (int it = threadIdx.x; it < qc * 6; it += NT) {
-            const int q = it / 6, m = it - (it / 6) * 6;
-            const int f = queue[q0 + q];
+    weno_queue<T, DIM, DIR, NCELL, NFACE, QC, NT>(
+        a, qcount, cq, fh, fr, fpm, res, queue, [&](int f, int m) -> int {
             int l, p;
             fdec(f, l, p);
-            Roe<T, DIM> r;
-#pragma unroll
-            for (int k = 0; k < DIM; ++k) r.u[k] = fr[(FR::U + k) * NFACE + f];
-            r.ic = fr[FR::IC * NFACE + f];
-            r.b1 = fr[FR::B1 * NFACE + f];
-            r.hq2 = fr[FR::HQ2 * NFACE + f];
-            const T am = fr[FR::AM * NFACE + f];
-            const T a0 = fr[FR::A0 * NFACE + f];
-            const T ap = fr[FR::AP * NFACE + f];
-            const int ci = cidx(l, p + m);
-            T xu[NV], xf[NV], wv[NV], wg[NV];
-#pragma unroll
-            for (int v = 0; v < NV; ++v) {
-                xu[v] = cq[(CL::U + v) * NCELL + ci];
-                xf[v] = cq[(CL::F + v) * NCELL + ci];
-            }
-            proj_all<T, DIM, DIR>(r, xu, wv);
-            proj_all<T, DIM, DIR>(r, xf, wg);
-#pragma unroll
-            for (int s = 0; s < NV; ++s) {
-                const T al = s == 0 ? am : (s == NV - 1 ? ap : a0);
-                const T h = halve(wg[s]);
-                const T k = al * wv[s];   // al holds alpha / 2
-                // f+ in stencil order j-2 .. j+3, f- mirrored (j+3 .. j-2), so
-                // that both signs take the same call in 2b (neighbouring lanes
-                // hold the two signs and would otherwise diverge)
-                fpm[((q * NV + s) * 2 + 0) * 6 + m] = h + k;
-                fpm[((q * NV + s) * 2 + 1) * 6 + (5 - m)] = h - k;
-            }
-        }
-        __syncthreads();
-        // 2b: one reconstruction per (face, field, sign): Eq. eq6, eq11, eq18,
-        //     eq8-r; the minus part on the mirrored stencil j+3 .. j-1 (stored
-        //     mirrored by 2a)
-        for (int it = threadIdx.x; it < qc * NV * 2; it += NT) {
-            const int q = it / (2 * NV);
-            const int rem = it - q * (2 * NV);
-            const int s = rem >> 1, sg = rem & 1;
-            const int f = queue[q0 + q];
-            // Eq. eq27, eq29: lambda^s = c (dv^s / rho~)^2 = c w_s^2 / (3600 rho~^2)
-            const T ws = fr[(FR::W + s) * NFACE + f];
-            const T lam = lam_scale * (ws * ws) * fr[FR::IRT2 * NFACE + f];
-            // per-field hybrid: the linear scheme for a smooth field
-            const int fm_bits = (int)fr[FR::MASK * NFACE + f];
-            const int wm = (fm_bits >> s) & 1 ? W_LINEAR : a.wmode;
-            const T* v = fpm + ((q * NV + s) * 2 + sg) * 6;
-            res[(q * NV + s) * 2 + sg] = recon<T>(v[0], v[1], v[2], v[3], v[4], lam, eps, wm);
-        }
-        __syncthreads();
-        // 2c: Eq. reconstruction1 and the back-projection Eq. reconstruction2,
-        //     one work item per (face, conserved variable)
-        for (int it = threadIdx.x; it < qc * NV; it += NT) {
-            const int q = it / NV, v = it - (it / NV) * NV;
-            const int f = queue[q0 + q];
-            Roe<T, DIM> r;
-#pragma unroll
-            for (int k = 0; k < DIM; ++k) r.u[k] = fr[(FR::U + k) * NFACE + f];
-            r.c = fr[FR::C * NFACE + f];
-            r.H = fr[FR::H * NFACE + f];
-            r.hq2 = fr[FR::HQ2 * NFACE + f];
-            T wch[NV];
-#pragma unroll
-            for (int s = 0; s < NV; ++s) wch[s] = res[(q * NV + s) * 2] + res[(q * NV + s) * 2 + 1];
-            fh[v * NFACE + f] = T(60) * back_proj_row<T, DIM, DIR>(r, wch, v);
-        }
-    }
+            return cidx(l, p + m);
+        });
     __syncthreads();
     if (threadIdx.x == 0 && a.weno_count != nullptr && wcount != 0u)
         atomicAdd(a.weno_count, (unsigned long long)wcount);
@@ -757,6 +817,11 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
             for (int k = 0; k < DIM; ++k) m2 = fmaT(nu[1 + k], nu[1 + k], m2);
             const T chk = T(2) * nu[0] * nu[DIM + 1] - m2;
             if (!(nu[0] > T(0)) || !(chk > T(0)) || !isfinite(chk)) bad = true;
+            if (cfl != nullptr) {
+                T sp;
+                if (!cell_speed<T, DIM>(nu, gamma, cfl->inv_dx, sp)) cfl->bad = true;
+                else cfl->smax = max_nn(cfl->smax, sp);
+            }
         }
     }
     __syncthreads();
@@ -797,6 +862,16 @@ struct GhostArgs {
     double stage_c, t_fixed;
 };
 
+// warp maximum of non-negative values on their bit patterns (a double compare
+// would take the FP64 pipe in float kernels too)
+template <typename T>
+__device__ __forceinline__ T warp_max_nn(T v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_nn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
 // ------------------------------------------------------- CFL reduction
 struct CflArgs {
     const void* U;
@@ -813,40 +888,6 @@ __device__ __forceinline__ double warp_max(double v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = maxT(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
-}
-
-// CFL wave-speed sum sum_d (|u_d| + c) / dx_d of one cell; false if the cell
-// is not admissible (rho <= 0, p <= 0 or non-finite).  Shared by the grid
-// reduction and the batched solver so both take identical time steps.
-template <typename T, int DIM>
-__device__ __forceinline__ bool cell_speed(const T* u, T gamma, const T* inv_dx, T& s)
-{
-    const T gm1 = gamma - T(1);
-    const T irho = Ar<T>::rcp_f(u[0]);
-    T ke2 = T(0);
-    T vel[DIM];
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) { vel[d] = u[1 + d] * irho; ke2 = fmaT(u[1 + d], vel[d], ke2); }
-    const T p = gm1 * fmaT(T(-0.5), ke2, u[DIM + 1]);
-    const T c2 = gamma * p * irho;
-    const T c = c2 * Ar<T>::rsqrt_(c2);   // NaN for p <= 0, rejected below
-    s = T(0);
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) s = fmaT(absT(vel[d]) + c, inv_dx[d], s);
-    return (u[0] > T(0)) && (p > T(0)) && isfinite(s);
-}
-
-// dt = CFL / smax clipped to t_end (the clipped step lands exactly on t_end)
-__device__ __forceinline__ double cfl_step(double cfl, double smax, double t, double t_end, int* clipped)
-{
-    double dt = 0.0;
-    *clipped = 0;
-    if (t < t_end) {
-        if (smax > 0.0) dt = cfl / smax;
-        if (t + dt >= t_end) { dt = t_end - t; *clipped = 1; }
-        if (!(dt > 0.0)) { dt = 0.0; *clipped = 0; }
-    }
-    return dt;
 }
 
 template <typename T, int DIM>
