@@ -66,6 +66,7 @@ struct weno_ctx {
     double smax_floor = 0.0;    // CFL wave-speed sum of the fixed boundary states
     cudaGraphExec_t graph[3] = {nullptr, nullptr, nullptr};
     bool graphs_ready = false;
+    int run1d = 0;              // CTAs of the one-launch stepping of a small 1D problem (0: kernels per step)
     std::string err;
 };
 
@@ -290,6 +291,20 @@ static weno_status build_graphs(weno_ctx* ctx)
     return WENO_OK;
 }
 
+// up to `steps` steps of a small 1D problem in one launch (t_end is set)
+static cudaError_t issue_run1d(weno_ctx* c, int steps, cudaStream_t s)
+{
+    wis::Run1DArgs r;
+    r.a = sweep_args(c, 0);
+    r.a.tm = c->tm;
+    for (int k = 0; k < 3; ++k) r.buf[k] = c->buf[k];
+    r.nsteps = steps;
+    r.cfl = c->p.cfl;
+    r.smax_floor = c->smax_floor;
+    if (c->prec == WENO_FP64) return wis::run1d_f64(r, c->run1d, s);
+    return c->prec == WENO_FP32 ? wis::run1d_f32(r, c->run1d, s) : wis::run1d_mixed(r, c->run1d, s);
+}
+
 static weno_status read_time(weno_ctx* ctx)
 {
     CK(cudaMemcpyAsync(ctx->tm_host, ctx->tm, sizeof(DevTime), cudaMemcpyDeviceToHost, ctx->stream));
@@ -500,6 +515,22 @@ weno_status weno_create(const weno_grid* grid, const weno_params* params, void* 
         ctx->x_first = dim >= 2 && ctx->tile[dim - 1] == 7;
     }
     if (dim == 1) ctx->tile[0] = 0;
+    // short 1D lines step in one launch (global Lax-Friedrichs needs its
+    // per-stage maxima over the domain and keeps the kernels per step)
+    if (dim == 1 && ctx->p.splitting != wis::SPLIT_LF) {
+        int most = 0;
+        e = ctx->prec == WENO_FP64 ? wis::run1d_prepare_f64(&most)
+                                   : (ctx->prec == WENO_FP32 ? wis::run1d_prepare_f32(&most)
+                                                             : wis::run1d_prepare_mixed(&most));
+        if (e != cudaSuccess) {
+            g_create_err = std::string("weno_create: ") + cudaGetErrorString(e);
+            free_all(ctx);
+            delete ctx;
+            return WENO_ERR_CUDA;
+        }
+        if (most > 0) ctx->run1d = wis::run1d_ctas(ctx->n[0], ctx->prec == WENO_FP64 ? wis::run1d_cells<double>() : wis::run1d_cells<float>(),
+                                                      most);
+    }
     *out = ctx;
     return WENO_OK;
 }
@@ -786,7 +817,7 @@ weno_status weno_step(weno_ctx* ctx, double t_end, double* dt_taken)
     if (st != WENO_OK) return st;
     const double t0 = ctx->tm_host->t;
     if ((st = set_t_end(ctx, t_end)) != WENO_OK) return st;
-    CK(issue_step(ctx, ctx->phase, ctx->stream));
+    CK(ctx->run1d ? issue_run1d(ctx, 1, ctx->stream) : issue_step(ctx, ctx->phase, ctx->stream));
     st = finish_steps(ctx);
     if (dt_taken) *dt_taken = ctx->tm_host->t - t0;
     return st;
@@ -799,14 +830,17 @@ weno_status weno_advance(weno_ctx* ctx, double t_end, int max_steps, int* steps_
     weno_status st = read_time(ctx);
     if (st != WENO_OK) return st;
     const long long s0 = ctx->tm_host->steps;
-    if ((st = build_graphs(ctx)) != WENO_OK) return st;
+    if (!ctx->run1d && (st = build_graphs(ctx)) != WENO_OK) return st;
     if ((st = set_t_end(ctx, t_end)) != WENO_OK) return st;
     int remaining = max_steps;
-    const int chunk = 64;
+    // a few milliseconds of work between two looks at the time
+    const int chunk = ctx->run1d ? 1024 : 64;
     while (remaining > 0 && ctx->tm_host->status == 0 && ctx->tm_host->t < t_end) {
         const int k = remaining < chunk ? remaining : chunk;
         const long long before = ctx->tm_host->steps;
-        for (int i = 0; i < k; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
+        if (ctx->run1d) CK(issue_run1d(ctx, k, ctx->stream));
+        else
+            for (int i = 0; i < k; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
         if ((st = read_time(ctx)) != WENO_OK) return st;
         remaining -= k;
         if (ctx->tm_host->steps - before < k) break;
@@ -818,11 +852,15 @@ weno_status weno_advance(weno_ctx* ctx, double t_end, int max_steps, int* steps_
 weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps)
 {
     if (!ctx || nsteps < 0) return WENO_ERR_INVALID_ARG;
-    weno_status st = build_graphs(ctx);
+    weno_status st = ctx->run1d ? WENO_OK : build_graphs(ctx);
     if (st != WENO_OK) return st;
     wis::k_set_tend<<<1, 1, 0, ctx->stream>>>(ctx->tm, t_end);
     CK(cudaGetLastError());
-    for (int i = 0; i < nsteps; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
+    if (ctx->run1d) {
+        if (nsteps > 0) CK(issue_run1d(ctx, nsteps, ctx->stream));
+    } else {
+        for (int i = 0; i < nsteps; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
+    }
     ctx->phase = (ctx->phase + nsteps) % 3;
     return WENO_OK;
 }

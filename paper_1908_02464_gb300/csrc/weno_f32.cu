@@ -34,4 +34,7 @@ cudaError_t lf_f32(int dim, const CflArgs& a, unsigned long long* out, int nsm, 
     return launch_lf_t<float>(dim, a, out, nsm, s);
 }
 
+cudaError_t run1d_prepare_f32(int* max_cluster) { return run1d_prepare<float, false>(max_cluster); }
+cudaError_t run1d_f32(const Run1DArgs& r, int ctas, cudaStream_t s) { return launch_run1d<float, false>(r, ctas, s); }
+
 }  // namespace wis

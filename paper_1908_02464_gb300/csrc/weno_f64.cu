@@ -33,4 +33,7 @@ cudaError_t lf_f64(int dim, const CflArgs& a, unsigned long long* out, int nsm, 
     return launch_lf_t<double>(dim, a, out, nsm, s);
 }
 
+cudaError_t run1d_prepare_f64(int* max_cluster) { return run1d_prepare<double, false>(max_cluster); }
+cudaError_t run1d_f64(const Run1DArgs& r, int ctas, cudaStream_t s) { return launch_run1d<double, false>(r, ctas, s); }
+
 }  // namespace wis

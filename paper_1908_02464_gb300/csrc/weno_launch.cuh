@@ -9,6 +9,7 @@
 #include "weno_adjoint.cuh"
 #include "weno_kernels.cuh"
 #include "weno_march.cuh"
+#include "weno_run1d.cuh"
 
 namespace wis {
 
@@ -269,6 +270,12 @@ cudaError_t ghost_adj_f32(int dim, const GhostArgs& a, const void* ghost, void* 
 cudaError_t sweep_f64(int dim, int dir, int variant, const SweepArgs& a, cudaStream_t s);
 cudaError_t sweep_f32(int dim, int dir, int variant, const SweepArgs& a, cudaStream_t s);
 cudaError_t sweep_mixed(int dim, int dir, int variant, const SweepArgs& a, cudaStream_t s);
+cudaError_t run1d_prepare_f64(int* max_cluster);
+cudaError_t run1d_prepare_f32(int* max_cluster);
+cudaError_t run1d_prepare_mixed(int* max_cluster);
+cudaError_t run1d_f64(const Run1DArgs& r, int ctas, cudaStream_t s);
+cudaError_t run1d_f32(const Run1DArgs& r, int ctas, cudaStream_t s);
+cudaError_t run1d_mixed(const Run1DArgs& r, int ctas, cudaStream_t s);
 cudaError_t cfl_f64(int dim, const CflArgs& a, int nsm, cudaStream_t s);
 cudaError_t cfl_f32(int dim, const CflArgs& a, int nsm, cudaStream_t s);
 cudaError_t lf_f64(int dim, const CflArgs& a, unsigned long long* out, int nsm, cudaStream_t s);
