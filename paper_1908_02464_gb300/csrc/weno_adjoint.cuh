@@ -7,7 +7,7 @@
 // face recomputes its forward quantities (Roe state, detector, LLF speeds,
 // projections, reconstructions: nothing is stored by the forward pass) and
 // then runs the reverse of each step:
-//   back-projection (Eq. reconstruction2)  -> back_proj_adj
+//   back-projection (Eq. reconstruction2)  -> the face steps of vjp_weno_line
 //   reconstruction (Eq. eq6, eq11, eq18, eq8-r) -> recon_adj
 //   splitting and projection (Eq. flxuspliting, eqchara) -> proj_all_adj
 //   regularization parameter (Eq. eq27-29) and detector (Eq. eq28)
@@ -26,13 +26,14 @@
 // face adds Roe-field bars for its two neighbours and one bar per LLF speed
 // for the cell attaining it.
 //
-// Each direction runs in two passes over the same tiles.  Pass 0 takes the
-// linear-upwind faces, writes (or adds) the gradient, and flags each tile
-// that has a WENO face among the faces it recomputes.  Pass 1 runs on the
-// flagged tiles only, takes their WENO faces and adds their contributions.
-// The WENO reverse needs the registers of the 6 x nvar projections and
-// their bars; keeping it out of pass 0 lets the common linear-upwind tiles
-// run with far fewer registers and more resident warps.
+// Each direction runs in two passes over the same tiles.  Pass 0 (k_vjp)
+// takes the linear-upwind faces, writes (or adds) the gradient, and lists
+// each tile that has a WENO face among the faces it recomputes, with a mask
+// of its lines.  Pass 1 (k_vjp_weno) takes the WENO faces of the listed lines
+// and adds their contributions.  The WENO reverse of a face holds 6 x nvar
+// projections and their bars; pass 1 spreads it over the lanes as the forward
+// sweep does, and keeping it out of pass 0 lets the common linear-upwind
+// tiles run with far fewer registers and more resident warps.
 // Contributions to ghost cells go to a per-line buffer that a second kernel
 // maps back through the boundary conditions.
 #pragma once
@@ -156,38 +157,6 @@ __device__ __forceinline__ void proj_all_adj(const Roe<T, DIM>& r, const T* x, c
     for (int k = 0; k < DIM; ++k) { rb.u[k] -= yb * x[1 + k]; xb[1 + k] -= yb * r.u[k]; }
 }
 
-// adjoint of out = R w (back_proj_add): sets wb, accumulates rb
-template <typename T, int DIM, int DIR>
-__device__ __forceinline__ void back_proj_adj(const Roe<T, DIM>& r, const T* w, const T* ob, T* wb,
-                                              RoeBar<T, DIM>& rb)
-{
-    constexpr int LAST = DIM + 1;
-    const T sum = w[0] + w[1] + w[LAST];
-    const T dif = w[LAST] - w[0];
-    const T oE = ob[LAST];
-    T sumb = ob[0];
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) { sumb = fmaT(ob[1 + k], r.u[k], sumb); rb.u[k] += ob[1 + k] * sum; }
-    const T difb = (ob[1 + DIR] + oE * r.u[DIR]) * r.c;
-    rb.c += (ob[1 + DIR] + oE * r.u[DIR]) * dif;
-    rb.u[DIR] += oE * r.c * dif;
-#pragma unroll
-    for (int s = 0; s <= LAST; ++s) wb[s] = T(0);
-    int s = 2;
-#pragma unroll
-    for (int k = 0; k < DIM; ++k) {
-        if (k == DIR) continue;
-        wb[s] = ob[1 + k] + oE * r.u[k];
-        rb.u[k] += oE * w[s];
-        ++s;
-    }
-    rb.H += oE * (w[0] + w[LAST]);
-    rb.hq2 += oE * w[1];
-    wb[0] += oE * r.H + sumb - difb;
-    wb[1] += oE * r.hq2 + sumb;
-    wb[LAST] += oE * r.H + sumb + difb;
-}
-
 // adjoint of the Roe average; gab/gbb: bars of the Roe fields of cells j and
 // j+1, relative to CL::SU (sqrt(rho) u at 0 .. DIM-1, sqrt(rho) H at DIM,
 // sqrt(rho) at DIM + 1)
@@ -221,9 +190,14 @@ __device__ __forceinline__ void roe_adj(GA get_a, GB get_b, T gamma, const Roe<T
     gbb[DIM + 1] += sb_ + rb.rt * sa;
 }
 
-// adjoint of the reconstruction: fb -> bars of a..e (accumulated) and of lam
+// 1 / x of a positive normal number: refined in double, rounded in float
+__device__ __forceinline__ double inv_pos(double x) { return rcp_newton(x); }
+__device__ __forceinline__ float inv_pos(float x) { return 1.0f / x; }
+
+// adjoint of the reconstruction: fb -> bars of a..e (set) and of lam; returns
+// the reconstructed value
 template <typename T>
-__device__ __forceinline__ void recon_adj(T a, T b, T c, T d, T e, T lam, T eps, T fb, T* xb, T& lamb)
+__device__ __forceinline__ T recon_adj(T a, T b, T c, T d, T e, T lam, T eps, T fb, T* xb, T& lamb)
 {
     const T q0 = T(0.5) * (c + d);
     const T q1 = fmaT(T(1.5), c, T(-0.5) * b);
@@ -241,15 +215,15 @@ __device__ __forceinline__ void recon_adj(T a, T b, T c, T d, T e, T lam, T eps,
     const T dk[4] = {T(0.4), T(0.2), T(0.3), T(0.1)};
     const T beta[4] = {b0, b1, be2, be3};
     const T lt = lam * tau;
-    T D[4], al[4];
+    T iD[4], al[4];
     T S = T(0);
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        D[k] = fmaT(lam, beta[k], (k < 2 ? E : T(0)) + eps);
-        al[k] = dk[k] * (T(1) + lt / D[k]);
+        iD[k] = inv_pos(fmaT(lam, beta[k], (k < 2 ? E : T(0)) + eps));
+        al[k] = dk[k] * (T(1) + lt * iD[k]);
         S += al[k];
     }
-    const T iS = T(1) / S;
+    const T iS = inv_pos(S);
     const T q[4] = {q0, q1, q2, q3};
     T fh = T(0);
 #pragma unroll
@@ -261,9 +235,9 @@ __device__ __forceinline__ void recon_adj(T a, T b, T c, T d, T e, T lam, T eps,
     for (int k = 0; k < 4; ++k) {
         qb[k] = fb * al[k] * iS;
         const T alb = (q[k] - fh) * fb * iS;
-        const T r = alb * dk[k] / D[k];
+        const T r = alb * dk[k] * iD[k];
         ltb += r;
-        const T Db = -r * (lt / D[k]);
+        const T Db = -r * (lt * iD[k]);
         lamb += Db * beta[k];
         betab[k] = Db * lam;
         if (k < 2) Eb += Db;
@@ -292,7 +266,8 @@ __device__ __forceinline__ void recon_adj(T a, T b, T c, T d, T e, T lam, T eps,
     cb += T(0.5) * qb[0] + T(1.5) * qb[1] + T(1.0 / 3.0) * qb[2] + T(11.0 / 6.0) * qb[3];
     db += T(0.5) * qb[0] + T(5.0 / 6.0) * qb[2];
     eb += T(-1.0 / 6.0) * qb[2];
-    xb[0] += ab; xb[1] += bb; xb[2] += cb; xb[3] += db; xb[4] += eb;
+    xb[0] = ab; xb[1] = bb; xb[2] = cb; xb[3] = db; xb[4] = eb;
+    return fh;
 }
 
 struct VjpArgs {
@@ -301,7 +276,8 @@ struct VjpArgs {
     void* G;            // gradient, interior only (written / accumulated)
     void* ghost;        // [line][6][NV] gradients of ghost cells
     int* n_weno_tiles;  // tiles of this direction with a WENO face (zero before pass 0)
-    int* weno_tiles;    // their linear tile indices, in no particular order (pass 0 appends)
+    int2* weno_tiles;   // their linear indices and the mask of their lines with one, in no
+                        // particular order (pass 0 appends)
     int tiles[3];       // tile grid of this direction (set by the launcher)
     int accumulate;     // 0: G = ..., 1: G += ... (pass 0; pass 1 always adds)
     int n[3];
@@ -331,7 +307,7 @@ template <typename T, int DIM, int DIR> struct VjpTile {
     static constexpr int NT = LINES * (SEG + 5);
 };
 
-template <typename T, int DIM, int DIR, int PASS>
+template <typename T, int DIM, int DIR>
 struct VjpSmem {
     static constexpr int LINES = VjpTile<T, DIM, DIR>::LINES;
     static constexpr int SEG = VjpTile<T, DIM, DIR>::SEG;
@@ -340,48 +316,37 @@ struct VjpSmem {
     static constexpr int LNF = LINES * NF, LNC = LINES * NC;
     static constexpr int NQ = CellLayout<DIM>::NQ;
     static constexpr int NV = DIM + 2;
-    // per face: U and F bars of the six stencil cells (pass 1) or the two
-    // bar vectors of a linear-upwind face (pass 0, NUF entries), Roe-field
-    // bars of cells 2 and 3 (the face's neighbours), the three LLF speed
-    // bars, and (as one int) the stencil slots of the cells attaining the
-    // speeds and whether the pass takes the face
+    // per face: the two bar vectors of a linear-upwind face (NUF entries),
+    // Roe-field bars of cells 2 and 3 (the face's neighbours), the three LLF
+    // speed bars, and (as one int) the stencil slots of the cells attaining
+    // the speeds and whether the pass takes the face
     // per cell after the record: 1/sqrt(rho), 1/c and, in FP64, p and c
     // (in FP32 the per-cell reverse recomputes those two: two more staged
     // rows cost the shared-memory-bound float tiles more than they save)
     static constexpr int NX = sizeof(T) == 8 ? 4 : 2;
     static constexpr int NUF = 2 * NV;
-    static constexpr int NUFF = PASS == 0 ? NUF : 6 * NUF;
     static constexpr int NRB = DIM + 2;
-    static constexpr int NFB = NUFF + 2 * NRB + 3;
+    static constexpr int NFB = NUF + 2 * NRB + 3;
     static constexpr size_t bytes =
         sizeof(T) * ((size_t)(NQ + NX) * LNC + (size_t)NV * LNC + (size_t)LNF * NFB) + sizeof(int) * (size_t)LNF;
 };
 
-// Residency of the WENO pass: its per-face reverse needs more than 255
-// registers, which leaves 8 warps per SM in FP64.  FP32 code needs more
-// warps to hide its latencies, so its register count is capped at 128 (8
-// CTAs of the 64-thread x tiles, 2 of the 256-thread y/z tiles) at the cost
-// of spills.
-template <typename T, int NT, int PASS> struct VjpMinBlocks {
-    static constexpr int value = PASS == 0 ? 1 : (sizeof(T) == 4 ? (NT == 64 ? 8 : 2) : 1);
-};
-
 // One tile of one direction of the VJP: tile (bx, by, bz) = LINES grid lines
 // x SEG cells; shared arrays hold position p of line l at p * LINES + l.
-// Returns (to every thread, pass 0) whether a face of the tile took WENO.
-template <typename T, int DIM, int DIR, int PASS>
-__device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int bz, unsigned char* smem_raw)
+// Returns (to every thread) the mask of its lines that have a WENO face.
+template <typename T, int DIM, int DIR>
+__device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int by, int bz, unsigned char* smem_raw)
 {
     using CL = CellLayout<DIM>;
-    using SM = VjpSmem<T, DIM, DIR, PASS>;
+    using SM = VjpSmem<T, DIM, DIR>;
     constexpr int NV = DIM + 2, NQ = CL::NQ, SEG = SM::SEG, NF = SM::NF;
     constexpr int LINES = SM::LINES, LNF = SM::LNF, LNC = SM::LNC;
     constexpr int NT = VjpTile<T, DIM, DIR>::NT;
-    constexpr int NUF = SM::NUF, NUFF = SM::NUFF, NRB = SM::NRB;
+    constexpr int NUF = SM::NUF, NRB = SM::NRB;
     T* cq = reinterpret_cast<T*>(smem_raw);   // [NQ + NX][NC][LINES] records, 1/sqrt(rho), 1/c (, p, c)
     T* wq = cq + (NQ + SM::NX) * LNC;         // [NV][NC][LINES] cotangent
-    T* UF = wq + NV * LNC;                    // [NF][LINES][NUFF] U and F bars (see below)
-    T* RB = UF + LNF * NUFF;                  // [NF][LINES][2][NRB] Roe-field bars of cells 2 and 3
+    T* UF = wq + NV * LNC;                    // [NF][LINES][NUF] bars of dU and of the central-flux sum
+    T* RB = UF + LNF * NUF;                  // [NF][LINES][2][NRB] Roe-field bars of cells 2 and 3
     T* SP = RB + LNF * 2 * NRB;               // [NF][LINES][3] LLF speed bars
     int* SL = reinterpret_cast<int*>(SP + LNF * 3);   // [NF][LINES] slots attaining the speeds, face taken
     constexpr int SKIP = 1 << 12;   // the face belongs to the other pass
@@ -470,17 +435,18 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
     const T slim = T(a.slim);
     const T lam_k = T(a.c_lambda / 3600.0);
     const T eps = T(a.eps), inv_dx = T(a.inv_dx);
-    bool has_weno = false;
+    __shared__ unsigned int weno_lines;
+    if (threadIdx.x == 0) weno_lines = 0u;
+    __syncthreads();
     for (int ff = threadIdx.x; ff < LNF; ff += NT) {
         const int f = ff / LINES, l = ff - (ff / LINES) * LINES;
         const int face = c0 - 2 + f;            // face i' between cells i'-1 and i'
         if (l >= nlx || face < 0 || face > nd) continue;
         // stencil cell j-2 = face-3 sits at position f of line l
         auto rec = [&](int m, int kk) -> T { return cq[kk * LNC + (f + m) * LINES + l]; };
-        // pass 1 (WENO faces): U and F bars of each of the six stencil
-        // cells; pass 0 (linear-upwind faces): the bars of the detector
-        // difference (U slots) and of the central-flux sum (F slots)
-        T* UFf = UF + (size_t)ff * NUFF;
+        // the bars of the detector difference (U slots) and of the
+        // central-flux sum (F slots)
+        T* UFf = UF + (size_t)ff * NUF;
         T* RBf = RB + (size_t)ff * 2 * NRB;    // Roe-field bars of cells 2 and 3
         // cotangent of the face flux: (w_{right} - w_{left}) / dx
         T phi[NV];
@@ -505,8 +471,8 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
         bool smooth = a.hybrid != 0;
 #pragma unroll
         for (int s = 0; s < NV; ++s) smooth = smooth && abs_lt(w[s], lim);
-        if (smooth != (PASS == 0)) {   // the other pass takes this face
-            has_weno = has_weno || !smooth;
+        if (!smooth) {   // pass 1 takes this face
+            atomicOr(&weno_lines, 1u << l);
             SL[ff] = SKIP;
             continue;
         }
@@ -526,7 +492,7 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
         T wb[NV], dUb[NV];
 #pragma unroll
         for (int s = 0; s < NV; ++s) { wb[s] = T(0); dUb[s] = T(0); }
-        if constexpr (PASS == 0) {
+        {
             // F = [central(F) + a0 dU + k0 R^{u-c} + k3 R^{u+c}] / 60 with
             // k0 = (am - a0) w_0, k3 = (ap - a0) w_last, the form the forward
             // sweep evaluates (ups_dissipation_add); the gather applies the
@@ -566,102 +532,11 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
                 dUb[v] = a0 * Fb[v];
             }
             alb_0 = dot - alb_m - alb_p;
-        } else {
-            // projections of the six cells, all fields
-            T vv[6][NV], gg[6][NV];
-#pragma unroll
-            for (int m = 0; m < 6; ++m) {
-                T xu[NV], xf[NV];
-#pragma unroll
-                for (int v = 0; v < NV; ++v) { xu[v] = rec(m, CL::U + v); xf[v] = rec(m, CL::F + v); }
-                proj_all<T, DIM, DIR>(r, xu, vv[m]);
-                proj_all<T, DIM, DIR>(r, xf, gg[m]);
-            }
-            const T irt2 = T(1) / (r.rt * r.rt);
-            T wch[NV];
-            T lam[NV];
-#pragma unroll
-            for (int s = 0; s < NV; ++s) {
-                const T al = s == 0 ? am : (s == NV - 1 ? ap : a0);
-                lam[s] = lam_k * (w[s] * w[s]) * irt2;
-                T fp[6], fm[6];
-#pragma unroll
-                for (int m = 0; m < 6; ++m) {
-                    const T h = T(0.5) * gg[m][s], kq = T(0.5) * al * vv[m][s];
-                    fp[m] = h + kq;
-                    fm[m] = h - kq;
-                }
-                wch[s] = recon<T>(fp[0], fp[1], fp[2], fp[3], fp[4], lam[s], eps) +
-                         recon<T>(fm[5], fm[4], fm[3], fm[2], fm[1], lam[s], eps);
-            }
-            T wchb[NV];
-            back_proj_adj<T, DIM, DIR>(r, wch, phi, wchb, rb);
-            T vb[6][NV], gbar[6][NV];
-#pragma unroll
-            for (int m = 0; m < 6; ++m)
-#pragma unroll
-                for (int s = 0; s < NV; ++s) { vb[m][s] = T(0); gbar[m][s] = T(0); }
-#pragma unroll
-            for (int s = 0; s < NV; ++s) {
-                const T al = s == 0 ? am : (s == NV - 1 ? ap : a0);
-                T fp[6], fm[6];
-#pragma unroll
-                for (int m = 0; m < 6; ++m) {
-                    const T h = T(0.5) * gg[m][s], kq = T(0.5) * al * vv[m][s];
-                    fp[m] = h + kq;
-                    fm[m] = h - kq;
-                }
-                T xp[5] = {T(0), T(0), T(0), T(0), T(0)}, xm[5] = {T(0), T(0), T(0), T(0), T(0)};
-                T lbp, lbm;
-                recon_adj<T>(fp[0], fp[1], fp[2], fp[3], fp[4], lam[s], eps, wchb[s], xp, lbp);
-                recon_adj<T>(fm[5], fm[4], fm[3], fm[2], fm[1], lam[s], eps, wchb[s], xm, lbm);
-                // fm input order was m = 5, 4, 3, 2, 1
-                T fpb[6] = {xp[0], xp[1], xp[2], xp[3], xp[4], T(0)};
-                T fmb[6] = {T(0), xm[4], xm[3], xm[2], xm[1], xm[0]};
-                T alb = T(0);
-#pragma unroll
-                for (int m = 0; m < 6; ++m) {
-                    gbar[m][s] += T(0.5) * (fpb[m] + fmb[m]);
-                    vb[m][s] += T(0.5) * al * (fpb[m] - fmb[m]);
-                    alb += T(0.5) * vv[m][s] * (fpb[m] - fmb[m]);
-                }
-                if (s == 0) alb_m += alb;
-                else if (s == NV - 1) alb_p += alb;
-                else alb_0 += alb;
-                // lam = c w^2 / (3600 rt^2)
-                const T lb = lbp + lbm;
-                wb[s] += lb * T(2) * lam_k * w[s] * irt2;
-                rb.rt += lb * (T(-2) * lam[s] / r.rt);
-            }
-#pragma unroll
-            for (int m = 0; m < 6; ++m) {
-                T xu[NV], xf[NV], xub[NV], xfb[NV];
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    xu[v] = rec(m, CL::U + v); xf[v] = rec(m, CL::F + v);
-                    xub[v] = T(0); xfb[v] = T(0);
-                }
-                proj_all_adj<T, DIM, DIR>(r, xu, vb[m], xub, rb);
-                proj_all_adj<T, DIM, DIR>(r, xf, gbar[m], xfb, rb);
-#pragma unroll
-                for (int v = 0; v < NV; ++v) {
-                    UFf[m * NUF + CL::U + v] = xub[v];
-                    UFf[m * NUF + CL::F + v] = xfb[v];
-                }
-            }
         }
         // detector: w = L dU, dU = (U0 - U5) + 5 (U4 - U1) + 10 (U2 - U3)
         proj_all_adj<T, DIM, DIR>(r, dU, wb, dUb, rb);
-        if constexpr (PASS == 0) {
 #pragma unroll
-            for (int v = 0; v < NV; ++v) UFf[CL::U + v] = dUb[v];
-        } else {
-            const T cd[6] = {T(1), T(-5), T(10), T(-10), T(5), T(-1)};
-#pragma unroll
-            for (int m = 0; m < 6; ++m)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) UFf[m * NUF + CL::U + v] += cd[m] * dUb[v];
-        }
+        for (int v = 0; v < NV; ++v) UFf[CL::U + v] = dUb[v];
         SP[ff * 3 + 0] = alb_m;
         SP[ff * 3 + 1] = alb_0;
         SP[ff * 3 + 2] = alb_p;
@@ -670,7 +545,8 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
         for (int kk = 0; kk < 2 * NRB; ++kk) RBf[kk] = T(0);
         roe_adj<T, DIM>(ga, gb, gamma, r, rb, RBf, RBf + NRB);
     }
-    const bool any_weno = __syncthreads_or(has_weno ? 1 : 0) != 0;
+    __syncthreads();
+    const unsigned int any_weno = weno_lines;
 
     // ---- gather per cell: faces i' in [i-2, i+3], stencil slot m = i - i' + 3
     T* Gg = reinterpret_cast<T*>(a.G);
@@ -686,11 +562,10 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
         T qb[NQ];
 #pragma unroll
         for (int kk = 0; kk < NQ; ++kk) qb[kk] = T(0);
-        bool touched = false;
-        // pass 0 in FP64: the face (index into the face arrays) that gives
+        // FP64: the face (index into the face arrays) that gives
         // this cell its stencil slot m, -1 where none does
         int fslot[6] = {-1, -1, -1, -1, -1, -1};
-        // central-flux and detector weights of stencil slot m (pass 0 in FP32)
+        // central-flux and detector weights of stencil slot m (FP32)
         constexpr T cf[6] = {T(1), T(-8), T(37), T(37), T(-8), T(1)};
         constexpr T cd[6] = {T(1), T(-5), T(10), T(-10), T(5), T(-1)};
 #pragma unroll
@@ -702,17 +577,12 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
             const int ff = f * LINES + l;
             const int sl = SL[ff];
             if (sl & SKIP) continue;
-            touched = true;
             // the entries this cell receives from face fi, in the record
             // layout; the others are zero for it
-            if constexpr (PASS == 1) {
-                const T* uf = UF + (size_t)ff * NUFF + m * NUF;
-#pragma unroll
-                for (int kk = 0; kk < NUF; ++kk) qb[kk] += uf[kk];
-            } else if constexpr (sizeof(T) == 8) {
+            if constexpr (sizeof(T) == 8) {
                 fslot[m] = ff;
             } else {
-                const T* uf = UF + (size_t)ff * NUFF;
+                const T* uf = UF + (size_t)ff * NUF;
 #pragma unroll
                 for (int v = 0; v < NV; ++v) {
                     qb[CL::U + v] = fmaT(cd[m], uf[CL::U + v], qb[CL::U + v]);
@@ -728,7 +598,7 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
             if (((sl >> 4) & 15) == m) qb[CL::L0] += SP[ff * 3 + 1];
             if (((sl >> 8) & 15) == m) qb[CL::LP] += SP[ff * 3 + 2];
         }
-        if constexpr (PASS == 0 && sizeof(T) == 8) {
+        if constexpr (sizeof(T) == 8) {
             // stencil weights of slot m: detector (1, -5, 10, -10, 5, -1)
             // on the U slots, central flux (1, -8, 37, 37, -8, 1) on the F
             // slots, applied as sums and differences of the symmetric pairs
@@ -740,7 +610,7 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
                 T bu[6], bf[6];
 #pragma unroll
                 for (int m = 0; m < 6; ++m) {
-                    const T* uf = UF + (size_t)(fslot[m] < 0 ? 0 : fslot[m]) * NUFF;
+                    const T* uf = UF + (size_t)(fslot[m] < 0 ? 0 : fslot[m]) * NUF;
                     bu[m] = fslot[m] < 0 ? T(0) : uf[CL::U + v];
                     bf[m] = fslot[m] < 0 ? T(0) : uf[CL::F + v];
                 }
@@ -748,7 +618,6 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
                 qb[CL::F + v] = fmaT(T(37), bf[2] + bf[3], fmaT(T(-8), bf[1] + bf[4], bf[0] + bf[5]));
             }
         }
-        if (PASS == 1 && !touched) continue;
         const int pc = cell - (c0 - 5);
         T U[NV], Ub[NV];
 #pragma unroll
@@ -773,7 +642,7 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
             const long long g = base0 + l + (long long)cell * sd;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                if (PASS == 1 || a.accumulate) Gg[g + v * a.sv] += Ub[v];
+                if (a.accumulate) Gg[g + v * a.sv] += Ub[v];
                 else Gg[g + v * a.sv] = Ub[v];
             }
         } else {
@@ -783,35 +652,407 @@ __device__ __forceinline__ bool vjp_tile(const VjpArgs& a, int bx, int by, int b
             const int slot = gl ? (-cell - 1) : (3 + cell - nd);   // 0..2 left (-1,-2,-3), 3..5 right
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                if (PASS == 1) ghost[(line * 6 + slot) * NV + v] += Ub[v];
-                else ghost[(line * 6 + slot) * NV + v] = Ub[v];
+                ghost[(line * 6 + slot) * NV + v] = Ub[v];
             }
         }
     }
     return any_weno;
 }
 
-// Pass 0: one CTA per tile; a tile with a WENO face appends its index to
-// the list.  Pass 1: a grid of resident CTAs takes the listed tiles in turn
-// (each tile writes only its own cells and ghost slots, so the order in
-// which the tiles are taken does not change the result).
-template <typename T, int DIM, int DIR, int PASS>
-__global__ void __launch_bounds__(VjpTile<T, DIM, DIR>::NT, VjpMinBlocks<T, VjpTile<T, DIM, DIR>::NT, PASS>::value)
-    k_vjp(VjpArgs a)
+// Pass 0: one CTA per tile; a tile with a WENO face appends itself to the
+// list.
+template <typename T, int DIM, int DIR>
+__global__ void __launch_bounds__(VjpTile<T, DIM, DIR>::NT) k_vjp(VjpArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    if constexpr (PASS == 0) {
-        const bool any = vjp_tile<T, DIM, DIR, 0>(a, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
-        if (any && threadIdx.x == 0)
-            a.weno_tiles[atomicAdd(a.n_weno_tiles, 1)] = blockIdx.x + a.tiles[0] * (blockIdx.y + a.tiles[1] * blockIdx.z);
-    } else {
-        const int n = *a.n_weno_tiles;
-        for (int it = blockIdx.x; it < n; it += gridDim.x) {
-            const int t = a.weno_tiles[it];
-            const int bx = t % a.tiles[0], byz = t / a.tiles[0];
-            vjp_tile<T, DIM, DIR, 1>(a, bx, byz % a.tiles[1], byz / a.tiles[1], smem_raw);
-            __syncthreads();   // shared memory is reused by the next tile
+    const unsigned int lines = vjp_tile<T, DIM, DIR>(a, blockIdx.x, blockIdx.y, blockIdx.z, smem_raw);
+    if (lines != 0u && threadIdx.x == 0)
+        a.weno_tiles[atomicAdd(a.n_weno_tiles, 1)] =
+            make_int2(blockIdx.x + a.tiles[0] * (blockIdx.y + a.tiles[1] * blockIdx.z), (int)lines);
+}
+
+// Shared memory of pass 1: one line of a tile.
+template <typename T, int DIM, int DIR>
+struct VjpWenoSmem {
+    static constexpr int SEG = VjpTile<T, DIM, DIR>::SEG;
+    static constexpr int NF = SEG + 5, NC = SEG + 10;
+    static constexpr int NV = DIM + 2, NQ = CellLayout<DIM>::NQ, NX = 4;   // record, then 1/sqrt(rho), 1/c, p, c
+    static constexpr int QC = 12;             // WENO faces per chunk
+    static constexpr int NUF = 2 * NV, NRB = DIM + 2;
+    // face data: Roe state, detector difference and its projection, flux
+    // cotangent and its projection, splitting speeds
+    static constexpr int U = 0, C = DIM, IC = DIM + 1, H = DIM + 2, B1 = DIM + 3, HQ2 = DIM + 4, RT = DIM + 5,
+                         IRT2 = DIM + 6, DU = DIM + 7, W = DU + NV, PHI = W + NV, WCB = PHI + NV, AL = WCB + NV,
+                         NFD = AL + 3;
+    // sums over a face: bars of u, 1/c, b1, |u|^2/2 and of the three speeds,
+    // then the bars of lambda^s and the reconstructed values of the fields
+    static constexpr int NPB = DIM + 6, NFS = NPB + 2 * NV;
+    static constexpr size_t cells = (size_t)NC * (NQ + NX + NV);
+    static constexpr size_t faces = (size_t)NF * (6 * NUF + NFD + NFS + NV + 2 * NRB + 3);
+    static constexpr size_t chunk = (size_t)QC * (NV * 2 * 6 + NV * 2 * 2 + 6 * NPB);
+    static constexpr size_t bytes = sizeof(T) * (cells + faces + chunk) + sizeof(int) * 2 * (size_t)NF;
+};
+constexpr int kVjpWenoThreads = 128;
+
+// The WENO faces of one line of a tile: line l of tile (bx, by, bz).
+//
+// A face's reverse is about 3500 FP64 instructions.  With one thread per face
+// (255 registers and spills) a tile's dozen WENO faces filled a dozen lanes
+// of two warps; here one lane takes a (face, cell) of the projections and
+// their adjoints and a (face, field, sign) of the reconstruction's, in chunks
+// of QC queued faces, and one lane per face the rest.  Ragged 121x97x113 box
+// in FP64 with a slab across z: pass 1 of the z direction 11.76 -> 2.84 ms.
+template <typename T, int DIM, int DIR>
+__device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, int bz, int l, unsigned char* smem_raw)
+{
+    using CL = CellLayout<DIM>;
+    using PL = PrimLayout<DIM>;
+    using SM = VjpWenoSmem<T, DIM, DIR>;
+    constexpr int NV = SM::NV, NQ = SM::NQ, NX = SM::NX, SEG = SM::SEG, NF = SM::NF, NC = SM::NC;
+    constexpr int QC = SM::QC, NUF = SM::NUF, NRB = SM::NRB, NFD = SM::NFD, NFS = SM::NFS, NPB = SM::NPB;
+    constexpr int NT = kVjpWenoThreads, LINES = VjpTile<T, DIM, DIR>::LINES, LAST = NV - 1;
+    T* cq = reinterpret_cast<T*>(smem_raw);   // [NQ + NX][NC]
+    T* wq = cq + (NQ + NX) * NC;              // [NV][NC] cotangent
+    T* UF = wq + NV * NC;                     // [NF][6][NUF] projections of U and F, then their bars
+    T* FD = UF + NF * 6 * NUF;                // [NF][NFD]
+    T* FS = FD + NF * NFD;                    // [NF][NFS]
+    T* DB = FS + NF * NFS;                    // [NF][NV] bars of the detector difference
+    T* RB = DB + NF * NV;                     // [NF][2][NRB] Roe-field bars of cells 2 and 3
+    T* SP = RB + NF * 2 * NRB;                // [NF][3] speed bars
+    T* XB = SP + NF * 3;                      // [QC][NV][2][6] bars of f+-
+    T* LF = XB + QC * NV * 2 * 6;             // [QC][NV][2][2] bar of lambda^s, reconstructed value
+    T* PB = LF + QC * NV * 2 * 2;             // [QC][6][NPB] per-cell parts of the face sums
+    int* SL = reinterpret_cast<int*>(PB + QC * 6 * NPB);   // [NF] slots attaining the speeds
+    int* queue = SL + NF;
+    __shared__ int qcount;
+    constexpr int SKIP = 1 << 12;
+
+    const int nd = a.n[DIR], c0 = bx * SEG;
+    int ix = 0, j = 0, k = 0;
+    if (DIR == 0) { j = by; k = bz; }
+    else if (DIR == 1) { ix = by * LINES + l; k = bz; }
+    else { ix = by * LINES + l; j = bz; }
+    const long long sd = DIR == 0 ? 1LL : (DIR == 1 ? a.sy : a.sz);
+    const long long base = a.off0 + (long long)ix + (long long)j * a.sy + (long long)k * a.sz;
+    const int line = DIR == 0 ? j : ix;   // in-plane index for the boundary conditions
+    const T* Ug = reinterpret_cast<const T*>(a.U);
+    const T* Wg = reinterpret_cast<const T*>(a.W);
+    const T gamma = T(a.gamma), gm1 = gamma - T(1);
+    if (threadIdx.x == 0) qcount = 0;
+
+    // ---- cells c0 - 5 .. c0 + SEG + 4 that exist
+    for (int p = threadIdx.x; p < NC; p += NT) {
+        const int cell = c0 - 5 + p;
+        const bool inside = cell >= 0 && cell < nd;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) wq[v * NC + p] = inside ? Wg[base + (long long)cell * sd + v * a.sv] : T(0);
+        if (cell >= -3 && cell <= nd + 2) {
+            T U[NV], q[NQ], inv[2], P[PL::NP];
+            stage_cell<T, DIM, DIR>(a.bc, Ug, base, line, cell, nd, U);
+            cell_prims<T, DIM>(U, gamma, gm1, P, inv);
+            cell_record<T, DIM, DIR>(U, P, q);
+#pragma unroll
+            for (int kk = 0; kk < NQ; ++kk) cq[kk * NC + p] = q[kk];
+            cq[NQ * NC + p] = inv[0];
+            cq[(NQ + 1) * NC + p] = inv[1];
+            cq[(NQ + 2) * NC + p] = P[PL::P];
+            cq[(NQ + 3) * NC + p] = P[PL::C];
         }
+    }
+    __syncthreads();
+
+    // ---- WENO faces: the forward quantities of the whole face
+    const T lam_k = T(a.c_lambda / 3600.0), eps = T(a.eps), inv_dx = T(a.inv_dx), slim = T(a.slim);
+    for (int f = threadIdx.x; f < NF; f += NT) {
+        const int face = c0 - 2 + f;
+        SL[f] = SKIP;
+        if (face < 0 || face > nd) continue;
+        auto rec = [&](int m, int kk) -> T { return cq[kk * NC + f + m]; };
+        auto ga = [&](int kk) -> T { return rec(2, kk); };
+        auto gb = [&](int kk) -> T { return rec(3, kk); };
+        const Roe<T, DIM> r = roe_state<T, DIM>(ga, gb, gm1);
+        T dU[NV], w[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const int kk = CL::U + v;
+            dU[v] = fmaT(T(10), rec(2, kk) - rec(3, kk), fmaT(T(5), rec(4, kk) - rec(1, kk), rec(0, kk) - rec(5, kk)));
+        }
+        proj_all<T, DIM, DIR>(r, dU, w);
+        const T lim = slim * r.rt;
+        bool smooth = a.hybrid != 0;
+#pragma unroll
+        for (int s = 0; s < NV; ++s) smooth = smooth && abs_lt(w[s], lim);
+        if (smooth) continue;   // pass 0 took this face
+        T am = rec(0, CL::LM), a0 = rec(0, CL::L0), ap = rec(0, CL::LP);
+        int im = 0, i0 = 0, ip = 0;
+#pragma unroll
+        for (int m = 1; m < 6; ++m) {
+            const T xm = rec(m, CL::LM), x0 = rec(m, CL::L0), xp = rec(m, CL::LP);
+            if (lt_nn(am, xm)) { am = xm; im = m; }
+            if (lt_nn(a0, x0)) { a0 = x0; i0 = m; }
+            if (lt_nn(ap, xp)) { ap = xp; ip = m; }
+        }
+        SL[f] = im | (i0 << 4) | (ip << 8);
+        T* fd = FD + f * NFD;
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) fd[SM::U + kk] = r.u[kk];
+        fd[SM::C] = r.c; fd[SM::IC] = r.ic; fd[SM::H] = r.H; fd[SM::B1] = r.b1; fd[SM::HQ2] = r.hq2; fd[SM::RT] = r.rt;
+        fd[SM::IRT2] = T(1) / (r.rt * r.rt);
+        fd[SM::AL] = am; fd[SM::AL + 1] = a0; fd[SM::AL + 2] = ap;
+        // cotangent of the face flux, (w_right - w_left) / dx, and R^T of it
+        T phi[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            phi[v] = (wq[v * NC + f + 3] - wq[v * NC + f + 2]) * inv_dx;
+            fd[SM::PHI + v] = phi[v];
+            fd[SM::DU + v] = dU[v];
+            fd[SM::W + v] = w[v];
+        }
+        T sumb = phi[0];
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) sumb = fmaT(phi[1 + kk], r.u[kk], sumb);
+        const T difb = fmaT(phi[LAST], r.u[DIR], phi[1 + DIR]) * r.c, eh = fmaT(phi[LAST], r.H, sumb);
+        fd[SM::WCB] = eh - difb;
+        fd[SM::WCB + 1] = fmaT(phi[LAST], r.hq2, sumb);
+        int s = 2;
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) {
+            if (kk == DIR) continue;
+            fd[SM::WCB + s] = fmaT(phi[LAST], r.u[kk], phi[1 + kk]);
+            ++s;
+        }
+        fd[SM::WCB + LAST] = eh + difb;
+        queue[atomicAdd(&qcount, 1)] = f;
+    }
+    __syncthreads();
+
+    const int nq = qcount;
+    auto load_roe = [&](const T* fd, Roe<T, DIM>& r) {
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) r.u[kk] = fd[SM::U + kk];
+        r.c = fd[SM::C]; r.ic = fd[SM::IC]; r.H = fd[SM::H]; r.b1 = fd[SM::B1]; r.hq2 = fd[SM::HQ2]; r.rt = fd[SM::RT];
+    };
+    for (int q0 = 0; q0 < nq; q0 += QC) {
+        const int qc = nq - q0 < QC ? nq - q0 : QC;
+        // projections of U_m and F_m (Eq. eqchara)
+        for (int it = threadIdx.x; it < qc * 6; it += NT) {
+            const int f = queue[q0 + it / 6], m = it % 6;
+            Roe<T, DIM> r;
+            load_roe(FD + f * NFD, r);
+            T xu[NV], xf[NV], vv[NV], gg[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) { xu[v] = cq[(CL::U + v) * NC + f + m]; xf[v] = cq[(CL::F + v) * NC + f + m]; }
+            proj_all<T, DIM, DIR>(r, xu, vv);
+            proj_all<T, DIM, DIR>(r, xf, gg);
+            T* uf = UF + (f * 6 + m) * NUF;
+#pragma unroll
+            for (int s = 0; s < NV; ++s) { uf[s] = vv[s]; uf[NV + s] = gg[s]; }
+        }
+        __syncthreads();
+        // reconstructions and their reverse; the minus part on the mirrored
+        // stencil m = 5 .. 1
+        for (int it = threadIdx.x; it < qc * NV * 2; it += NT) {
+            const int q = it / (2 * NV), rem = it - q * 2 * NV, s = rem >> 1, sg = rem & 1;
+            const int f = queue[q0 + q];
+            const T* fd = FD + f * NFD;
+            const T al = fd[SM::AL + (s == 0 ? 0 : (s == LAST ? 2 : 1))];
+            const T ws = fd[SM::W + s], lam = lam_k * (ws * ws) * fd[SM::IRT2];
+            const T ha = sg ? T(-0.5) * al : T(0.5) * al;
+            T x[5], xb[5], lb;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) {
+                const T* uf = UF + (f * 6 + (sg ? 5 - i : i)) * NUF + s;
+                x[i] = fmaT(ha, uf[0], T(0.5) * uf[NV]);
+            }
+            const T val = recon_adj<T>(x[0], x[1], x[2], x[3], x[4], lam, eps, fd[SM::WCB + s], xb, lb);
+            T* o = XB + ((q * NV + s) * 2 + sg) * 6;
+#pragma unroll
+            for (int i = 0; i < 5; ++i) o[sg ? 5 - i : i] = xb[i];
+            o[sg ? 0 : 5] = T(0);
+            LF[((q * NV + s) * 2 + sg) * 2] = lb;
+            LF[((q * NV + s) * 2 + sg) * 2 + 1] = val;
+        }
+        __syncthreads();
+        // splitting and projections in reverse, per stencil cell
+        for (int it = threadIdx.x; it < qc * 6; it += NT) {
+            const int q = it / 6, m = it - q * 6, f = queue[q0 + q];
+            const T* fd = FD + f * NFD;
+            Roe<T, DIM> r;
+            load_roe(fd, r);
+            T* uf = UF + (f * 6 + m) * NUF;
+            T vb[NV], gb[NV], alb[3] = {T(0), T(0), T(0)};
+#pragma unroll
+            for (int s = 0; s < NV; ++s) {
+                const T fp = XB[((q * NV + s) * 2) * 6 + m], fm = XB[((q * NV + s) * 2 + 1) * 6 + m];
+                const int as = s == 0 ? 0 : (s == LAST ? 2 : 1);
+                const T d = T(0.5) * (fp - fm);
+                gb[s] = T(0.5) * (fp + fm);
+                vb[s] = fd[SM::AL + as] * d;
+                alb[as] = fmaT(uf[s], d, alb[as]);
+            }
+            RoeBar<T, DIM> rb;
+            zero(rb);
+            T x[NV], xb[NV];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                for (int v = 0; v < NV; ++v) { x[v] = cq[((h ? CL::F : CL::U) + v) * NC + f + m]; xb[v] = T(0); }
+                proj_all_adj<T, DIM, DIR>(r, x, h ? gb : vb, xb, rb);
+#pragma unroll
+                for (int v = 0; v < NV; ++v) uf[h * NV + v] = xb[v];
+            }
+            T* o = PB + it * NPB;
+#pragma unroll
+            for (int kk = 0; kk < DIM; ++kk) o[kk] = rb.u[kk];
+            o[DIM] = rb.ic; o[DIM + 1] = rb.b1; o[DIM + 2] = rb.hq2;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) o[DIM + 3 + i] = alb[i];
+        }
+        __syncthreads();
+        // sums over the cells and over the signs
+        for (int it = threadIdx.x; it < qc * NFS; it += NT) {
+            const int q = it / NFS, c = it - q * NFS;
+            T sum;
+            if (c < NPB) {
+                const T* o = PB + q * 6 * NPB + c;
+                sum = o[0];
+#pragma unroll
+                for (int m = 1; m < 6; ++m) sum += o[m * NPB];
+            } else {
+                const int s = (c - NPB) % NV, w = (c - NPB) / NV;
+                const T* o = LF + (q * NV + s) * 4 + w;
+                sum = o[0] + o[2];
+            }
+            FS[queue[q0 + q] * NFS + c] = sum;
+        }
+    }
+    __syncthreads();
+
+    // ---- per face: weights' parameter, detector, back-projection and Roe average in reverse
+    for (int q = threadIdx.x; q < nq; q += NT) {
+        const int f = queue[q];
+        const T *fd = FD + f * NFD, *fs = FS + f * NFS, *lb = fs + NPB, *wch = lb + NV;
+        Roe<T, DIM> r;
+        load_roe(fd, r);
+        RoeBar<T, DIM> rb;
+        zero(rb);
+        const T sum = wch[0] + wch[1] + wch[LAST], dif = wch[LAST] - wch[0], oE = fd[SM::PHI + LAST];
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) rb.u[kk] = fmaT(fd[SM::PHI + 1 + kk], sum, fs[kk]);
+        rb.c = fmaT(oE, r.u[DIR], fd[SM::PHI + 1 + DIR]) * dif;
+        rb.u[DIR] = fmaT(oE * r.c, dif, rb.u[DIR]);
+        int s = 2;
+#pragma unroll
+        for (int kk = 0; kk < DIM; ++kk) {
+            if (kk == DIR) continue;
+            rb.u[kk] = fmaT(oE, wch[s], rb.u[kk]);
+            ++s;
+        }
+        rb.H = oE * (wch[0] + wch[LAST]);
+        rb.ic = fs[DIM];
+        rb.b1 = fs[DIM + 1];
+        rb.hq2 = fmaT(oE, wch[1], fs[DIM + 2]);
+        // lam = c w^2 / (3600 rt^2)
+        const T irt2 = fd[SM::IRT2], irt = irt2 * r.rt;
+        T wb[NV], dUb[NV], dU[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const T w = fd[SM::W + v], lw = lam_k * w * irt2;
+            wb[v] = lb[v] * (lw + lw);
+            rb.rt = fmaT(lb[v], T(-2) * (lw * w) * irt, rb.rt);
+            dU[v] = fd[SM::DU + v];
+            dUb[v] = T(0);
+        }
+        proj_all_adj<T, DIM, DIR>(r, dU, wb, dUb, rb);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) DB[f * NV + v] = dUb[v];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) SP[f * 3 + i] = fs[DIM + 3 + i];
+        T* RBf = RB + f * 2 * NRB;
+        T ra[NRB], rbb[NRB];
+#pragma unroll
+        for (int kk = 0; kk < NRB; ++kk) ra[kk] = rbb[kk] = T(0);
+        roe_adj<T, DIM>([&](int kk) -> T { return cq[kk * NC + f + 2]; }, [&](int kk) -> T { return cq[kk * NC + f + 3]; },
+                        gamma, r, rb, ra, rbb);
+#pragma unroll
+        for (int kk = 0; kk < NRB; ++kk) { RBf[kk] = ra[kk]; RBf[NRB + kk] = rbb[kk]; }
+    }
+    __syncthreads();
+
+    // ---- gather per cell, as in pass 0
+    T* Gg = reinterpret_cast<T*>(a.G);
+    T* ghost = reinterpret_cast<T*>(a.ghost);
+    const bool first = c0 == 0, last = c0 + SEG >= nd;
+    for (int p = threadIdx.x; p < SEG + 6; p += NT) {
+        const int cell = c0 - 3 + p;
+        const bool owned = cell >= c0 && cell < c0 + SEG && cell < nd;
+        const bool gl = first && cell < 0 && cell >= -3;
+        const bool gr = last && cell >= nd && cell <= nd + 2;
+        if (!owned && !gl && !gr) continue;
+        T qb[NQ];
+#pragma unroll
+        for (int kk = 0; kk < NQ; ++kk) qb[kk] = T(0);
+        bool touched = false;
+        constexpr T cd[6] = {T(1), T(-5), T(10), T(-10), T(5), T(-1)};
+#pragma unroll
+        for (int m = 5; m >= 0; --m) {
+            const int f = cell - m + 3 - (c0 - 2);   // faces in increasing order
+            if (f < 0 || f >= NF) continue;
+            const int sl = SL[f];
+            if (sl & SKIP) continue;
+            touched = true;
+            const T* uf = UF + (f * 6 + m) * NUF;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) {
+                qb[CL::U + v] += fmaT(cd[m], DB[f * NV + v], uf[v]);
+                qb[CL::F + v] += uf[NV + v];
+            }
+            if (m == 2 || m == 3) {
+                const T* rbp = RB + (f * 2 + (m - 2)) * NRB;
+#pragma unroll
+                for (int kk = 0; kk < NRB; ++kk) qb[CL::SU + kk] += rbp[kk];
+            }
+            if ((sl & 15) == m) qb[CL::LM] += SP[f * 3 + 0];
+            if (((sl >> 4) & 15) == m) qb[CL::L0] += SP[f * 3 + 1];
+            if (((sl >> 8) & 15) == m) qb[CL::LP] += SP[f * 3 + 2];
+        }
+        if (!touched) continue;
+        const int pc = cell - (c0 - 5);
+        T U[NV], Ub[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) U[v] = cq[(CL::U + v) * NC + pc];
+        cell_adj<T, DIM, DIR>(U, gamma, cq[NQ * NC + pc], cq[(NQ + 1) * NC + pc], cq[(NQ + 2) * NC + pc],
+                              cq[(NQ + 3) * NC + pc], qb, Ub);
+        if (owned) {
+            const long long g = base + (long long)cell * sd;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) Gg[g + v * a.sv] += Ub[v];
+        } else {
+            const long long ln = DIR == 0 ? ((long long)k * a.n[1] + j)
+                                          : (DIR == 1 ? ((long long)k * a.n[0] + ix) : ((long long)j * a.n[0] + ix));
+            const int slot = gl ? (-cell - 1) : (3 + cell - nd);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) ghost[(ln * 6 + slot) * NV + v] += Ub[v];
+        }
+    }
+    __syncthreads();   // shared memory is reused by the next line
+}
+
+// Pass 1: a grid of resident CTAs takes the listed tiles in turn (each line
+// writes only its own cells and ghost slots, so the order in which they are
+// taken does not change the result).
+template <typename T, int DIM, int DIR>
+__global__ void __launch_bounds__(kVjpWenoThreads) k_vjp_weno(VjpArgs a)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int LINES = VjpTile<T, DIM, DIR>::LINES;
+    const long long n = (long long)*a.n_weno_tiles * LINES;
+    for (long long it = blockIdx.x; it < n; it += gridDim.x) {
+        const int2 t = a.weno_tiles[it / LINES];
+        const int l = (int)(it % LINES);
+        if (!((t.y >> l) & 1)) continue;
+        const int bx = t.x % a.tiles[0], byz = t.x / a.tiles[0];
+        vjp_weno_line<T, DIM, DIR>(a, bx, byz % a.tiles[1], byz / a.tiles[1], l, smem_raw);
     }
 }
 

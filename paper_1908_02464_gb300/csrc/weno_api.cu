@@ -51,7 +51,8 @@ struct weno_ctx {
     void* stage_io = nullptr;   // interior-size staging for host copies
     void* vjp_w = nullptr;      // ghosted cotangent (ghost layers stay zero)
     void* vjp_ghost = nullptr;  // per-line ghost-cell gradients
-    int* vjp_tiles = nullptr;   // per direction: count (entries 0..2), then lists of tiles with WENO faces
+    int* vjp_tiles = nullptr;   // per direction: count (entries 0..2), then lists of tiles with WENO faces (two
+                                // ints each)
     long long vjp_tiles_max = 0;
     unsigned long long* alpha_g = nullptr;   // global LF speeds [stage 0..3][dir][3]
     DevTime* tm = nullptr;
@@ -742,7 +743,7 @@ weno_status weno_rhs_vjp(weno_ctx* ctx, const void* U_dev, const void* w_dev, vo
             ctx->err = "grid too large for the adjoint's tile lists";
             return WENO_ERR_INVALID_ARG;
         }
-        CK(cudaMalloc(&ctx->vjp_tiles, (size_t)(4 + 3 * tiles) * sizeof(int)));
+        CK(cudaMalloc(&ctx->vjp_tiles, (size_t)(4 + 6 * tiles) * sizeof(int)));
         ctx->vjp_tiles_max = tiles;
     }
     CK(cudaMemsetAsync(ctx->vjp_tiles, 0, 3 * sizeof(int), ctx->stream));
@@ -759,7 +760,7 @@ weno_status weno_rhs_vjp(weno_ctx* ctx, const void* U_dev, const void* w_dev, vo
         a.G = gU_dev;
         a.ghost = ctx->vjp_ghost;
         a.n_weno_tiles = ctx->vjp_tiles + d;
-        a.weno_tiles = ctx->vjp_tiles + 4 + d * ctx->vjp_tiles_max;
+        a.weno_tiles = reinterpret_cast<int2*>(ctx->vjp_tiles + 4) + d * ctx->vjp_tiles_max;
         a.accumulate = d > 0;
         for (int k = 0; k < 3; ++k) a.n[k] = ctx->n[k];
         a.sy = sy; a.sz = sz; a.sv = sv; a.off0 = 0;

@@ -184,45 +184,41 @@ dim3 vjp_grid(const int* n)
     return dim3((n[DIR] + TL::SEG - 1) / TL::SEG, e0, e1);
 }
 
-template <typename T, int DIM, int DIR, int PASS>
-cudaError_t launch_vjp_pass(const VjpArgs& a, cudaStream_t s)
+// pass 0 (linear-upwind faces, lists the tiles with WENO faces), then pass 1
+// (the WENO faces of the listed lines)
+template <typename T, int DIM, int DIR>
+cudaError_t launch_vjp_one(const VjpArgs& a, cudaStream_t s)
 {
-    using SM = VjpSmem<T, DIM, DIR, PASS>;
+    using S0 = VjpSmem<T, DIM, DIR>;
+    using S1 = VjpWenoSmem<T, DIM, DIR>;
     constexpr int NT = VjpTile<T, DIM, DIR>::NT;
-    auto kern = k_vjp<T, DIM, DIR, PASS>;
-    static int resident = 0;   // CTAs per SM (pass 1 grid)
+    auto k0 = k_vjp<T, DIM, DIR>;
+    auto k1 = k_vjp_weno<T, DIM, DIR>;
+    static int resident = 0;   // CTAs per SM of pass 1
     if (resident == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
+        int fit = 0;
+        cudaError_t e = cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S0::bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S1::bytes);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k1, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, k1, kVjpWenoThreads, S1::bytes);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kern, NT, SM::bytes);
-        if (e != cudaSuccess) return e;
-        if (resident < 1) resident = 1;
+        resident = fit < 1 ? 1 : fit;
     }
     const dim3 g = vjp_grid<T, DIM, DIR>(a.n);
     VjpArgs b = a;
     b.tiles[0] = (int)g.x; b.tiles[1] = (int)g.y; b.tiles[2] = (int)g.z;
-    if (PASS == 0) {
-        kern<<<g, NT, SM::bytes, s>>>(b);
-    } else {
-        int dev = 0, nsm = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        const long long tiles = (long long)g.x * g.y * g.z;
-        const long long blocks = (long long)resident * nsm < tiles ? (long long)resident * nsm : tiles;
-        kern<<<(unsigned)(blocks > 0 ? blocks : 1), NT, SM::bytes, s>>>(b);
-    }
-    return cudaGetLastError();
-}
-
-// pass 0 (linear-upwind faces, lists the tiles with WENO faces), then pass 1
-// (the WENO faces of the listed tiles)
-template <typename T, int DIM, int DIR>
-cudaError_t launch_vjp_one(const VjpArgs& a, cudaStream_t s)
-{
-    cudaError_t e = launch_vjp_pass<T, DIM, DIR, 0>(a, s);
+    k0<<<g, NT, S0::bytes, s>>>(b);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    return launch_vjp_pass<T, DIM, DIR, 1>(a, s);
+    int dev = 0, nsm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long long lines = (long long)g.x * g.y * g.z * VjpTile<T, DIM, DIR>::LINES;
+    const long long blocks = (long long)resident * nsm < lines ? (long long)resident * nsm : lines;
+    k1<<<(unsigned)(blocks > 0 ? blocks : 1), kVjpWenoThreads, S1::bytes, s>>>(b);
+    return cudaGetLastError();
 }
 
 template <typename T>
