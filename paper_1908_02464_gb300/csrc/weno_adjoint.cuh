@@ -284,6 +284,11 @@ struct VjpArgs {
     long long sy, sz, sv, off0;
     double inv_dx, eps_h, gamma, eps, c_lambda;
     double slim;   // 60 sqrt(eps_h), as in the forward sweep
+    double lam_k;  // c_lambda / 3600
+    // the same pre-rounded for float kernels: a conversion or a division per
+    // thread would run on the slow FP64 pipe (38% of the cycles of the float
+    // x pass)
+    float inv_dx_f, gamma_f, eps_f, slim_f, lam_k_f;
     int hybrid;
     // boundary conditions of this direction, for the ghost cells computed
     // while staging (the fields stage_cell reads: bc_lo, bc_hi, bc_state,
@@ -364,7 +369,10 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
     const long long base0 = a.off0 + (long long)ix0 + (long long)j * a.sy + (long long)k * a.sz;
     const T* Ug = reinterpret_cast<const T*>(a.U);
     const T* Wg = reinterpret_cast<const T*>(a.W);
-    const T gamma = T(a.gamma);
+    const T gamma = pick<T>(a.gamma, a.gamma_f);
+
+    __shared__ unsigned int weno_lines;
+    if (threadIdx.x == 0) weno_lines = 0u;
 
     // stage cells c0-5 .. c0+SEG+4 that exist (-3 .. nd+2); ghost cells come
     // from the boundary conditions, and the cotangent is zero on them
@@ -376,7 +384,11 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
             // for x sweeps, the column for y and z sweeps
             const int line = DIR == 0 ? j : ix0 + l;
             using PL = PrimLayout<DIM>;
-            T U[NV], q[NQ], inv[2], P[PL::NP];
+            T U[NV], q[NQ], inv[2], P[PL::NP], W[NV];
+            const bool inside = cell >= 0 && cell < nd;
+            const long long g = base0 + l + (long long)cell * sd;
+#pragma unroll
+            for (int v = 0; v < NV; ++v) W[v] = inside ? Wg[g + v * a.sv] : T(0);
             if constexpr (sizeof(T) == 8) {
                 long long gs = 0;
                 bool flip = false;
@@ -411,10 +423,8 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
                 stage_cell<T, DIM, DIR>(a.bc, Ug, base0 + l, line, cell, nd, U);
                 cell_prims<T, DIM>(U, gamma, gamma - T(1), P, inv);
             }
-            const bool inside = cell >= 0 && cell < nd;
-            const long long g = base0 + l + (long long)cell * sd;
 #pragma unroll
-            for (int v = 0; v < NV; ++v) wq[v * LNC + idx] = inside ? Wg[g + v * a.sv] : T(0);
+            for (int v = 0; v < NV; ++v) wq[v * LNC + idx] = W[v];
             cell_record<T, DIM, DIR>(U, P, q);
 #pragma unroll
             for (int kk = 0; kk < NQ; ++kk) cq[kk * LNC + idx] = q[kk];
@@ -432,12 +442,20 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
     __syncthreads();
 
     // ---- per face: forward recompute and reverse -------------------------
-    const T slim = T(a.slim);
-    const T lam_k = T(a.c_lambda / 3600.0);
-    const T eps = T(a.eps), inv_dx = T(a.inv_dx);
-    __shared__ unsigned int weno_lines;
-    if (threadIdx.x == 0) weno_lines = 0u;
-    __syncthreads();
+    const T slim = pick<T>(a.slim, a.slim_f), inv_dx = pick<T>(a.inv_dx, a.inv_dx_f);
+    // Float: the gradient of earlier directions is loaded before the faces,
+    // for the first cell that this thread gathers
+    constexpr bool EARLY = sizeof(T) == 4;
+    T eg[NV];
+    if constexpr (EARLY) {
+        const int p = threadIdx.x / LINES, l = threadIdx.x - (threadIdx.x / LINES) * LINES;
+        const int cell = c0 - 3 + p;
+        const bool read = a.accumulate && l < nlx && cell >= c0 && cell < c0 + SEG && cell < nd;
+        const T* Gr = reinterpret_cast<const T*>(a.G) + base0 + l + (long long)cell * sd;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) eg[v] = read ? Gr[v * a.sv] : T(0);
+    }
+
     for (int ff = threadIdx.x; ff < LNF; ff += NT) {
         const int f = ff / LINES, l = ff - (ff / LINES) * LINES;
         const int face = c0 - 2 + f;            // face i' between cells i'-1 and i'
@@ -642,8 +660,9 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
             const long long g = base0 + l + (long long)cell * sd;
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                if (a.accumulate) Gg[g + v * a.sv] += Ub[v];
-                else Gg[g + v * a.sv] = Ub[v];
+                if (!a.accumulate) Gg[g + v * a.sv] = Ub[v];
+                else if (EARLY && idx == (int)threadIdx.x) Gg[g + v * a.sv] = eg[v] + Ub[v];
+                else Gg[g + v * a.sv] += Ub[v];
             }
         } else {
             const long long i = ix0 + l;
@@ -737,7 +756,7 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
     const int line = DIR == 0 ? j : ix;   // in-plane index for the boundary conditions
     const T* Ug = reinterpret_cast<const T*>(a.U);
     const T* Wg = reinterpret_cast<const T*>(a.W);
-    const T gamma = T(a.gamma), gm1 = gamma - T(1);
+    const T gamma = pick<T>(a.gamma, a.gamma_f), gm1 = gamma - T(1);
     if (threadIdx.x == 0) qcount = 0;
 
     // ---- cells c0 - 5 .. c0 + SEG + 4 that exist
@@ -762,7 +781,8 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
     __syncthreads();
 
     // ---- WENO faces: the forward quantities of the whole face
-    const T lam_k = T(a.c_lambda / 3600.0), eps = T(a.eps), inv_dx = T(a.inv_dx), slim = T(a.slim);
+    const T lam_k = pick<T>(a.lam_k, a.lam_k_f), eps = pick<T>(a.eps, a.eps_f);
+    const T inv_dx = pick<T>(a.inv_dx, a.inv_dx_f), slim = pick<T>(a.slim, a.slim_f);
     for (int f = threadIdx.x; f < NF; f += NT) {
         const int face = c0 - 2 + f;
         SL[f] = SKIP;

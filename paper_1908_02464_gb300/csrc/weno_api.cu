@@ -314,6 +314,37 @@ static weno_status read_time(weno_ctx* ctx)
     return WENO_OK;
 }
 
+// Default tile of direction d (variants of weno_launch.cuh; the times are
+// sweeps on one GB300, us).
+static int default_tile(const weno_ctx* c, int d)
+{
+    const int n = c->n[d];
+    const bool f64 = c->prec == WENO_FP64;
+    // lines shorter than a flat tile: the shape with the fewest tiles per
+    // line, between 1 x 127, 4 x 31 and (FP32) 2 x 63
+    auto per_line = [&](int seg, int lines) { return (double)((n + seg - 1) / seg) / lines; };
+    if (!f64) {
+        if (d > 0) return 1;   // 8 x 15: coalesced rows
+        // Along x the last tile of a line may be nearly empty (256 cells in
+        // 1 x 127 tiles: a third of the work on 2 cells).  1 x 127, or 1 x 95
+        // where that fills better (256^3 x-sweep 486 -> 390), or flat tiles
+        // (128^3: 79 -> 57), or several short lines (55 cells: 13.3 -> 11.3)
+        const double e3 = n / (127.0 * ((n + 126) / 127)), e4 = n / (95.0 * ((n + 94) / 95));
+        if (e3 >= 0.85 && e3 >= e4 - 0.05) return 3;
+        if (e4 >= 0.85) return 4;
+        if (n >= wis::Tile<5>::SEG) return 5;
+        return per_line(31, 4) < per_line(127, 1) ? 2 : 3;
+    }
+    if (d == 0) return n >= wis::Tile<5>::SEG || per_line(31, 4) >= per_line(127, 1) ? 5 : 2;
+    // Across x, 4 x 31: four x-adjacent lines share the 32-byte sectors of the
+    // strided loads (256^3: y 3524 -> 3130, z 4046 -> 3933; 637 x 159: y 46.6
+    // -> 39.1).  A 2D grid with fewer such tiles than the chip holds CTAs is
+    // bound by the time of one tile, which is shorter for the flat ones
+    // (512 x 128: 39.1 against 44.8, 177 x 70: 23 against 34).
+    const long long tiles = (long long)((c->n[0] + 3) / 4) * ((n + 30) / 31) * (c->dim == 3 ? c->n[3 - d] : 1);
+    return tiles > 5LL * c->nsm ? 2 : 5;
+}
+
 // ----------------------------------------------------------- ABI
 extern "C" {
 
@@ -494,18 +525,11 @@ weno_status weno_create(const weno_grid* grid, const weno_params* params, void* 
         return WENO_ERR_CUDA;
     }
     std::memset(ctx->tm_host, 0, sizeof(DevTime));
-    // default tiles, measured on the 2048 x 512 double Mach reflection: FP64 flat
-    // 128-face tiles (ALU bound, every lane busy), FP32 1 x 127 along x and
-    // 8 x 15 across (coalesced rows); weno_autotune refines them per state
-    // FP64: flat tiles, except along y in 3D, where 4 x-adjacent lines per
-    // tile share the 32-byte sectors of the strided loads (256^3 RHS 18.4
-    // -> 17.3 ms); FP32 and mixed: 1 x 127 along x, 8 x 15 across, and the
-    // marching sweep (variant 7) across x when its lanes (lines x segments)
-    // fill at least four rounds of 16 warps per SM: on the 256^3
-    // vortex it runs the RHS in 1.72 ms against 2.07, on the 2048 x 512
+    for (int d = 0; d < dim; ++d) ctx->tile[d] = default_tile(ctx, d);
+    // FP32 and mixed: the marching sweep (variant 7) across x when its lanes
+    // (lines x segments) fill at least four rounds of 16 warps per SM: on the
+    // 256^3 vortex it runs the RHS in 1.72 ms against 2.07, on the 2048 x 512
     // double Mach reflection (0.3 rounds) its y-sweep takes 3x the tiles' time
-    for (int d = 0; d < dim; ++d)
-        ctx->tile[d] = ctx->prec == WENO_FP64 ? (dim == 3 && d == 1 ? 2 : 5) : (d == 0 ? 3 : 1);
     if (ctx->prec != WENO_FP64) {
         for (int d = 1; d < dim; ++d) {
             const long long lines = (long long)ctx->n[0] * (d == 1 ? ctx->n[2] : ctx->n[1]);
@@ -768,6 +792,9 @@ weno_status weno_rhs_vjp(weno_ctx* ctx, const void* U_dev, const void* w_dev, vo
         a.eps_h = ctx->eps_h[d];
         a.slim = std::sqrt(3600.0 * a.eps_h);
         a.gamma = ctx->p.gamma; a.eps = ctx->p.eps; a.c_lambda = ctx->p.c_lambda; a.hybrid = ctx->p.hybrid;
+        a.lam_k = a.c_lambda / 3600.0;
+        a.inv_dx_f = (float)a.inv_dx; a.gamma_f = (float)a.gamma; a.eps_f = (float)a.eps; a.slim_f = (float)a.slim;
+        a.lam_k_f = (float)a.lam_k;
         a.bc = sweep_args(ctx, d);
         a.bc.sy = sy; a.bc.sz = sz; a.bc.sv = sv; a.bc.off0 = 0;
         a.bc.tm = nullptr;

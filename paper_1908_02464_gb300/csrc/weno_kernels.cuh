@@ -62,6 +62,8 @@ struct DevTime {
     long long steps;                // completed steps
     int status;                     // 0 ok, else WENO_ERR_NONPHYSICAL latched
     int clipped;                    // 1 if dt was clipped to reach t_end
+    int go;                         // dt > 0 (float kernels keep off the FP64 pipe)
+    float dt_f;
     double xs_top[3];               // double Mach top boundary: shock position at the
                                     // stage times t, t + dt, t + dt/2
 };
@@ -585,6 +587,56 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     }
     __syncthreads();
 
+    // the output cell of this thread: its global index, its left face, its
+    // right face and the start of the left face's stencil
+    static_assert(LINES * SEG <= NT, "one output cell per thread");
+    auto out_cell = [&](long long& g, int& l, int& fl, int& fr_, int& cpos) -> bool {
+        const int idx = threadIdx.x;
+        if (idx >= LINES * SEG) return false;
+        int p;
+        if (DIR == 0) { l = idx / SEG; p = idx - l * SEG; }
+        else { p = idx / LINES; l = idx - p * LINES; }
+        if constexpr (FLAT) {
+            // the cell between faces idx and idx + 1 of the same piece
+            const bool inA = idx + 1 < nA;
+            if (!inA && (idx < nA || idx + 1 >= nA + nB)) return false;   // line junction or past the end
+            int inplane;
+            g = flat_line(inA ? LA : LA + 1, inplane) + (long long)(inA ? fA0 + idx : idx - nA) * sd;
+            fl = idx;
+            fr_ = idx + 1;
+            cpos = inA ? idx : idx + 5;
+        } else {
+            const int line = line0 + l;
+            const int cell = c0 + p;
+            if (line >= nline || cell >= nd) return false;
+            g = a.off0 + (long long)line * sl + (long long)pb * sp + (long long)cell * sd;
+            fl = DIR == 0 ? l * FACES + p : p * LINES + l;
+            fr_ = DIR == 0 ? fl + 1 : fl + LINES;
+            cpos = p;
+        }
+        return true;
+    };
+    const T rka = pick<T>(a.rk_a, a.rk_a_f), rkb = pick<T>(a.rk_b, a.rk_b_f);
+    // Float: the accumulator and the base state of the output cell are loaded
+    // before the faces; a tile waited for them at its end (10 of 17 stalled
+    // cycles per issue in the accumulating 160^3 y-sweep, which took 186 us
+    // against 115 us without the accumulator; 10 steps of the 2048 x 512 grid
+    // 2.06 -> 2.02 ms).  FP64 tiles, bound by their pipe, keep the registers.
+    constexpr bool EARLY = sizeof(T) == 4;
+    T ea[NV], en[NV];
+    if constexpr (EARLY) {
+        long long g = 0;
+        int l = 0, fl = 0, fr_ = 0, cpos = 0;
+        const bool read = a.mode != MODE_ACC_SET && out_cell(g, l, fl, fr_, cpos);
+        const T* accr = reinterpret_cast<const T*>(a.acc);
+        const T* Unr = reinterpret_cast<const T*>(a.Un);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            ea[v] = read && accr != nullptr ? accr[g + v * a.sv] : T(0);
+            en[v] = read && a.mode == MODE_COMBINE && rka != T(0) ? Unr[g + v * a.sv] : T(0);
+        }
+    }
+
     // shared-memory order follows the global order: along-the-line for x
     // sweeps, across the lines (x fastest) for y/z sweeps; consecutive
     // threads read consecutive words in both cases
@@ -756,71 +808,48 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     T* outp = reinterpret_cast<T*>(a.out);
     T* accp = reinterpret_cast<T*>(a.acc);
     const T* Unp = reinterpret_cast<const T*>(a.Un);
-    const T rka = pick<T>(a.rk_a, a.rk_a_f), rkb = pick<T>(a.rk_b, a.rk_b_f);
     const T acs = pick<T>(a.acc_scale, a.acc_scale_f);
     bool bad = false;
-    for (int idx = threadIdx.x; idx < LINES * SEG; idx += NT) {
-        int l, p;
-        if (DIR == 0) { l = idx / SEG; p = idx - l * SEG; }
-        else { p = idx / LINES; l = idx - p * LINES; }
-        long long g;
-        int fl, fr_, cpos;   // left and right face, stencil start of the left face
-        if constexpr (FLAT) {
-            // the cell between faces idx and idx + 1 of the same piece
-            const bool inA = idx + 1 < nA;
-            if (!inA && (idx < nA || idx + 1 >= nA + nB)) continue;   // line junction or past the end
-            int inplane;
-            g = flat_line(inA ? LA : LA + 1, inplane) + (long long)(inA ? fA0 + idx : idx - nA) * sd;
-            fl = idx;
-            fr_ = idx + 1;
-            cpos = inA ? idx : idx + 5;
-        } else {
-            const int line = line0 + l;
-            const int cell = c0 + p;
-            if (line >= nline || cell >= nd) continue;
-            g = a.off0 + (long long)line * sl + (long long)pb * sp + (long long)cell * sd;
-            fl = DIR == 0 ? l * FACES + p : p * LINES + l;
-            fr_ = DIR == 0 ? fl + 1 : fl + LINES;
-            cpos = p;
-        }
+    long long g = 0;
+    int l = 0, fl = 0, fr_ = 0, cpos = 0;
+    if (out_cell(g, l, fl, fr_, cpos)) {
         if (a.mode == MODE_ACC_SET) {
             // the flux difference unscaled: the sweep that reads the
             // accumulator multiplies it by acc_scale
 #pragma unroll
             for (int v = 0; v < NV; ++v) accp[g + v * a.sv] = fh[v * NFACE + fl] - fh[v * NFACE + fr_];
-            continue;
-        }
-        T rv[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) rv[v] = (fh[v * NFACE + fl] - fh[v * NFACE + fr_]) * inv_dx;
-        if (a.mode == MODE_ACC_ADD) {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) accp[g + v * a.sv] = fmaT(accp[g + v * a.sv], acs, rv[v]);
-        } else if (a.mode == MODE_RHS) {
-#pragma unroll
-            for (int v = 0; v < NV; ++v) outp[g + v * a.sv] = accp ? fmaT(accp[g + v * a.sv], acs, rv[v]) : rv[v];
         } else {
-            const int ci = FLAT ? cpos + 3 : cidx(l, cpos + 3);
-            T nu[NV];
+            T tot[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                T tot = rv[v];
-                if (accp) tot = fmaT(accp[g + v * a.sv], acs, tot);
-                T val = rkb * fmaT(dt, tot, cq[(CL::U + v) * NCELL + ci]);
-                if (rka != T(0)) val = fmaT(rka, Unp[g + v * a.sv], val);
-                nu[v] = val;
-                outp[g + v * a.sv] = val;
+                tot[v] = (fh[v * NFACE + fl] - fh[v * NFACE + fr_]) * inv_dx;
+                if (accp) tot[v] = fmaT(EARLY ? ea[v] : accp[g + v * a.sv], acs, tot[v]);
             }
-            // admissibility: rho > 0, p > 0  <=>  2 rho E > |m|^2, finite
-            T m2 = T(0);
+            if (a.mode != MODE_COMBINE) {
+                T* o = a.mode == MODE_ACC_ADD ? accp : outp;
 #pragma unroll
-            for (int k = 0; k < DIM; ++k) m2 = fmaT(nu[1 + k], nu[1 + k], m2);
-            const T chk = T(2) * nu[0] * nu[DIM + 1] - m2;
-            if (!(nu[0] > T(0)) || !(chk > T(0)) || !isfinite(chk)) bad = true;
-            if (cfl != nullptr) {
-                T sp;
-                if (!cell_speed<T, DIM>(nu, gamma, cfl->inv_dx, sp)) cfl->bad = true;
-                else cfl->smax = max_nn(cfl->smax, sp);
+                for (int v = 0; v < NV; ++v) o[g + v * a.sv] = tot[v];
+            } else {
+                const int ci = FLAT ? cpos + 3 : cidx(l, cpos + 3);
+                T nu[NV];
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    T val = rkb * fmaT(dt, tot[v], cq[(CL::U + v) * NCELL + ci]);
+                    if (rka != T(0)) val = fmaT(rka, EARLY ? en[v] : Unp[g + v * a.sv], val);
+                    nu[v] = val;
+                    outp[g + v * a.sv] = val;
+                }
+                // admissibility: rho > 0, p > 0  <=>  2 rho E > |m|^2, finite
+                T m2 = T(0);
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) m2 = fmaT(nu[1 + k], nu[1 + k], m2);
+                const T chk = T(2) * nu[0] * nu[DIM + 1] - m2;
+                if (!(nu[0] > T(0)) || !(chk > T(0)) || !isfinite(chk)) bad = true;
+                if (cfl != nullptr) {
+                    T sp;
+                    if (!cell_speed<T, DIM>(nu, gamma, cfl->inv_dx, sp)) cfl->bad = true;
+                    else cfl->smax = max_nn(cfl->smax, sp);
+                }
             }
         }
     }
@@ -833,7 +862,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 2) k_sweep(SweepArgs a)
 {
     pdl_enter();
     if (a.tm != nullptr) {
-        if (a.tm->status != 0 || !(a.tm->dt > 0.0)) return;
+        if (a.tm->status != 0 || a.tm->go == 0) return;
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int seg_blk, line0, pb;
@@ -841,7 +870,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 2) k_sweep(SweepArgs a)
     else if (DIR == 0) { seg_blk = blockIdx.x; line0 = blockIdx.y * LINES; pb = blockIdx.z; }
     else if (DIR == 1) { seg_blk = blockIdx.y; line0 = blockIdx.x * LINES; pb = blockIdx.z; }
     else { seg_blk = blockIdx.z; line0 = blockIdx.x * LINES; pb = blockIdx.y; }
-    const T dt = a.mode == MODE_COMBINE ? T(a.tm->dt) : T(0);
+    const T dt = a.mode == MODE_COMBINE ? pick<T>(a.tm->dt, a.tm->dt_f) : T(0);
     const bool bad = sweep_tile<T, DIM, DIR, LINES, SEG, NT, EXACTDET, FLAT>(a, seg_blk, line0, pb, dt, smem_raw);
     if (bad) atomicOr(&a.tm->status, 1);
 }
@@ -946,7 +975,7 @@ __global__ void __launch_bounds__(256) k_lf_alpha(CflArgs a, unsigned long long*
 {
     pdl_enter();
     constexpr int NV = DIM + 2;
-    if (a.tm != nullptr && (a.tm->status != 0 || !(a.tm->dt > 0.0))) return;
+    if (a.tm != nullptr && (a.tm->status != 0 || a.tm->go == 0)) return;
     const T* U = reinterpret_cast<const T*>(a.U);
     const long long nx = a.n[0], ny = a.n[1];
     const long long total = nx * ny * (long long)a.n[2];
@@ -998,6 +1027,8 @@ static __global__ void k_dt(DevTime* tm, double cfl, double smax_floor)
         dt = cfl_step(cfl, smax, tm->t, tm->t_end, &clipped);
     }
     tm->dt = dt;
+    tm->dt_f = (float)dt;
+    tm->go = dt > 0.0;
     tm->clipped = clipped;
     tm->smax_bits = 0ull;
     // boundary times of the three stages (Shu-Osher RK3: t, t + dt, t + dt/2)
@@ -1021,6 +1052,7 @@ static __global__ void k_post(DevTime* tm)
         tm->steps += 1;
     }
     tm->dt = 0.0;
+    tm->go = 0;
 }
 
 // ------------------------------------------------------- conserved totals

@@ -65,7 +65,7 @@ __global__ void __launch_bounds__(WPB * 32, MINW / WPB) k_march(SweepArgs a)
 
     pdl_enter();
     if (a.tm != nullptr) {
-        if (a.tm->status != 0 || !(a.tm->dt > 0.0)) return;
+        if (a.tm->status != 0 || a.tm->go == 0) return;
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(WPB * 32, MINW / WPB) k_march(SweepArgs a)
     const T* Unp = reinterpret_cast<const T*>(a.Un);
     const T rka = pick<T>(a.rk_a, a.rk_a_f), rkb = pick<T>(a.rk_b, a.rk_b_f);
     const T acs = pick<T>(a.acc_scale, a.acc_scale_f);
-    const T dt = a.mode == MODE_COMBINE ? T(a.tm->dt) : T(0);
+    const T dt = a.mode == MODE_COMBINE ? pick<T>(a.tm->dt, a.tm->dt_f) : T(0);
     bool bad = false;
     // cells in batches of CH: the loads of a batch are issued before its
     // arithmetic and stores (one memory latency per batch, not per cell)
