@@ -157,27 +157,34 @@ __device__ __forceinline__ int cell_source(const SweepArgs& a, long long line_ba
     const long long sd = DIR == 0 ? 1LL : (DIR == 1 ? a.sy : a.sz);
     int src = along;
     flip = false;
-    if (along < 0 || along >= nd) {
+    if ((unsigned)along >= (unsigned)nd) {
         const int side = along < 0 ? 0 : 1;
         const int gl = side == 0 ? -along : along - nd + 1;
         int bc = side == 0 ? a.bc_lo : a.bc_hi;
-        int fixed = -1;
-        if (bc == BC_INFLOW) {
-            fixed = 0;
-        } else if (bc == BC_DMR_BOTTOM) {
-            const double x = a.lo0 + (line + 0.5) * a.dx0;
-            if (x < 1.0 / 6.0) fixed = 0;
-            else bc = BC_REFLECT;
-        } else if (bc == BC_DMR_TOP) {
-            // shock position on the top boundary at the boundary time
-            const double xs = a.tm != nullptr ? a.tm->xs_top[a.stage] : a.xs_fixed;
-            const double x = a.lo0 + (line + 0.5) * a.dx0;
-            fixed = x < xs ? 0 : 1;
-        } else if (bc == BC_JET) {
-            const double y = a.lo1 + (line + 0.5) * a.dx1;
-            fixed = y < JET_HALF_WIDTH ? 0 : 1;
+        if (bc >= BC_INFLOW) {
+            // The boundaries that compare a coordinate.  The empty asm keeps
+            // their double arithmetic inside this branch: speculated, it ran
+            // for every cell of a tile at the end of a line (34% of the
+            // FP64-pipe cycles of the float 224^3 x-sweep)
+            asm volatile("" ::: "memory");
+            int fixed = -1;
+            if (bc == BC_INFLOW) {
+                fixed = 0;
+            } else if (bc == BC_DMR_BOTTOM) {
+                const double x = a.lo0 + (line + 0.5) * a.dx0;
+                if (x < 1.0 / 6.0) fixed = 0;
+                else bc = BC_REFLECT;
+            } else if (bc == BC_DMR_TOP) {
+                // shock position on the top boundary at the boundary time
+                const double xs = a.tm != nullptr ? a.tm->xs_top[a.stage] : a.xs_fixed;
+                const double x = a.lo0 + (line + 0.5) * a.dx0;
+                fixed = x < xs ? 0 : 1;
+            } else if (bc == BC_JET) {
+                const double y = a.lo1 + (line + 0.5) * a.dx1;
+                fixed = y < JET_HALF_WIDTH ? 0 : 1;
+            }
+            if (fixed >= 0) return fixed;
         }
-        if (fixed >= 0) return fixed;
         if (bc == BC_TRANSMISSIVE) src = side == 0 ? 0 : nd - 1;
         else if (bc == BC_REFLECT) { src = side == 0 ? gl - 1 : nd - gl; flip = true; }
         else src = side == 0 ? nd - gl : gl - 1;
