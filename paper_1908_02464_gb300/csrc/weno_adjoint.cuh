@@ -292,7 +292,7 @@ struct VjpArgs {
     int hybrid;
     // boundary conditions of this direction, for the ghost cells computed
     // while staging (the fields stage_cell reads: bc_lo, bc_hi, bc_state,
-    // lo0, dx0, lo1, dx1, tm = null, xs_fixed)
+    // fix_line, tm = null)
     SweepArgs bc;
     // cell primitives (cell_prims, PrimLayout records at STRIDE g): P read
     // (an earlier direction stored them), Pout computed and stored for the

@@ -3,11 +3,16 @@
 //
 // Step sequence (one RK3 step, Sec. 4 of the paper) on three rotating state
 // buffers (cur, x, y) selected by phase = completed steps mod 3:
-//   k_cfl(cur) -> k_dt (dt, and the boundary times t, t+dt, t+dt/2)
 //   stage 1: sweeps(cur)         -> x = cur + dt L(cur)
 //   stage 2: sweeps(x), base cur -> y = 3/4 cur + 1/4 (x + dt L(x))
-//   stage 3: sweeps(y), base cur -> x = 1/3 cur + 2/3 (y + dt L(y))
-//   k_post (t += dt, steps += 1 unless a stage failed)
+//   stage 3: sweeps(y), base cur -> x = 1/3 cur + 2/3 (y + dt L(y)); the last
+//            one also takes the CFL wave speeds of the state it writes
+//   k_next (t += dt, steps += 1 unless a stage failed; the next dt, and the
+//            boundary times t, t+dt, t+dt/2)
+// A call begins with k_cfl(cur), which does nothing when the last step has
+// left its wave speeds, and k_begin (dt towards the call's target time).  CFL,
+// dt and bookkeeping kernels in every step took 13 of 206 us on the 2048 x 512
+// grid in mixed precision and 14 of 300 us on 512 x 128 in FP64.
 // The sweeps take the ghost cells from the boundary conditions at the
 // stage's time while staging their tiles; no ghost-cell kernel runs.
 // The new state is x, i.e. buffer (phase + 1) mod 3.  A failed admissibility
@@ -131,12 +136,18 @@ static wis::SweepArgs sweep_args(weno_ctx* c, int dir)
             a.bc_state[s][v] = c->g.bc_state[s][v];
             a.bc_state_f[s][v] = (float)c->g.bc_state[s][v];
         }
-    a.lo0 = c->g.lo[0];
-    a.dx0 = c->dx[0];
-    a.lo1 = c->g.lo[1];
-    a.dx1 = c->dx[1];
+    for (int s = 0; s < 2; ++s) {
+        const int bc = s == 0 ? a.bc_lo : a.bc_hi;
+        a.fix_line[s] = INT_MAX;   // one state on the whole side
+        if (bc == wis::BC_DMR_BOTTOM) a.fix_line[s] = wis::cells_below(1.0 / 6.0, c->g.lo[0], c->dx[0], c->n[0]);
+        if (bc == wis::BC_JET) a.fix_line[s] = wis::cells_below(wis::JET_HALF_WIDTH, c->g.lo[1], c->dx[1], c->n[1]);
+    }
     a.acc_scale = 1.0;
     a.acc_scale_f = 1.0f;
+    for (int d = 0; d < 3; ++d) {
+        a.cfl_inv_dx[d] = d < c->dim ? c->inv_dx[d] : 0.0;
+        a.cfl_inv_dx_f[d] = (float)a.cfl_inv_dx[d];
+    }
     a.fx = c->prec == WENO_FP64 && wis::use_fx((long long)interior_cells(c)) ? 1 : 0;
     // a stage sweeps the directions from the last to x: the first one
     // computes and stores the primitives, the others read them
@@ -145,6 +156,14 @@ static wis::SweepArgs sweep_args(weno_ctx* c, int dir)
         else a.P = c->prim;
     }
     return a;
+}
+
+// boundary time of sweeps without a DevTime
+static void set_time(const weno_ctx* c, wis::SweepArgs& a, double t)
+{
+    for (int s = 0; s < 2; ++s)
+        if ((s == 0 ? a.bc_lo : a.bc_hi) == wis::BC_DMR_TOP)
+            a.fix_line[s] = wis::cells_below(wis::dmr_shock_x(t), c->g.lo[0], c->dx[0], c->n[0]);
 }
 
 // Direction of the sweep at position i of a stage.  The last sweep reads
@@ -236,6 +255,7 @@ static cudaError_t issue_stage(weno_ctx* c, void* in, const void* base, void* ou
             a.out = out;
             a.acc = c->dim > 1 ? c->acc : nullptr;
             set_rk(a, ra, rb);
+            a.cfl = stage == 2;   // the state of the finished step
         } else {
             a.mode = i == 0 ? wis::MODE_ACC_SET : wis::MODE_ACC_ADD;
             a.acc = c->acc;
@@ -246,26 +266,45 @@ static cudaError_t issue_stage(weno_ctx* c, void* in, const void* base, void* ou
     return cudaSuccess;
 }
 
-static cudaError_t issue_step(weno_ctx* c, int ph, cudaStream_t s)
+static wis::StepArgs step_args(const weno_ctx* c)
 {
-    void* cur = c->buf[ph % 3];
-    void* x = c->buf[(ph + 1) % 3];
-    void* y = c->buf[(ph + 2) % 3];
+    wis::StepArgs a;
+    a.cfl = c->p.cfl;
+    a.smax_floor = c->smax_floor;
+    a.dmr_top = c->g.bc_lo[1] == wis::BC_DMR_TOP || c->g.bc_hi[1] == wis::BC_DMR_TOP;
+    a.n0 = c->n[0];
+    a.lo0 = c->g.lo[0];
+    a.dx0 = c->dx[0];
+    return a;
+}
+
+// Before the first step of a call: the wave speeds of the current state,
+// unless the step that wrote it has left them (k_cfl returns at once then),
+// and dt towards the target time.
+static cudaError_t issue_begin(weno_ctx* c, int ph, cudaStream_t s)
+{
     wis::CflArgs ca;
     std::memset(&ca, 0, sizeof(ca));
-    ca.U = cur;
+    ca.U = c->buf[ph % 3];
     for (int k = 0; k < 3; ++k) { ca.n[k] = c->n[k]; ca.inv_dx[k] = k < c->dim ? c->inv_dx[k] : 0.0; }
     ca.sy = c->sy; ca.sz = c->sz; ca.sv = c->sv; ca.off0 = c->off0;
     ca.gamma = c->p.gamma;
     ca.tm = c->tm;
     cudaError_t e = do_cfl(c, ca, s);
     if (e != cudaSuccess) return e;
-    e = wis::launch_pdl(wis::k_dt, dim3(1), dim3(1), 0, s, c->tm, c->p.cfl, c->smax_floor);
-    if (e != cudaSuccess) return e;
+    return wis::launch_pdl(wis::k_begin, dim3(1), dim3(32), 0, s, c->tm, step_args(c));
+}
+
+static cudaError_t issue_step(weno_ctx* c, int ph, cudaStream_t s)
+{
+    void* cur = c->buf[ph % 3];
+    void* x = c->buf[(ph + 1) % 3];
+    void* y = c->buf[(ph + 2) % 3];
+    cudaError_t e;
     if ((e = issue_stage(c, cur, nullptr, x, 0.0, 1.0, 0, 0, s)) != cudaSuccess) return e;
     if ((e = issue_stage(c, x, cur, y, 0.75, 0.25, 1, 1, s)) != cudaSuccess) return e;
     if ((e = issue_stage(c, y, cur, x, 1.0 / 3.0, 2.0 / 3.0, 2, 2, s)) != cudaSuccess) return e;
-    return wis::launch_pdl(wis::k_post, dim3(1), dim3(1), 0, s, c->tm);
+    return wis::launch_pdl(wis::k_next, dim3(1), dim3(32), 0, s, c->tm, step_args(c));
 }
 
 static weno_status build_graphs(weno_ctx* ctx)
@@ -707,7 +746,7 @@ static weno_status issue_rhs(weno_ctx* ctx, const void* U, void* out, double t, 
         set_acc_scale(ctx, a, i);
         a.sy = sy; a.sz = sz; a.sv = sv; a.off0 = 0;
         a.U = U;
-        a.xs_fixed = wis::dmr_shock_x(t);
+        set_time(ctx, a, t);
         a.alpha_g = ctx->alpha_g + 3 * 9 + 3 * d;
         if (flags) a.flags = flags + foff[d];
         if (i == ctx->dim - 1) {
@@ -798,7 +837,7 @@ weno_status weno_rhs_vjp(weno_ctx* ctx, const void* U_dev, const void* w_dev, vo
         a.bc = sweep_args(ctx, d);
         a.bc.sy = sy; a.bc.sz = sz; a.bc.sv = sv; a.bc.off0 = 0;
         a.bc.tm = nullptr;
-        a.bc.xs_fixed = wis::dmr_shock_x(t);
+        set_time(ctx, a.bc, t);
         // FP64: the x pass computes the cell primitives of U and stores
         // them, the y and z passes read them (as the forward sweeps share
         // theirs within a stage)
@@ -845,7 +884,12 @@ weno_status weno_step(weno_ctx* ctx, double t_end, double* dt_taken)
     if (st != WENO_OK) return st;
     const double t0 = ctx->tm_host->t;
     if ((st = set_t_end(ctx, t_end)) != WENO_OK) return st;
-    CK(ctx->run1d ? issue_run1d(ctx, 1, ctx->stream) : issue_step(ctx, ctx->phase, ctx->stream));
+    if (ctx->run1d) {
+        CK(issue_run1d(ctx, 1, ctx->stream));
+    } else {
+        CK(issue_begin(ctx, ctx->phase, ctx->stream));
+        CK(issue_step(ctx, ctx->phase, ctx->stream));
+    }
     st = finish_steps(ctx);
     if (dt_taken) *dt_taken = ctx->tm_host->t - t0;
     return st;
@@ -863,6 +907,8 @@ weno_status weno_advance(weno_ctx* ctx, double t_end, int max_steps, int* steps_
     int remaining = max_steps;
     // a few milliseconds of work between two looks at the time
     const int chunk = ctx->run1d ? 1024 : 64;
+    if (!ctx->run1d && remaining > 0 && ctx->tm_host->status == 0 && ctx->tm_host->t < t_end)
+        CK(issue_begin(ctx, ctx->phase, ctx->stream));
     while (remaining > 0 && ctx->tm_host->status == 0 && ctx->tm_host->t < t_end) {
         const int k = remaining < chunk ? remaining : chunk;
         const long long before = ctx->tm_host->steps;
@@ -887,6 +933,7 @@ weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps)
     if (ctx->run1d) {
         if (nsteps > 0) CK(issue_run1d(ctx, nsteps, ctx->stream));
     } else {
+        if (nsteps > 0) CK(issue_begin(ctx, ctx->phase, ctx->stream));
         for (int i = 0; i < nsteps; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
     }
     ctx->phase = (ctx->phase + nsteps) % 3;
@@ -905,7 +952,7 @@ static weno_status time_sweep_dir(weno_ctx* ctx, int d, int reps, void* flush_de
         CK(cudaMemsetAsync(ctx->wcount, 0, sizeof(unsigned long long), ctx->stream));
         wis::SweepArgs a = sweep_args(ctx, d);
         a.U = cur;
-        a.xs_fixed = wis::dmr_shock_x(ctx->tm_host->t);
+        set_time(ctx, a, ctx->tm_host->t);
         a.alpha_g = ctx->alpha_g + 3 * 9 + 3 * d;
         a.mode = wis::MODE_ACC_SET;
         a.acc = ctx->dim > 1 ? ctx->acc : ctx->rhs_out;
@@ -937,7 +984,7 @@ static weno_status prepare_timing(weno_ctx* ctx)
         const int d = ctx->dim - 1;
         wis::SweepArgs a = sweep_args(ctx, d);
         a.U = cur;
-        a.xs_fixed = wis::dmr_shock_x(ctx->tm_host->t);
+        set_time(ctx, a, ctx->tm_host->t);
         a.alpha_g = ctx->alpha_g + 3 * 9 + 3 * d;
         a.mode = wis::MODE_ACC_SET;
         a.acc = ctx->acc;

@@ -132,7 +132,6 @@ __device__ __forceinline__ SweepArgs batch_sweep_args(const BatchArgs& b, const 
     a.gamma_f = b.gamma_f; a.eps_f = b.eps_f; a.lam_scale_f = b.lam_scale_f;
     a.bc_lo = b.bc_lo[d]; a.bc_hi = b.bc_hi[d];
     a.stage = 0;
-    a.xs_fixed = 0.0;
     a.fx = FX && use_fx(cells);
     return a;
 }

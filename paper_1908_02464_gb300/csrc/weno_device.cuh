@@ -398,6 +398,18 @@ __device__ __forceinline__ bool abs_lt(double w, double lim)
 }
 __device__ __forceinline__ bool abs_lt(float w, float lim) { return (__float_as_int(w) & 0x7fffffff) < __float_as_int(lim); }
 
+// |x|, zero for NaN (integer pipes)
+__device__ __forceinline__ double abs_or_zero(double x)
+{
+    const long long b = __double_as_longlong(x) & 0x7fffffffffffffffLL;
+    return __longlong_as_double(b > 0x7ff0000000000000LL ? 0LL : b);
+}
+__device__ __forceinline__ float abs_or_zero(float x)
+{
+    const int b = __float_as_int(x) & 0x7fffffff;
+    return __int_as_float(b > 0x7f800000 ? 0 : b);
+}
+
 // w[s] = L^s . x for all fields.
 template <typename T, int DIM, int DIR>
 __device__ __forceinline__ void proj_all(const Roe<T, DIM>& r, const T* x, T* w)

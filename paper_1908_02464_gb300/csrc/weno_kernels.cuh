@@ -12,7 +12,7 @@
 //             divergence and writes an accumulator, a right-hand side or the
 //             RK3 stage combination (Sec. 4).
 //   k_cfl     CFL wave-speed max-reduction and admissibility check.
-//   k_dt, k_post   single-thread time-step bookkeeping on the device.
+//   k_begin, k_next  single-thread time-step bookkeeping on the device.
 //   k_totals  conserved totals, FP64 accumulation.
 #pragma once
 
@@ -58,19 +58,33 @@ struct DevTime {
     double t;                       // time of the current state
     double dt;                      // step in progress (0: nothing to do)
     double t_end;                   // target of the step in progress
-    unsigned long long smax_bits;   // max wave speed sum (bits of a positive double)
+    unsigned long long smax_bits;   // max wave speed sum of the current state (bits of a positive double)
+    unsigned long long smax_next;   // the same of the state that the step in progress writes
+    int smax_valid;                 // smax_bits holds the current state's
+    int cfl_bad;                    // a cell of the current state has no admissible wave speed
     long long steps;                // completed steps
     int status;                     // 0 ok, else WENO_ERR_NONPHYSICAL latched
     int clipped;                    // 1 if dt was clipped to reach t_end
     int go;                         // dt > 0 (float kernels keep off the FP64 pipe)
     float dt_f;
-    double xs_top[3];               // double Mach top boundary: shock position at the
-                                    // stage times t, t + dt, t + dt/2
+    int top_line[3];                // double Mach top boundary: columns behind the shock
+                                    // at the stage times t, t + dt, t + dt/2
 };
 
 // Shock position on the top boundary of the double Mach reflection at time t
 // (the Mach 10 shock through (1/6, 0) at 60 degrees moves at 10 / sin 60).
 __host__ __device__ inline double dmr_shock_x(double t) { return 1.0 / 6.0 + (1.0 + 20.0 * t) / sqrt(3.0); }
+
+// number of cells of a line (n cells of size dx from lo) whose centres lie
+// below x, from an estimate in float
+__host__ __device__ inline int cells_below(double x, double lo, double dx, int n)
+{
+    const float e = (float)(x - lo) / (float)dx;
+    int k = e > (float)n ? n : (e > 0.0f ? (int)e : 0);
+    while (k < n && fma(k + 0.5, dx, lo) < x) ++k;
+    while (k > 0 && !(fma(k - 0.5, dx, lo) < x)) --k;
+    return k;
+}
 
 enum { MODE_ACC_SET = 0, MODE_ACC_ADD = 1, MODE_COMBINE = 2, MODE_RHS = 3 };
 // flux splitting (Eq. flxuspliting): local LF over the six stencil cells,
@@ -103,9 +117,9 @@ struct SweepArgs {
     int bc_lo, bc_hi;
     double bc_state[2][5];
     float bc_state_f[2][5];
-    double lo0, dx0, lo1, dx1;   // x and y geometry (double Mach, jet)
-    int stage;                   // RK stage (index of tm->xs_top)
-    double xs_fixed;             // double Mach shock position when tm is null
+    int fix_line[2];             // per side: lines below it take bc_state[0] (double Mach top:
+                                 // when tm is null)
+    int stage;                   // RK stage (index of tm->top_line)
     // Primitives (cell_prims) of U's interior cells: the record of the cell
     // at index g of U's layout at P + PrimLayout::STRIDE g.  P: read them (the first sweep of the stage
     // wrote them); Pout: the tiles compute them and store those of their own
@@ -119,6 +133,11 @@ struct SweepArgs {
     double acc_scale = 1.0;
     float acc_scale_f = 1.0f;
     int fx = 0;   // FP64: the six-point sums in 64-bit integers (use_fx)
+    // last sweep of a step: the CFL wave speeds of the cells written go to
+    // tm->smax_next and tm->cfl_bad (1 / dx of every direction)
+    int cfl = 0;
+    double cfl_inv_dx[3];
+    float cfl_inv_dx_f[3];
 };
 
 // FP64 problems of at least this many cells form their six-point sums on the
@@ -162,28 +181,14 @@ __device__ __forceinline__ int cell_source(const SweepArgs& a, long long line_ba
         const int gl = side == 0 ? -along : along - nd + 1;
         int bc = side == 0 ? a.bc_lo : a.bc_hi;
         if (bc >= BC_INFLOW) {
-            // The boundaries that compare a coordinate.  The empty asm keeps
-            // their double arithmetic inside this branch: speculated, it ran
-            // for every cell of a tile at the end of a line (34% of the
-            // FP64-pipe cycles of the float 224^3 x-sweep)
-            asm volatile("" ::: "memory");
-            int fixed = -1;
-            if (bc == BC_INFLOW) {
-                fixed = 0;
-            } else if (bc == BC_DMR_BOTTOM) {
-                const double x = a.lo0 + (line + 0.5) * a.dx0;
-                if (x < 1.0 / 6.0) fixed = 0;
-                else bc = BC_REFLECT;
-            } else if (bc == BC_DMR_TOP) {
-                // shock position on the top boundary at the boundary time
-                const double xs = a.tm != nullptr ? a.tm->xs_top[a.stage] : a.xs_fixed;
-                const double x = a.lo0 + (line + 0.5) * a.dx0;
-                fixed = x < xs ? 0 : 1;
-            } else if (bc == BC_JET) {
-                const double y = a.lo1 + (line + 0.5) * a.dx1;
-                fixed = y < JET_HALF_WIDTH ? 0 : 1;
-            }
-            if (fixed >= 0) return fixed;
+            // fixed states; the boundaries that compare a coordinate do so by
+            // the line's index (as doubles, the comparison ran speculated for
+            // every cell of a tile at the end of a line: 34% of the FP64-pipe
+            // cycles of the float 224^3 x-sweep)
+            const int lim = bc == BC_DMR_TOP && a.tm != nullptr ? a.tm->top_line[a.stage] : a.fix_line[side];
+            if (line < lim) return 0;
+            if (bc != BC_DMR_BOTTOM) return 1;
+            bc = BC_REFLECT;
         }
         if (bc == BC_TRANSMISSIVE) src = side == 0 ? 0 : nd - 1;
         else if (bc == BC_REFLECT) { src = side == 0 ? gl - 1 : nd - gl; flip = true; }
@@ -307,6 +312,26 @@ __device__ __forceinline__ T fifth_difference(T u0, T u1, T u2, T u3, T u4, T u5
     T c0 = b1 - b0, c1 = b2 - b1, c2 = b3 - b2;
     T d0 = c1 - c0, d1 = c2 - c1;
     return d1 - d0;
+}
+
+// warp maximum of non-negative values on their bit patterns (a double compare
+// would take the FP64 pipe in float kernels too)
+template <typename T>
+__device__ __forceinline__ T warp_max_nn(T v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = max_nn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// *to = max(*to, m) for a non-negative m, as bits of a double; a value below
+// the maximum so far costs no atomic
+template <typename T>
+__device__ __forceinline__ void raise_max(unsigned long long* to, T m)
+{
+    if (!(m > T(0))) return;
+    const unsigned long long b = (unsigned long long)__double_as_longlong((double)m);
+    if (b > *(volatile unsigned long long*)to) atomicMax(to, b);
 }
 
 // CFL wave-speed sum sum_d (|u_d| + c) / dx_d of one cell; false if the cell
@@ -447,6 +472,8 @@ __device__ __forceinline__ void weno_queue(const SweepArgs& a, int nq, const T* 
 // full set of faces, and a tile that reaches the end of a line continues on
 // the next one, each piece with its own halo.  line0 and pb are unused then.
 // FX: a.fx may ask for the integer six-point sums (FP64).
+// FIRST: a.mode is MODE_ACC_SET, known when compiled (the first sweep of a
+// float stage then holds no registers for the accumulator and base state).
 // cfl (COMBINE mode, may be null): the CFL wave speeds of the cells written
 // (cell_speed), for the step that follows.
 template <typename T, int DIM>
@@ -454,9 +481,24 @@ struct TileCfl {
     T inv_dx[DIM];   // 1 / dx per direction
     T smax;          // running maximum over the cells this thread wrote
     bool bad;        // a cell this thread wrote is not admissible
+
+    __device__ __forceinline__ void init(const SweepArgs& a)
+    {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) inv_dx[d] = pick<T>(a.cfl_inv_dx[d], a.cfl_inv_dx_f[d]);
+        smax = T(0);
+        bad = false;
+    }
+    // by every thread of the warp
+    __device__ __forceinline__ void note(DevTime* tm) const
+    {
+        const T m = warp_max_nn(smax);
+        if ((threadIdx.x & 31) == 0) raise_max(&tm->smax_next, m);
+        if (bad) atomicOr(&tm->cfl_bad, 1);
+    }
 };
 template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false,
-          bool FX = sizeof(T) == 8>
+          bool FX = sizeof(T) == 8, bool FIRST = false>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int line0, int pb, T dt,
                                            unsigned char* smem_raw, TileCfl<T, DIM>* cfl = nullptr)
 {
@@ -629,18 +671,19 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     // cycles per issue in the accumulating 160^3 y-sweep, which took 186 us
     // against 115 us without the accumulator; 10 steps of the 2048 x 512 grid
     // 2.06 -> 2.02 ms).  FP64 tiles, bound by their pipe, keep the registers.
-    constexpr bool EARLY = sizeof(T) == 4;
+    constexpr bool EARLY = sizeof(T) == 4 && !FIRST;
+    const int mode = FIRST ? MODE_ACC_SET : a.mode;
     T ea[NV], en[NV];
     if constexpr (EARLY) {
         long long g = 0;
         int l = 0, fl = 0, fr_ = 0, cpos = 0;
-        const bool read = a.mode != MODE_ACC_SET && out_cell(g, l, fl, fr_, cpos);
+        const bool read = mode != MODE_ACC_SET && out_cell(g, l, fl, fr_, cpos);
         const T* accr = reinterpret_cast<const T*>(a.acc);
         const T* Unr = reinterpret_cast<const T*>(a.Un);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             ea[v] = read && accr != nullptr ? accr[g + v * a.sv] : T(0);
-            en[v] = read && a.mode == MODE_COMBINE && rka != T(0) ? Unr[g + v * a.sv] : T(0);
+            en[v] = read && mode == MODE_COMBINE && rka != T(0) ? Unr[g + v * a.sv] : T(0);
         }
     }
 
@@ -820,7 +863,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     long long g = 0;
     int l = 0, fl = 0, fr_ = 0, cpos = 0;
     if (out_cell(g, l, fl, fr_, cpos)) {
-        if (a.mode == MODE_ACC_SET) {
+        if (mode == MODE_ACC_SET) {
             // the flux difference unscaled: the sweep that reads the
             // accumulator multiplies it by acc_scale
 #pragma unroll
@@ -832,8 +875,8 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
                 tot[v] = (fh[v * NFACE + fl] - fh[v * NFACE + fr_]) * inv_dx;
                 if (accp) tot[v] = fmaT(EARLY ? ea[v] : accp[g + v * a.sv], acs, tot[v]);
             }
-            if (a.mode != MODE_COMBINE) {
-                T* o = a.mode == MODE_ACC_ADD ? accp : outp;
+            if (mode != MODE_COMBINE) {
+                T* o = mode == MODE_ACC_ADD ? accp : outp;
 #pragma unroll
                 for (int v = 0; v < NV; ++v) o[g + v * a.sv] = tot[v];
             } else {
@@ -864,7 +907,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     return bad;
 }
 
-template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false>
+template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false, bool FIRST = false>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 2) k_sweep(SweepArgs a)
 {
     pdl_enter();
@@ -877,9 +920,31 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 4 : 2) k_sweep(SweepArgs a)
     else if (DIR == 0) { seg_blk = blockIdx.x; line0 = blockIdx.y * LINES; pb = blockIdx.z; }
     else if (DIR == 1) { seg_blk = blockIdx.y; line0 = blockIdx.x * LINES; pb = blockIdx.z; }
     else { seg_blk = blockIdx.z; line0 = blockIdx.x * LINES; pb = blockIdx.y; }
+    if constexpr (FIRST) {
+        sweep_tile<T, DIM, DIR, LINES, SEG, NT, EXACTDET, FLAT, sizeof(T) == 8, true>(a, seg_blk, line0, pb, T(0),
+                                                                                      smem_raw);
+        return;
+    }
     const T dt = a.mode == MODE_COMBINE ? pick<T>(a.tm->dt, a.tm->dt_f) : T(0);
-    const bool bad = sweep_tile<T, DIM, DIR, LINES, SEG, NT, EXACTDET, FLAT>(a, seg_blk, line0, pb, dt, smem_raw);
+    TileCfl<T, DIM> cfl;
+    cfl.init(a);
+    const bool bad = sweep_tile<T, DIM, DIR, LINES, SEG, NT, EXACTDET, FLAT>(a, seg_blk, line0, pb, dt, smem_raw,
+                                                                             a.cfl ? &cfl : nullptr);
     if (bad) atomicOr(&a.tm->status, 1);
+    if (a.cfl) {
+        // per block: the first wave's warps would all raise the maximum
+        __shared__ T red[NT / 32];
+        const T m = warp_max_nn(cfl.smax);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            T b = red[0];
+#pragma unroll
+            for (int w = 1; w < NT / 32; ++w) b = max_nn(b, red[w]);
+            raise_max(&a.tm->smax_next, b);
+        }
+        if (cfl.bad) atomicOr(&a.tm->cfl_bad, 1);
+    }
 }
 
 // ---------------------------------------------------------------- ghosts
@@ -898,16 +963,6 @@ struct GhostArgs {
     double stage_c, t_fixed;
 };
 
-// warp maximum of non-negative values on their bit patterns (a double compare
-// would take the FP64 pipe in float kernels too)
-template <typename T>
-__device__ __forceinline__ T warp_max_nn(T v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max_nn(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 // ------------------------------------------------------- CFL reduction
 struct CflArgs {
     const void* U;
@@ -919,19 +974,12 @@ struct CflArgs {
     int parts;    // k_cfl: x-parts per grid row (rows x parts blocks of work)
 };
 
-__device__ __forceinline__ double warp_max(double v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = maxT(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
 template <typename T, int DIM>
 __global__ void __launch_bounds__(256) k_cfl(CflArgs a)
 {
     pdl_enter();
     constexpr int NV = DIM + 2;
-    if (a.tm->status != 0) return;
+    if (a.tm->status != 0 || a.tm->smax_valid != 0) return;
     const T* U = reinterpret_cast<const T*>(a.U);
     const int nx = a.n[0], ny = a.n[1];
     const long long rows = (long long)ny * a.n[2];
@@ -960,16 +1008,14 @@ __global__ void __launch_bounds__(256) k_cfl(CflArgs a)
             else smax_t = max_nn(smax_t, s);
         }
     }
-    double smax = (double)smax_t;
-    __shared__ double red[8];
-    smax = warp_max(smax);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = smax;
+    const T m = warp_max_nn(smax_t);
+    __shared__ T red[8];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        double v = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-        v = warp_max(v);
-        if (threadIdx.x == 0 && v > 0.0)
-            atomicMax(&a.tm->smax_bits, (unsigned long long)__double_as_longlong(v));
+    if (threadIdx.x == 0) {
+        T b = red[0];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) b = max_nn(b, red[w]);
+        raise_max(&a.tm->smax_bits, b);
     }
     if (bad) atomicOr(&a.tm->status, 1);
 }
@@ -977,6 +1023,9 @@ __global__ void __launch_bounds__(256) k_cfl(CflArgs a)
 // global Lax-Friedrichs speeds (Sec. 2.4 step (4), l = the whole domain):
 // per direction d, max over interior cells of |u_d - c|, |u_d|, |u_d + c|,
 // as bits of non-negative doubles (out[3 d + k], zeroed beforehand)
+// The maxima are taken on the bit patterns (a double compare takes the FP64
+// pipe) and per block before the atomics (20.4 -> 12.3 us at 637 x 159).  NaN speeds of
+// inadmissible cells are left out, as fmax leaves them out.
 template <typename T, int DIM>
 __global__ void __launch_bounds__(256) k_lf_alpha(CflArgs a, unsigned long long* out)
 {
@@ -984,64 +1033,100 @@ __global__ void __launch_bounds__(256) k_lf_alpha(CflArgs a, unsigned long long*
     constexpr int NV = DIM + 2;
     if (a.tm != nullptr && (a.tm->status != 0 || a.tm->go == 0)) return;
     const T* U = reinterpret_cast<const T*>(a.U);
-    const long long nx = a.n[0], ny = a.n[1];
-    const long long total = nx * ny * (long long)a.n[2];
+    const int nx = a.n[0], ny = a.n[1];
+    const long long rows = (long long)ny * a.n[2];
     const T gamma = T(a.gamma), gm1 = gamma - T(1);
-    double mx[3 * DIM];
+    T mx[3 * DIM];
 #pragma unroll
-    for (int q = 0; q < 3 * DIM; ++q) mx[q] = 0.0;
-    for (long long id = blockIdx.x * (long long)blockDim.x + threadIdx.x; id < total;
-         id += (long long)gridDim.x * blockDim.x) {
-        const long long i = id % nx, j = (id / nx) % ny, k = id / (nx * ny);
-        const long long g = a.off0 + i + j * a.sy + k * a.sz;
-        T u[NV];
+    for (int q = 0; q < 3 * DIM; ++q) mx[q] = T(0);
+    auto take = [](T& m, T x) { m = max_nn(m, abs_or_zero(x)); };
+    const int span = (nx + a.parts - 1) / a.parts;
+    for (long long c = blockIdx.x; c < rows * a.parts; c += gridDim.x) {
+        const long long row = c / a.parts;
+        const int part = (int)(c - row * a.parts);
+        const int j = (int)(row % ny), k = (int)(row / ny);
+        const long long gr = a.off0 + (long long)j * a.sy + (long long)k * a.sz;
+        const int x1 = min(nx, (part + 1) * span);
+        for (int i = part * span + threadIdx.x; i < x1; i += blockDim.x) {
+            T u[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) u[v] = U[g + v * a.sv];
-        T q[CellLayout<DIM>::NQ];
-        const T irho = Ar<T>::rcp(u[0]);
-        T ke2 = T(0);
+            for (int v = 0; v < NV; ++v) u[v] = U[gr + i + v * a.sv];
+            const T irho = Ar<T>::rcp(u[0]);
+            T ke2 = T(0);
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) ke2 = fmaT(u[1 + d], u[1 + d] * irho, ke2);
-        const T p = gm1 * fmaT(T(-0.5), ke2, u[DIM + 1]);
-        const T c = Ar<T>::sqrt_(gamma * p * irho);
-        (void)q;
+            for (int d = 0; d < DIM; ++d) ke2 = fmaT(u[1 + d], u[1 + d] * irho, ke2);
+            const T p = gm1 * fmaT(T(-0.5), ke2, u[DIM + 1]);
+            const T cs = Ar<T>::sqrt_(gamma * p * irho);
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            const T un = u[1 + d] * irho;
-            mx[3 * d + 0] = maxT(mx[3 * d + 0], (double)absT(un - c));
-            mx[3 * d + 1] = maxT(mx[3 * d + 1], (double)absT(un));
-            mx[3 * d + 2] = maxT(mx[3 * d + 2], (double)absT(un + c));
+            for (int d = 0; d < DIM; ++d) {
+                const T un = u[1 + d] * irho;
+                take(mx[3 * d + 0], un - cs);
+                take(mx[3 * d + 1], un);
+                take(mx[3 * d + 2], un + cs);
+            }
         }
     }
+    __shared__ T red[3 * DIM][8];
 #pragma unroll
     for (int q = 0; q < 3 * DIM; ++q) {
-        const double v = warp_max(mx[q]);
-        if ((threadIdx.x & 31) == 0 && v > 0.0) atomicMax(&out[q], (unsigned long long)__double_as_longlong(v));
+        const T m = warp_max_nn(mx[q]);
+        if ((threadIdx.x & 31) == 0) red[q][threadIdx.x >> 5] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 * DIM) {
+        T m = red[threadIdx.x][0];
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = max_nn(m, red[threadIdx.x][w]);
+        raise_max(&out[threadIdx.x], m);
     }
 }
 
-// dt = CFL / smax clipped to t_end; resets the reduction cell
-// smax_floor: wave-speed sum of the fixed boundary states (they enter the
-// domain through the ghost cells)
-static __global__ void k_dt(DevTime* tm, double cfl, double smax_floor)
+struct StepArgs {
+    double cfl;
+    double smax_floor;   // wave-speed sum of the fixed boundary states (they enter the domain
+                         // through the ghost cells)
+    int dmr_top, n0;     // double Mach top boundary, and the x axis
+    double lo0, dx0;
+};
+
+// The next step: dt = CFL / smax clipped to t_end, and its boundary times.
+// Called by one warp: lane 0 takes the step, three lanes its boundary times.
+__device__ __forceinline__ void take_dt(DevTime* tm, const StepArgs& a)
+{
+    double dt = 0.0;
+    const int lane = threadIdx.x;
+    if (lane == 0) {
+        int clipped = 0;
+        if (tm->status == 0 && tm->cfl_bad == 0) {
+            const double smax = maxT(__longlong_as_double((long long)tm->smax_bits), a.smax_floor);
+            dt = cfl_step(a.cfl, smax, tm->t, tm->t_end, &clipped);
+        }
+        tm->dt = dt;
+        tm->dt_f = (float)dt;
+        tm->go = dt > 0.0;
+        tm->clipped = clipped;
+    }
+    if (a.dmr_top) {
+        // stage times (Shu-Osher RK3: t, t + dt, t + dt/2)
+        __syncwarp();
+        const double t = tm->t;
+        dt = __shfl_sync(0xffffffffu, dt, 0);
+        if (lane < 3)
+            tm->top_line[lane] =
+                cells_below(dmr_shock_x(lane == 0 ? t : (lane == 1 ? t + dt : t + 0.5 * dt)), a.lo0, a.dx0, a.n0);
+    }
+}
+
+// before the first step of a call, after k_cfl (the target time may be new)
+static __global__ void k_begin(DevTime* tm, StepArgs a)
 {
     pdl_enter();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double dt = 0.0;
-    int clipped = 0;
-    if (tm->status == 0) {
-        const double smax = maxT(__longlong_as_double((long long)tm->smax_bits), smax_floor);
-        dt = cfl_step(cfl, smax, tm->t, tm->t_end, &clipped);
+    if (threadIdx.x == 0) {
+        if (tm->cfl_bad != 0) { tm->status = 1; tm->cfl_bad = 0; }
+        tm->smax_valid = tm->status == 0;
+        tm->smax_next = 0ull;
     }
-    tm->dt = dt;
-    tm->dt_f = (float)dt;
-    tm->go = dt > 0.0;
-    tm->clipped = clipped;
-    tm->smax_bits = 0ull;
-    // boundary times of the three stages (Shu-Osher RK3: t, t + dt, t + dt/2)
-    tm->xs_top[0] = dmr_shock_x(tm->t);
-    tm->xs_top[1] = dmr_shock_x(tm->t + dt);
-    tm->xs_top[2] = dmr_shock_x(tm->t + 0.5 * dt);
+    __syncwarp();
+    take_dt(tm, a);
 }
 
 // target time for the steps that follow on the stream
@@ -1050,16 +1135,25 @@ static __global__ void k_set_tend(DevTime* tm, double t_end)
     if (threadIdx.x == 0 && blockIdx.x == 0) tm->t_end = t_end;
 }
 
-static __global__ void k_post(DevTime* tm)
+// After a step: counts it unless a stage failed, and takes the next one from
+// the wave speeds of the state it wrote.  A state without an admissible wave
+// speed fails the step that is tried from it.
+static __global__ void k_next(DevTime* tm, StepArgs a)
 {
     pdl_enter();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (tm->status == 0 && tm->dt > 0.0) {
-        tm->t = tm->clipped ? tm->t_end : tm->t + tm->dt;
-        tm->steps += 1;
+    if (threadIdx.x == 0) {
+        if (tm->status == 0 && tm->go != 0) {
+            tm->t = tm->clipped ? tm->t_end : tm->t + tm->dt;
+            tm->steps += 1;
+            tm->smax_bits = tm->smax_next;
+        } else {
+            if (tm->status == 0 && tm->cfl_bad != 0) tm->status = 1;
+            tm->cfl_bad = 0;
+        }
+        tm->smax_next = 0ull;
     }
-    tm->dt = 0.0;
-    tm->go = 0;
+    __syncwarp();
+    take_dt(tm, a);
 }
 
 // ------------------------------------------------------- conserved totals

@@ -48,11 +48,11 @@ template <> struct Tile<5> { static constexpr int LINES = 1, SEG = 122, NT = 128
 template <> struct Tile<6> { static constexpr int LINES = 1, SEG = 250, NT = 256; static constexpr bool FLAT = true; };
 struct Tile1D { static constexpr int LINES = 1, SEG = 127, NT = 128; static constexpr bool FLAT = false; };
 
-template <typename T, int DIM, int DIR, bool EXACTDET, typename TL>
-cudaError_t launch_sweep_one(const SweepArgs& a, cudaStream_t s)
+template <typename T, int DIM, int DIR, bool EXACTDET, typename TL, bool FIRST>
+cudaError_t launch_sweep_as(const SweepArgs& a, cudaStream_t s)
 {
     using SM = SweepSmem<T, DIM, TL::LINES, TL::SEG, TL::FLAT>;
-    auto kern = k_sweep<T, DIM, DIR, TL::LINES, TL::SEG, TL::NT, EXACTDET, TL::FLAT>;
+    auto kern = k_sweep<T, DIM, DIR, TL::LINES, TL::SEG, TL::NT, EXACTDET, TL::FLAT, FIRST>;
     static bool configured = false;
     if (!configured) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes);
@@ -74,6 +74,16 @@ cudaError_t launch_sweep_one(const SweepArgs& a, cudaStream_t s)
     else if (DIR == 1) grid = dim3((a.n[0] + TL::LINES - 1) / TL::LINES, segs, a.n[2]);
     else grid = dim3((a.n[0] + TL::LINES - 1) / TL::LINES, a.n[1], segs);
     return launch_pdl(kern, grid, dim3(TL::NT), SM::bytes, s, a);
+}
+
+// the first sweep of a float stage has its own instantiation (see sweep_tile)
+template <typename T, int DIM, int DIR, bool EXACTDET, typename TL>
+cudaError_t launch_sweep_one(const SweepArgs& a, cudaStream_t s)
+{
+    if constexpr (sizeof(T) == 4 && DIM > 1) {
+        if (a.mode == MODE_ACC_SET) return launch_sweep_as<T, DIM, DIR, EXACTDET, TL, true>(a, s);
+    }
+    return launch_sweep_as<T, DIM, DIR, EXACTDET, TL, false>(a, s);
 }
 
 template <typename T, int DIM, int DIR, bool EXACTDET>
@@ -122,11 +132,9 @@ inline int grid_for(long long work, int threads, int cap)
     return (int)b;
 }
 
-template <typename T>
-cudaError_t launch_cfl_t(int dim, const CflArgs& a_in, int nsm, cudaStream_t s)
+inline int cfl_blocks(CflArgs& a, int nsm)
 {
     // rows x parts units of at least 256 cells each, about 8 blocks per SM
-    CflArgs a = a_in;
     const long long rows = (long long)a.n[1] * a.n[2];
     const long long want = (long long)nsm * 8;
     long long parts = (want + rows - 1) / rows;
@@ -134,17 +142,24 @@ cudaError_t launch_cfl_t(int dim, const CflArgs& a_in, int nsm, cudaStream_t s)
     if (parts > most) parts = most;
     if (parts < 1) parts = 1;
     a.parts = (int)parts;
-    const int blocks = grid_for(rows * parts * 256, 256, nsm * 8);
+    return grid_for(rows * parts * 256, 256, nsm * 8);
+}
+
+template <typename T>
+cudaError_t launch_cfl_t(int dim, const CflArgs& a_in, int nsm, cudaStream_t s)
+{
+    CflArgs a = a_in;
+    const int blocks = cfl_blocks(a, nsm);
     if (dim == 1) return launch_pdl(k_cfl<T, 1>, dim3(blocks), dim3(256), 0, s, a);
     if (dim == 2) return launch_pdl(k_cfl<T, 2>, dim3(blocks), dim3(256), 0, s, a);
     return launch_pdl(k_cfl<T, 3>, dim3(blocks), dim3(256), 0, s, a);
 }
 
 template <typename T>
-cudaError_t launch_lf_t(int dim, const CflArgs& a, unsigned long long* out, int nsm, cudaStream_t s)
+cudaError_t launch_lf_t(int dim, const CflArgs& a_in, unsigned long long* out, int nsm, cudaStream_t s)
 {
-    const long long cells = (long long)a.n[0] * a.n[1] * a.n[2];
-    const int blocks = grid_for(cells, 256, nsm * 8);
+    CflArgs a = a_in;
+    const int blocks = cfl_blocks(a, nsm);
     if (dim == 1) return launch_pdl(k_lf_alpha<T, 1>, dim3(blocks), dim3(256), 0, s, a, out);
     if (dim == 2) return launch_pdl(k_lf_alpha<T, 2>, dim3(blocks), dim3(256), 0, s, a, out);
     return launch_pdl(k_lf_alpha<T, 3>, dim3(blocks), dim3(256), 0, s, a, out);

@@ -338,6 +338,8 @@ __global__ void __launch_bounds__(WPB * 32, MINW / WPB) k_march(SweepArgs a)
     const T acs = pick<T>(a.acc_scale, a.acc_scale_f);
     const T dt = a.mode == MODE_COMBINE ? pick<T>(a.tm->dt, a.tm->dt_f) : T(0);
     bool bad = false;
+    TileCfl<T, DIM> cfl;
+    cfl.init(a);
     // cells in batches of CH: the loads of a batch are issued before its
     // arithmetic and stores (one memory latency per batch, not per cell)
     constexpr int CH = 4;
@@ -397,11 +399,17 @@ __global__ void __launch_bounds__(WPB * 32, MINW / WPB) k_march(SweepArgs a)
                     for (int k = 0; k < DIM; ++k) m2 = fmaT(nu[1 + k], nu[1 + k], m2);
                     const T chk = T(2) * nu[0] * nu[DIM + 1] - m2;
                     if (!(nu[0] > T(0)) || !(chk > T(0)) || !isfinite(chk)) bad = true;
+                    if (a.cfl) {
+                        T sp;
+                        if (!cell_speed<T, DIM>(nu, gamma, cfl.inv_dx, sp)) cfl.bad = true;
+                        else cfl.smax = max_nn(cfl.smax, sp);
+                    }
                 }
             }
         }
     }
     if (bad) atomicOr(&a.tm->status, 1);
+    if (a.cfl) cfl.note(a.tm);
 }
 
 // Launch of k_march: segments of 12 cells in 2D and 18 in 3D, two warps per
