@@ -285,6 +285,8 @@ struct VjpArgs {
     double inv_dx, eps_h, gamma, eps, c_lambda;
     double slim;   // 60 sqrt(eps_h), as in the forward sweep
     double lam_k;  // c_lambda / 3600
+    int fx;        // FP64: the six-point sums of linear faces in 64-bit integers, as in the
+                   // forward sweep (use_fx)
     // the same pre-rounded for float kernels: a conversion or a division per
     // thread would run on the slow FP64 pipe (38% of the cycles of the float
     // x pass)
@@ -481,7 +483,13 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             const int kk = CL::U + v;
-            dU[v] = fmaT(T(10), rec(2, kk) - rec(3, kk), fmaT(T(5), rec(4, kk) - rec(1, kk), rec(0, kk) - rec(5, kk)));
+            if (sizeof(T) == 8 && a.fx) {
+                const double x[6] = {rec(0, kk), rec(1, kk), rec(2, kk), rec(3, kk), rec(4, kk), rec(5, kk)};
+                dU[v] = T(fx_detector(x));
+            } else {
+                dU[v] = fmaT(T(10), rec(2, kk) - rec(3, kk),
+                             fmaT(T(5), rec(4, kk) - rec(1, kk), rec(0, kk) - rec(5, kk)));
+            }
         }
         T w[NV];
         proj_all<T, DIM, DIR>(r, dU, w);
@@ -620,7 +628,8 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
             // stencil weights of slot m: detector (1, -5, 10, -10, 5, -1)
             // on the U slots, central flux (1, -8, 37, 37, -8, 1) on the F
             // slots, applied as sums and differences of the symmetric pairs
-            // (10 FP64 operations per variable instead of 12; in FP32 the
+            // (10 FP64 operations per variable instead of 12, none with a.fx;
+            // 121x97x113: passes 0 of the three directions 3.53 -> 3.13 ms; in FP32 the
             // six loads held at once cost the 256-thread tiles a CTA per SM,
             // so FP32 keeps one multiply-add per slot)
 #pragma unroll
@@ -632,8 +641,13 @@ __device__ __forceinline__ unsigned int vjp_tile(const VjpArgs& a, int bx, int b
                     bu[m] = fslot[m] < 0 ? T(0) : uf[CL::U + v];
                     bf[m] = fslot[m] < 0 ? T(0) : uf[CL::F + v];
                 }
-                qb[CL::U + v] = fmaT(T(10), bu[2] - bu[3], fmaT(T(5), bu[4] - bu[1], bu[0] - bu[5]));
-                qb[CL::F + v] = fmaT(T(37), bf[2] + bf[3], fmaT(T(-8), bf[1] + bf[4], bf[0] + bf[5]));
+                if (a.fx) {
+                    qb[CL::U + v] = T(fx_detector(reinterpret_cast<const double*>(bu)));
+                    qb[CL::F + v] = T(fx_central_flux(reinterpret_cast<const double*>(bf)));
+                } else {
+                    qb[CL::U + v] = fmaT(T(10), bu[2] - bu[3], fmaT(T(5), bu[4] - bu[1], bu[0] - bu[5]));
+                    qb[CL::F + v] = fmaT(T(37), bf[2] + bf[3], fmaT(T(-8), bf[1] + bf[4], bf[0] + bf[5]));
+                }
             }
         }
         const int pc = cell - (c0 - 5);
@@ -696,7 +710,7 @@ struct VjpWenoSmem {
     static constexpr int SEG = VjpTile<T, DIM, DIR>::SEG;
     static constexpr int NF = SEG + 5, NC = SEG + 10;
     static constexpr int NV = DIM + 2, NQ = CellLayout<DIM>::NQ, NX = 4;   // record, then 1/sqrt(rho), 1/c, p, c
-    static constexpr int QC = 12;             // WENO faces per chunk
+    static constexpr int QC = 12, QB = 24;    // WENO faces per chunk, per batch
     static constexpr int NUF = 2 * NV, NRB = DIM + 2;
     // face data: Roe state, detector difference and its projection, flux
     // cotangent and its projection, splitting speeds
@@ -707,7 +721,7 @@ struct VjpWenoSmem {
     // then the bars of lambda^s and the reconstructed values of the fields
     static constexpr int NPB = DIM + 6, NFS = NPB + 2 * NV;
     static constexpr size_t cells = (size_t)NC * (NQ + NX + NV);
-    static constexpr size_t faces = (size_t)NF * (6 * NUF + NFD + NFS + NV + 2 * NRB + 3);
+    static constexpr size_t faces = (size_t)NF * NFD + (size_t)QB * (6 * NUF + NFS + NV + 2 * NRB + 3);
     static constexpr size_t chunk = (size_t)QC * (NV * 2 * 6 + NV * 2 * 2 + 6 * NPB);
     static constexpr size_t bytes = sizeof(T) * (cells + faces + chunk) + sizeof(int) * 2 * (size_t)NF;
 };
@@ -719,8 +733,11 @@ constexpr int kVjpWenoThreads = 128;
 // (255 registers and spills) a tile's dozen WENO faces filled a dozen lanes
 // of two warps; here one lane takes a (face, cell) of the projections and
 // their adjoints and a (face, field, sign) of the reconstruction's, in chunks
-// of QC queued faces, and one lane per face the rest.  Ragged 121x97x113 box
-// in FP64 with a slab across z: pass 1 of the z direction 11.76 -> 2.84 ms.
+// of QC queued faces, and one lane per face the rest.  The faces go in
+// batches of QB, each gathered into the bars that a thread keeps for its cell,
+// so that three CTAs fit an SM (two with room for all 64 faces: 2.91 ms); few
+// lines have more than one batch.  Ragged 121x97x113 box
+// in FP64 with a slab across z: pass 1 of the z direction 11.76 -> 2.31 ms.
 template <typename T, int DIM, int DIR>
 __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, int bz, int l, unsigned char* smem_raw)
 {
@@ -728,23 +745,24 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
     using PL = PrimLayout<DIM>;
     using SM = VjpWenoSmem<T, DIM, DIR>;
     constexpr int NV = SM::NV, NQ = SM::NQ, NX = SM::NX, SEG = SM::SEG, NF = SM::NF, NC = SM::NC;
-    constexpr int QC = SM::QC, NUF = SM::NUF, NRB = SM::NRB, NFD = SM::NFD, NFS = SM::NFS, NPB = SM::NPB;
+    constexpr int QC = SM::QC, QB = SM::QB, NUF = SM::NUF, NRB = SM::NRB, NFD = SM::NFD, NFS = SM::NFS, NPB = SM::NPB;
     constexpr int NT = kVjpWenoThreads, LINES = VjpTile<T, DIM, DIR>::LINES, LAST = NV - 1;
     T* cq = reinterpret_cast<T*>(smem_raw);   // [NQ + NX][NC]
     T* wq = cq + (NQ + NX) * NC;              // [NV][NC] cotangent
-    T* UF = wq + NV * NC;                     // [NF][6][NUF] projections of U and F, then their bars
-    T* FD = UF + NF * 6 * NUF;                // [NF][NFD]
-    T* FS = FD + NF * NFD;                    // [NF][NFS]
-    T* DB = FS + NF * NFS;                    // [NF][NV] bars of the detector difference
-    T* RB = DB + NF * NV;                     // [NF][2][NRB] Roe-field bars of cells 2 and 3
-    T* SP = RB + NF * 2 * NRB;                // [NF][3] speed bars
-    T* XB = SP + NF * 3;                      // [QC][NV][2][6] bars of f+-
+    T* FD = wq + NV * NC;                     // [NF][NFD]
+    T* UF = FD + NF * NFD;                    // [QB][6][NUF] projections of U and F, then their bars
+    T* FS = UF + QB * 6 * NUF;                // [QB][NFS]
+    T* DB = FS + QB * NFS;                    // [QB][NV] bars of the detector difference
+    T* RB = DB + QB * NV;                     // [QB][2][NRB] Roe-field bars of cells 2 and 3
+    T* SP = RB + QB * 2 * NRB;                // [QB][3] speed bars
+    T* XB = SP + QB * 3;                      // [QC][NV][2][6] bars of f+-
     T* LF = XB + QC * NV * 2 * 6;             // [QC][NV][2][2] bar of lambda^s, reconstructed value
     T* PB = LF + QC * NV * 2 * 2;             // [QC][6][NPB] per-cell parts of the face sums
     int* SL = reinterpret_cast<int*>(PB + QC * 6 * NPB);   // [NF] slots attaining the speeds
     int* queue = SL + NF;
-    __shared__ int qcount;
-    constexpr int SKIP = 1 << 12;
+    __shared__ int wcount[NT / 32];
+    constexpr int SKIP = 1 << 12;             // no WENO face; otherwise its place in the queue from bit 13 on
+    static_assert(NF <= NT, "one face per thread");
 
     const int nd = a.n[DIR], c0 = bx * SEG;
     int ix = 0, j = 0, k = 0;
@@ -757,7 +775,6 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
     const T* Ug = reinterpret_cast<const T*>(a.U);
     const T* Wg = reinterpret_cast<const T*>(a.W);
     const T gamma = pick<T>(a.gamma, a.gamma_f), gm1 = gamma - T(1);
-    if (threadIdx.x == 0) qcount = 0;
 
     // ---- cells c0 - 5 .. c0 + SEG + 4 that exist
     for (int p = threadIdx.x; p < NC; p += NT) {
@@ -783,10 +800,11 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
     // ---- WENO faces: the forward quantities of the whole face
     const T lam_k = pick<T>(a.lam_k, a.lam_k_f), eps = pick<T>(a.eps, a.eps_f);
     const T inv_dx = pick<T>(a.inv_dx, a.inv_dx_f), slim = pick<T>(a.slim, a.slim_f);
-    for (int f = threadIdx.x; f < NF; f += NT) {
+    const int myf = threadIdx.x;
+    int slots = SKIP;
+    auto face_data = [&](int f) {
         const int face = c0 - 2 + f;
-        SL[f] = SKIP;
-        if (face < 0 || face > nd) continue;
+        if (f >= NF || face < 0 || face > nd) return;
         auto rec = [&](int m, int kk) -> T { return cq[kk * NC + f + m]; };
         auto ga = [&](int kk) -> T { return rec(2, kk); };
         auto gb = [&](int kk) -> T { return rec(3, kk); };
@@ -800,9 +818,25 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
         proj_all<T, DIM, DIR>(r, dU, w);
         const T lim = slim * r.rt;
         bool smooth = a.hybrid != 0;
+        if (sizeof(T) == 8 && a.fx) {
+            // the flag is pass 0's; the weights keep the FP64 form of the
+            // detector (their derivative amplifies its rounding where a
+            // field's own data are smooth)
+            T dx[NV], wx[NV];
 #pragma unroll
-        for (int s = 0; s < NV; ++s) smooth = smooth && abs_lt(w[s], lim);
-        if (smooth) continue;   // pass 0 took this face
+            for (int v = 0; v < NV; ++v) {
+                const int kk = CL::U + v;
+                const double x[6] = {rec(0, kk), rec(1, kk), rec(2, kk), rec(3, kk), rec(4, kk), rec(5, kk)};
+                dx[v] = T(fx_detector(x));
+            }
+            proj_all<T, DIM, DIR>(r, dx, wx);
+#pragma unroll
+            for (int s = 0; s < NV; ++s) smooth = smooth && abs_lt(wx[s], lim);
+        } else {
+#pragma unroll
+            for (int s = 0; s < NV; ++s) smooth = smooth && abs_lt(w[s], lim);
+        }
+        if (smooth) return;   // pass 0 took this face
         T am = rec(0, CL::LM), a0 = rec(0, CL::L0), ap = rec(0, CL::LP);
         int im = 0, i0 = 0, ip = 0;
 #pragma unroll
@@ -812,7 +846,7 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
             if (lt_nn(a0, x0)) { a0 = x0; i0 = m; }
             if (lt_nn(ap, xp)) { ap = xp; ip = m; }
         }
-        SL[f] = im | (i0 << 4) | (ip << 8);
+        slots = im | (i0 << 4) | (ip << 8);
         T* fd = FD + f * NFD;
 #pragma unroll
         for (int kk = 0; kk < DIM; ++kk) fd[SM::U + kk] = r.u[kk];
@@ -842,201 +876,220 @@ __device__ __forceinline__ void vjp_weno_line(const VjpArgs& a, int bx, int by, 
             ++s;
         }
         fd[SM::WCB + LAST] = eh + difb;
-        queue[atomicAdd(&qcount, 1)] = f;
+    };
+    face_data(myf);
+    // the queue in face order
+    const unsigned int mine = __ballot_sync(0xffffffffu, slots != SKIP);
+    if ((threadIdx.x & 31) == 0) wcount[threadIdx.x >> 5] = __popc(mine);
+    __syncthreads();
+    int nq = 0, pos = __popc(mine & ((1u << (threadIdx.x & 31)) - 1u));
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+        if (w < (int)(threadIdx.x >> 5)) pos += wcount[w];
+        nq += wcount[w];
     }
+    if (slots != SKIP) queue[pos] = myf;
+    if (myf < NF) SL[myf] = slots == SKIP ? SKIP : slots | (pos << 13);
     __syncthreads();
 
-    const int nq = qcount;
     auto load_roe = [&](const T* fd, Roe<T, DIM>& r) {
 #pragma unroll
         for (int kk = 0; kk < DIM; ++kk) r.u[kk] = fd[SM::U + kk];
         r.c = fd[SM::C]; r.ic = fd[SM::IC]; r.H = fd[SM::H]; r.b1 = fd[SM::B1]; r.hq2 = fd[SM::HQ2]; r.rt = fd[SM::RT];
     };
-    for (int q0 = 0; q0 < nq; q0 += QC) {
-        const int qc = nq - q0 < QC ? nq - q0 : QC;
-        // projections of U_m and F_m (Eq. eqchara)
-        for (int it = threadIdx.x; it < qc * 6; it += NT) {
-            const int f = queue[q0 + it / 6], m = it % 6;
-            Roe<T, DIM> r;
-            load_roe(FD + f * NFD, r);
-            T xu[NV], xf[NV], vv[NV], gg[NV];
+    // the cell whose bars this thread gathers
+    static_assert(SEG + 6 <= NT, "one cell per thread");
+    const bool first = c0 == 0, last = c0 + SEG >= nd;
+    const int cell = c0 - 3 + (int)threadIdx.x;
+    const bool owned = cell >= c0 && cell < c0 + SEG && cell < nd;
+    const bool gl = first && cell < 0 && cell >= -3;
+    const bool gr = last && cell >= nd && cell <= nd + 2;
+    const bool gathers = (int)threadIdx.x < SEG + 6 && (owned || gl || gr);
+    bool touched = false;
+    T qb[NQ];
 #pragma unroll
-            for (int v = 0; v < NV; ++v) { xu[v] = cq[(CL::U + v) * NC + f + m]; xf[v] = cq[(CL::F + v) * NC + f + m]; }
-            proj_all<T, DIM, DIR>(r, xu, vv);
-            proj_all<T, DIM, DIR>(r, xf, gg);
-            T* uf = UF + (f * 6 + m) * NUF;
+    for (int kk = 0; kk < NQ; ++kk) qb[kk] = T(0);
+    for (int b0 = 0; b0 < nq; b0 += QB) {
+        const int qn = nq - b0 < QB ? nq : b0 + QB;
+        for (int q0 = b0; q0 < qn; q0 += QC) {
+            const int qc = qn - q0 < QC ? qn - q0 : QC;
+            // projections of U_m and F_m (Eq. eqchara)
+            for (int it = threadIdx.x; it < qc * 6; it += NT) {
+                const int f = queue[q0 + it / 6], m = it % 6, e = q0 - b0 + it / 6;
+                Roe<T, DIM> r;
+                load_roe(FD + f * NFD, r);
+                T xu[NV], xf[NV], vv[NV], gg[NV];
 #pragma unroll
-            for (int s = 0; s < NV; ++s) { uf[s] = vv[s]; uf[NV + s] = gg[s]; }
-        }
-        __syncthreads();
-        // reconstructions and their reverse; the minus part on the mirrored
-        // stencil m = 5 .. 1
-        for (int it = threadIdx.x; it < qc * NV * 2; it += NT) {
-            const int q = it / (2 * NV), rem = it - q * 2 * NV, s = rem >> 1, sg = rem & 1;
-            const int f = queue[q0 + q];
-            const T* fd = FD + f * NFD;
-            const T al = fd[SM::AL + (s == 0 ? 0 : (s == LAST ? 2 : 1))];
-            const T ws = fd[SM::W + s], lam = lam_k * (ws * ws) * fd[SM::IRT2];
-            const T ha = sg ? T(-0.5) * al : T(0.5) * al;
-            T x[5], xb[5], lb;
+                for (int v = 0; v < NV; ++v) { xu[v] = cq[(CL::U + v) * NC + f + m]; xf[v] = cq[(CL::F + v) * NC + f + m]; }
+                proj_all<T, DIM, DIR>(r, xu, vv);
+                proj_all<T, DIM, DIR>(r, xf, gg);
+                T* uf = UF + (e * 6 + m) * NUF;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) {
-                const T* uf = UF + (f * 6 + (sg ? 5 - i : i)) * NUF + s;
-                x[i] = fmaT(ha, uf[0], T(0.5) * uf[NV]);
+                for (int s = 0; s < NV; ++s) { uf[s] = vv[s]; uf[NV + s] = gg[s]; }
             }
-            const T val = recon_adj<T>(x[0], x[1], x[2], x[3], x[4], lam, eps, fd[SM::WCB + s], xb, lb);
-            T* o = XB + ((q * NV + s) * 2 + sg) * 6;
+            __syncthreads();
+            // reconstructions and their reverse; the minus part on the mirrored
+            // stencil m = 5 .. 1
+            for (int it = threadIdx.x; it < qc * NV * 2; it += NT) {
+                const int q = it / (2 * NV), rem = it - q * 2 * NV, s = rem >> 1, sg = rem & 1;
+                const int f = queue[q0 + q];
+                const T* fd = FD + f * NFD;
+                const T al = fd[SM::AL + (s == 0 ? 0 : (s == LAST ? 2 : 1))];
+                const T ws = fd[SM::W + s], lam = lam_k * (ws * ws) * fd[SM::IRT2];
+                const T ha = sg ? T(-0.5) * al : T(0.5) * al;
+                T x[5], xb[5], lb;
 #pragma unroll
-            for (int i = 0; i < 5; ++i) o[sg ? 5 - i : i] = xb[i];
-            o[sg ? 0 : 5] = T(0);
-            LF[((q * NV + s) * 2 + sg) * 2] = lb;
-            LF[((q * NV + s) * 2 + sg) * 2 + 1] = val;
+                for (int i = 0; i < 5; ++i) {
+                    const T* uf = UF + ((q0 - b0 + q) * 6 + (sg ? 5 - i : i)) * NUF + s;
+                    x[i] = fmaT(ha, uf[0], T(0.5) * uf[NV]);
+                }
+                const T val = recon_adj<T>(x[0], x[1], x[2], x[3], x[4], lam, eps, fd[SM::WCB + s], xb, lb);
+                T* o = XB + ((q * NV + s) * 2 + sg) * 6;
+#pragma unroll
+                for (int i = 0; i < 5; ++i) o[sg ? 5 - i : i] = xb[i];
+                o[sg ? 0 : 5] = T(0);
+                LF[((q * NV + s) * 2 + sg) * 2] = lb;
+                LF[((q * NV + s) * 2 + sg) * 2 + 1] = val;
+            }
+            __syncthreads();
+            // splitting and projections in reverse, per stencil cell
+            for (int it = threadIdx.x; it < qc * 6; it += NT) {
+                const int q = it / 6, m = it - q * 6, f = queue[q0 + q];
+                const T* fd = FD + f * NFD;
+                Roe<T, DIM> r;
+                load_roe(fd, r);
+                T* uf = UF + ((q0 - b0 + q) * 6 + m) * NUF;
+                T vb[NV], gb[NV], alb[3] = {T(0), T(0), T(0)};
+#pragma unroll
+                for (int s = 0; s < NV; ++s) {
+                    const T fp = XB[((q * NV + s) * 2) * 6 + m], fm = XB[((q * NV + s) * 2 + 1) * 6 + m];
+                    const int as = s == 0 ? 0 : (s == LAST ? 2 : 1);
+                    const T d = T(0.5) * (fp - fm);
+                    gb[s] = T(0.5) * (fp + fm);
+                    vb[s] = fd[SM::AL + as] * d;
+                    alb[as] = fmaT(uf[s], d, alb[as]);
+                }
+                RoeBar<T, DIM> rb;
+                zero(rb);
+                T x[NV], xb[NV];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) { x[v] = cq[((h ? CL::F : CL::U) + v) * NC + f + m]; xb[v] = T(0); }
+                    proj_all_adj<T, DIM, DIR>(r, x, h ? gb : vb, xb, rb);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) uf[h * NV + v] = xb[v];
+                }
+                T* o = PB + it * NPB;
+#pragma unroll
+                for (int kk = 0; kk < DIM; ++kk) o[kk] = rb.u[kk];
+                o[DIM] = rb.ic; o[DIM + 1] = rb.b1; o[DIM + 2] = rb.hq2;
+#pragma unroll
+                for (int i = 0; i < 3; ++i) o[DIM + 3 + i] = alb[i];
+            }
+            __syncthreads();
+            // sums over the cells and over the signs
+            for (int it = threadIdx.x; it < qc * NFS; it += NT) {
+                const int q = it / NFS, c = it - q * NFS;
+                T sum;
+                if (c < NPB) {
+                    const T* o = PB + q * 6 * NPB + c;
+                    sum = o[0];
+#pragma unroll
+                    for (int m = 1; m < 6; ++m) sum += o[m * NPB];
+                } else {
+                    const int s = (c - NPB) % NV, w = (c - NPB) / NV;
+                    const T* o = LF + (q * NV + s) * 4 + w;
+                    sum = o[0] + o[2];
+                }
+                FS[(q0 - b0 + q) * NFS + c] = sum;
+            }
         }
         __syncthreads();
-        // splitting and projections in reverse, per stencil cell
-        for (int it = threadIdx.x; it < qc * 6; it += NT) {
-            const int q = it / 6, m = it - q * 6, f = queue[q0 + q];
-            const T* fd = FD + f * NFD;
+
+        // ---- per face: weights' parameter, detector, back-projection and Roe average in reverse
+        for (int e = threadIdx.x; e < qn - b0; e += NT) {
+            const int f = queue[b0 + e];
+            const T *fd = FD + f * NFD, *fs = FS + e * NFS, *lb = fs + NPB, *wch = lb + NV;
             Roe<T, DIM> r;
             load_roe(fd, r);
-            T* uf = UF + (f * 6 + m) * NUF;
-            T vb[NV], gb[NV], alb[3] = {T(0), T(0), T(0)};
-#pragma unroll
-            for (int s = 0; s < NV; ++s) {
-                const T fp = XB[((q * NV + s) * 2) * 6 + m], fm = XB[((q * NV + s) * 2 + 1) * 6 + m];
-                const int as = s == 0 ? 0 : (s == LAST ? 2 : 1);
-                const T d = T(0.5) * (fp - fm);
-                gb[s] = T(0.5) * (fp + fm);
-                vb[s] = fd[SM::AL + as] * d;
-                alb[as] = fmaT(uf[s], d, alb[as]);
-            }
             RoeBar<T, DIM> rb;
             zero(rb);
-            T x[NV], xb[NV];
+            const T sum = wch[0] + wch[1] + wch[LAST], dif = wch[LAST] - wch[0], oE = fd[SM::PHI + LAST];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+            for (int kk = 0; kk < DIM; ++kk) rb.u[kk] = fmaT(fd[SM::PHI + 1 + kk], sum, fs[kk]);
+            rb.c = fmaT(oE, r.u[DIR], fd[SM::PHI + 1 + DIR]) * dif;
+            rb.u[DIR] = fmaT(oE * r.c, dif, rb.u[DIR]);
+            int s = 2;
 #pragma unroll
-                for (int v = 0; v < NV; ++v) { x[v] = cq[((h ? CL::F : CL::U) + v) * NC + f + m]; xb[v] = T(0); }
-                proj_all_adj<T, DIM, DIR>(r, x, h ? gb : vb, xb, rb);
-#pragma unroll
-                for (int v = 0; v < NV; ++v) uf[h * NV + v] = xb[v];
+            for (int kk = 0; kk < DIM; ++kk) {
+                if (kk == DIR) continue;
+                rb.u[kk] = fmaT(oE, wch[s], rb.u[kk]);
+                ++s;
             }
-            T* o = PB + it * NPB;
-#pragma unroll
-            for (int kk = 0; kk < DIM; ++kk) o[kk] = rb.u[kk];
-            o[DIM] = rb.ic; o[DIM + 1] = rb.b1; o[DIM + 2] = rb.hq2;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) o[DIM + 3 + i] = alb[i];
-        }
-        __syncthreads();
-        // sums over the cells and over the signs
-        for (int it = threadIdx.x; it < qc * NFS; it += NT) {
-            const int q = it / NFS, c = it - q * NFS;
-            T sum;
-            if (c < NPB) {
-                const T* o = PB + q * 6 * NPB + c;
-                sum = o[0];
-#pragma unroll
-                for (int m = 1; m < 6; ++m) sum += o[m * NPB];
-            } else {
-                const int s = (c - NPB) % NV, w = (c - NPB) / NV;
-                const T* o = LF + (q * NV + s) * 4 + w;
-                sum = o[0] + o[2];
-            }
-            FS[queue[q0 + q] * NFS + c] = sum;
-        }
-    }
-    __syncthreads();
-
-    // ---- per face: weights' parameter, detector, back-projection and Roe average in reverse
-    for (int q = threadIdx.x; q < nq; q += NT) {
-        const int f = queue[q];
-        const T *fd = FD + f * NFD, *fs = FS + f * NFS, *lb = fs + NPB, *wch = lb + NV;
-        Roe<T, DIM> r;
-        load_roe(fd, r);
-        RoeBar<T, DIM> rb;
-        zero(rb);
-        const T sum = wch[0] + wch[1] + wch[LAST], dif = wch[LAST] - wch[0], oE = fd[SM::PHI + LAST];
-#pragma unroll
-        for (int kk = 0; kk < DIM; ++kk) rb.u[kk] = fmaT(fd[SM::PHI + 1 + kk], sum, fs[kk]);
-        rb.c = fmaT(oE, r.u[DIR], fd[SM::PHI + 1 + DIR]) * dif;
-        rb.u[DIR] = fmaT(oE * r.c, dif, rb.u[DIR]);
-        int s = 2;
-#pragma unroll
-        for (int kk = 0; kk < DIM; ++kk) {
-            if (kk == DIR) continue;
-            rb.u[kk] = fmaT(oE, wch[s], rb.u[kk]);
-            ++s;
-        }
-        rb.H = oE * (wch[0] + wch[LAST]);
-        rb.ic = fs[DIM];
-        rb.b1 = fs[DIM + 1];
-        rb.hq2 = fmaT(oE, wch[1], fs[DIM + 2]);
-        // lam = c w^2 / (3600 rt^2)
-        const T irt2 = fd[SM::IRT2], irt = irt2 * r.rt;
-        T wb[NV], dUb[NV], dU[NV];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            const T w = fd[SM::W + v], lw = lam_k * w * irt2;
-            wb[v] = lb[v] * (lw + lw);
-            rb.rt = fmaT(lb[v], T(-2) * (lw * w) * irt, rb.rt);
-            dU[v] = fd[SM::DU + v];
-            dUb[v] = T(0);
-        }
-        proj_all_adj<T, DIM, DIR>(r, dU, wb, dUb, rb);
-#pragma unroll
-        for (int v = 0; v < NV; ++v) DB[f * NV + v] = dUb[v];
-#pragma unroll
-        for (int i = 0; i < 3; ++i) SP[f * 3 + i] = fs[DIM + 3 + i];
-        T* RBf = RB + f * 2 * NRB;
-        T ra[NRB], rbb[NRB];
-#pragma unroll
-        for (int kk = 0; kk < NRB; ++kk) ra[kk] = rbb[kk] = T(0);
-        roe_adj<T, DIM>([&](int kk) -> T { return cq[kk * NC + f + 2]; }, [&](int kk) -> T { return cq[kk * NC + f + 3]; },
-                        gamma, r, rb, ra, rbb);
-#pragma unroll
-        for (int kk = 0; kk < NRB; ++kk) { RBf[kk] = ra[kk]; RBf[NRB + kk] = rbb[kk]; }
-    }
-    __syncthreads();
-
-    // ---- gather per cell, as in pass 0
-    T* Gg = reinterpret_cast<T*>(a.G);
-    T* ghost = reinterpret_cast<T*>(a.ghost);
-    const bool first = c0 == 0, last = c0 + SEG >= nd;
-    for (int p = threadIdx.x; p < SEG + 6; p += NT) {
-        const int cell = c0 - 3 + p;
-        const bool owned = cell >= c0 && cell < c0 + SEG && cell < nd;
-        const bool gl = first && cell < 0 && cell >= -3;
-        const bool gr = last && cell >= nd && cell <= nd + 2;
-        if (!owned && !gl && !gr) continue;
-        T qb[NQ];
-#pragma unroll
-        for (int kk = 0; kk < NQ; ++kk) qb[kk] = T(0);
-        bool touched = false;
-        constexpr T cd[6] = {T(1), T(-5), T(10), T(-10), T(5), T(-1)};
-#pragma unroll
-        for (int m = 5; m >= 0; --m) {
-            const int f = cell - m + 3 - (c0 - 2);   // faces in increasing order
-            if (f < 0 || f >= NF) continue;
-            const int sl = SL[f];
-            if (sl & SKIP) continue;
-            touched = true;
-            const T* uf = UF + (f * 6 + m) * NUF;
+            rb.H = oE * (wch[0] + wch[LAST]);
+            rb.ic = fs[DIM];
+            rb.b1 = fs[DIM + 1];
+            rb.hq2 = fmaT(oE, wch[1], fs[DIM + 2]);
+            // lam = c w^2 / (3600 rt^2)
+            const T irt2 = fd[SM::IRT2], irt = irt2 * r.rt;
+            T wb[NV], dUb[NV], dU[NV];
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
-                qb[CL::U + v] += fmaT(cd[m], DB[f * NV + v], uf[v]);
-                qb[CL::F + v] += uf[NV + v];
+                const T w = fd[SM::W + v], lw = lam_k * w * irt2;
+                wb[v] = lb[v] * (lw + lw);
+                rb.rt = fmaT(lb[v], T(-2) * (lw * w) * irt, rb.rt);
+                dU[v] = fd[SM::DU + v];
+                dUb[v] = T(0);
             }
-            if (m == 2 || m == 3) {
-                const T* rbp = RB + (f * 2 + (m - 2)) * NRB;
+            proj_all_adj<T, DIM, DIR>(r, dU, wb, dUb, rb);
 #pragma unroll
-                for (int kk = 0; kk < NRB; ++kk) qb[CL::SU + kk] += rbp[kk];
-            }
-            if ((sl & 15) == m) qb[CL::LM] += SP[f * 3 + 0];
-            if (((sl >> 4) & 15) == m) qb[CL::L0] += SP[f * 3 + 1];
-            if (((sl >> 8) & 15) == m) qb[CL::LP] += SP[f * 3 + 2];
+            for (int v = 0; v < NV; ++v) DB[e * NV + v] = dUb[v];
+#pragma unroll
+            for (int i = 0; i < 3; ++i) SP[e * 3 + i] = fs[DIM + 3 + i];
+            T* RBf = RB + e * 2 * NRB;
+            T ra[NRB], rbb[NRB];
+#pragma unroll
+            for (int kk = 0; kk < NRB; ++kk) ra[kk] = rbb[kk] = T(0);
+            roe_adj<T, DIM>([&](int kk) -> T { return cq[kk * NC + f + 2]; }, [&](int kk) -> T { return cq[kk * NC + f + 3]; },
+                            gamma, r, rb, ra, rbb);
+#pragma unroll
+            for (int kk = 0; kk < NRB; ++kk) { RBf[kk] = ra[kk]; RBf[NRB + kk] = rbb[kk]; }
         }
-        if (!touched) continue;
+        __syncthreads();
+
+        // ---- gather per cell, as in pass 0, faces in increasing order
+        if (gathers) {
+            constexpr T cd[6] = {T(1), T(-5), T(10), T(-10), T(5), T(-1)};
+#pragma unroll
+            for (int m = 5; m >= 0; --m) {
+                const int f = cell - m + 3 - (c0 - 2);
+                if (f < 0 || f >= NF) continue;
+                const int sl = SL[f];
+                const int e = (sl >> 13) - b0;
+                if ((sl & SKIP) || e < 0 || e >= QB) continue;
+                touched = true;
+                const T* uf = UF + (e * 6 + m) * NUF;
+#pragma unroll
+                for (int v = 0; v < NV; ++v) {
+                    qb[CL::U + v] += fmaT(cd[m], DB[e * NV + v], uf[v]);
+                    qb[CL::F + v] += uf[NV + v];
+                }
+                if (m == 2 || m == 3) {
+                    const T* rbp = RB + (e * 2 + (m - 2)) * NRB;
+#pragma unroll
+                    for (int kk = 0; kk < NRB; ++kk) qb[CL::SU + kk] += rbp[kk];
+                }
+                if ((sl & 15) == m) qb[CL::LM] += SP[e * 3 + 0];
+                if (((sl >> 4) & 15) == m) qb[CL::L0] += SP[e * 3 + 1];
+                if (((sl >> 8) & 15) == m) qb[CL::LP] += SP[e * 3 + 2];
+            }
+        }
+        __syncthreads();   // the next batch reuses shared memory
+    }
+    T* Gg = reinterpret_cast<T*>(a.G);
+    T* ghost = reinterpret_cast<T*>(a.ghost);
+    if (touched) {
         const int pc = cell - (c0 - 5);
         T U[NV], Ub[NV];
 #pragma unroll

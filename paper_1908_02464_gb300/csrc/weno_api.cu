@@ -832,6 +832,7 @@ weno_status weno_rhs_vjp(weno_ctx* ctx, const void* U_dev, const void* w_dev, vo
         a.slim = std::sqrt(3600.0 * a.eps_h);
         a.gamma = ctx->p.gamma; a.eps = ctx->p.eps; a.c_lambda = ctx->p.c_lambda; a.hybrid = ctx->p.hybrid;
         a.lam_k = a.c_lambda / 3600.0;
+        a.fx = f64 && wis::use_fx((long long)interior_cells(ctx)) ? 1 : 0;
         a.inv_dx_f = (float)a.inv_dx; a.gamma_f = (float)a.gamma; a.eps_f = (float)a.eps; a.slim_f = (float)a.slim;
         a.lam_k_f = (float)a.lam_k;
         a.bc = sweep_args(ctx, d);
