@@ -65,6 +65,7 @@ struct weno_batch {
     wis::BatchInst* inst = nullptr;
     double* t_end = nullptr;
     void* work[4] = {nullptr, nullptr, nullptr, nullptr};   // the fourth: 2D accumulator
+    void* prim = nullptr;           // 2D FP64: cell primitives
     unsigned char* run = nullptr;   // BatchCtrl, the BatchState of every instance, the task queue
     size_t run_bytes = 0;
     long long places = 0;           // of the queue: the tiles of all instances
@@ -121,6 +122,7 @@ static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_ba
     b.U = U;
     for (int k = 0; k < 3; ++k) b.work[k] = bt->work[k];
     b.acc = bt->work[3];
+    b.prim = bt->prim;
     b.status = bt->status; b.steps = bt->steps; b.t_out = bt->t_out;
     b.weno_count = bt->wcount;
     b.max_steps = max_steps;
@@ -172,7 +174,7 @@ static cudaError_t enqueue_run(weno_batch* bt, void* U, int max_steps, int write
 static void batch_free(weno_batch* bt)
 {
     if (bt->graph) cudaGraphExecDestroy(bt->graph);
-    void* ptrs[] = {bt->order, bt->inst, bt->t_end, bt->work[0], bt->work[1], bt->work[2], bt->work[3], bt->run,
+    void* ptrs[] = {bt->order, bt->inst, bt->t_end, bt->work[0], bt->work[1], bt->work[2], bt->work[3], bt->prim, bt->run,
                     bt->status, bt->steps, bt->t_out, bt->wcount, bt->trial_caps};
     for (void* q : ptrs)
         if (q) cudaFree(q);
@@ -228,6 +230,8 @@ static cudaError_t batch_setup(weno_batch* bt, const int* nx, const int* ny, con
     alloc((void**)&bt->inst, sizeof(wis::BatchInst) * cnt);
     alloc((void**)&bt->t_end, sizeof(double) * cnt);
     for (int k = 0; k < (bt->dim == 2 ? 4 : 3); ++k) alloc(&bt->work[k], bt->esz * (size_t)bt->total);
+    if (bt->dim == 2 && bt->prec == WENO_FP64)
+        alloc(&bt->prim, bt->esz * (size_t)(bt->total / nv) * wis::PrimLayout<2>::STRIDE);
     alloc((void**)&bt->run, bt->run_bytes);
     alloc((void**)&bt->status, sizeof(int) * cnt);
     alloc((void**)&bt->steps, sizeof(long long) * cnt);

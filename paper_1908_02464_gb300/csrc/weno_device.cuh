@@ -232,7 +232,7 @@ __device__ __forceinline__ void load_prims(const double* P, long long g, double*
     const double2* p = reinterpret_cast<const double2*>(P + g * PrimLayout<DIM>::STRIDE);
 #pragma unroll
     for (int j = 0; j < PrimLayout<DIM>::STRIDE / 2; ++j) {
-        const double2 v = __ldg(p + j);
+        const double2 v = p[j];   // plain loads: a batch kernel reads what other CTAs stored
         if (2 * j < PrimLayout<DIM>::NP) out[2 * j] = v.x;
         if (2 * j + 1 < PrimLayout<DIM>::NP) out[2 * j + 1] = v.y;
     }
@@ -243,7 +243,7 @@ __device__ __forceinline__ void load_prims(const float* P, long long g, float* o
     const float4* p = reinterpret_cast<const float4*>(P + g * PrimLayout<DIM>::STRIDE);
 #pragma unroll
     for (int j = 0; j < PrimLayout<DIM>::STRIDE / 4; ++j) {
-        const float4 v = __ldg(p + j);
+        const float4 v = p[j];
         const float w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int k = 0; k < 4; ++k)

@@ -243,7 +243,6 @@ __device__ __forceinline__ void stage_record(const SweepArgs& a, const T* Ug, co
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[v] = Ug[g + v * a.sv];
     if (Pg != nullptr) {
-#pragma unroll
         load_prims<DIM>(Pg, g, P);
     } else {
         cell_prims<T, DIM>(U, gamma, gm1, P);
