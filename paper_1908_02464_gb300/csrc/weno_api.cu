@@ -376,11 +376,18 @@ static int default_tile(const weno_ctx* c, int d)
     }
     if (d == 0) return n >= wis::Tile<5>::SEG || per_line(31, 4) >= per_line(127, 1) ? 5 : 2;
     // Across x, 4 x 31: four x-adjacent lines share the 32-byte sectors of the
-    // strided loads (256^3: y 3524 -> 3130, z 4046 -> 3933; 637 x 159: y 46.6
-    // -> 39.1).  A 2D grid with fewer such tiles than the chip holds CTAs is
-    // bound by the time of one tile, which is shorter for the flat ones
-    // (512 x 128: 39.1 against 44.8, 177 x 70: 23 against 34).
-    const long long tiles = (long long)((c->n[0] + 3) / 4) * ((n + 30) / 31) * (c->dim == 3 ? c->n[3 - d] : 1);
+    // strided loads (256^3: y 3524 -> 3130, z 4046 -> 3933).
+    if (c->dim == 3) return 2;
+    // In 2D the flat tiles of long lines win or tie (RK3 steps of 2048 x 512
+    // 1707 against 1732, 1000 x 250 540 against 590); 4 x 31 wins on shorter
+    // ones (637 x 159: 290 against 306, 1651 x 135: y-sweep 76 against 85)
+    // unless the grid has fewer such tiles than the chip holds CTAs, where the
+    // time of one tile counts (512 x 128: 304 against 283); and on lines that
+    // leave most of a one-line tile empty (700 x 45: 119 against 171) unless
+    // even the one-line tiles are too few (177 x 70: 168 against 134).
+    const long long tiles = (long long)((c->n[0] + 3) / 4) * ((n + 30) / 31);
+    if (n < wis::Tile<5>::SEG) return c->n[0] > 2 * c->nsm && per_line(31, 4) < 0.8 ? 2 : 5;
+    if (n >= 192) return 5;
     return tiles > 5LL * c->nsm ? 2 : 5;
 }
 
