@@ -17,18 +17,15 @@
 namespace wis {
 
 // Line tiles on 128, 64 and 256 threads (LineTile).  1024 Riemann problems of
-// 100 to 2000 cells in FP64: 64, 68 and 65 ms, with the FP64 pipe 85% busy
+// 100 to 2000 cells in FP64: 63, 68 and 61 ms, with the FP64 pipe 85% busy
 // over the first steps (one CTA per instance: 125, 192 and 75 ms, the
 // heaviest instance alone 80 ms against 12 ms here); 4096 of 100 to 4000
-// cells in FP32: 147, 146 and 167 ms (231, 380 and 146 ms), issue 56% of the
-// cycles and the shared-memory data path 67%.  128 threads are the default.
-// Runs of 8 tiles: with single-tile tasks and a lane-by-lane queue the FP32
-// batch took 202 ms.
+// cells in FP32: 123, 142 and 129 ms (231, 380 and 146 ms).  128 threads are
+// the default.
 template <int V>
 struct Batch1Cfg {
     static constexpr int NT = V == 0 ? 128 : (V == 1 ? 64 : 256);
     static constexpr int XS = NT - 6, XL = 1, YL = 1, YS = 1;
-    static constexpr int RUN = 8;
     template <typename T> static constexpr size_t smem_bytes() { return LineTile<T, NT>::bytes; }
     template <typename T> static constexpr int min_blocks() { return (sizeof(T) == 8 ? 640 : 1024) / NT; }
 };
@@ -117,7 +114,6 @@ static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_ba
     b.state = reinterpret_cast<wis::BatchState*>(bt->run + kCtrlBytes);
     b.queue = reinterpret_cast<wis::BatchTask*>(bt->run + kCtrlBytes + sizeof(wis::BatchState) * (size_t)bt->count);
     b.places = bt->places;
-    b.total_tiles = bt->tiles_of[bt->variant];
     b.t_end = bt->t_end;
     b.U = U;
     for (int k = 0; k < 3; ++k) b.work[k] = bt->work[k];

@@ -12,7 +12,10 @@ namespace wis {
 // sweeps.  Batched instances have short lines (tens of cells), so the tiles
 // hold several lines; the y tiles hold 8 or 4 x-adjacent columns, so that
 // their loads are row pieces.  1024 explosions in FP64: 59, 57 and 60 ms (one
-// CTA per instance: 103, 106 and 150 ms).
+// CTA per instance: 103, 106 and 150 ms); with the primitives shared between
+// the sweeps the first takes 55 ms.  4096 boxes of 16 to 64 cells a side in
+// FP32: 70, 72 and 94 ms with 16 warps per SM (64 registers a thread; 112 to 124
+// registers and half as many warps took half as long again).
 template <int V> struct Batch2Shape;
 template <> struct Batch2Shape<0> { static constexpr int NT = 128, XL = 4, XS = 31, YL = 8, YS = 15; };
 template <> struct Batch2Shape<1> { static constexpr int NT = 128, XL = 2, XS = 63, YL = 4, YS = 31; };
@@ -21,13 +24,12 @@ template <> struct Batch2Shape<2> { static constexpr int NT = 64, XL = 2, XS = 3
 template <int V>
 struct Batch2Cfg : Batch2Shape<V> {
     using S = Batch2Shape<V>;
-    static constexpr int RUN = 4;
     template <typename T> static constexpr size_t smem_bytes()
     {
         constexpr size_t x = SweepSmem<T, 2, S::XL, S::XS>::bytes, y = SweepSmem<T, 2, S::YL, S::YS>::bytes;
         return x > y ? x : y;
     }
-    template <typename T> static constexpr int min_blocks() { return S::NT == 64 ? 8 : 4; }
+    template <typename T> static constexpr int min_blocks() { return (sizeof(T) == 8 ? 512 : 1024) / S::NT; }
 };
 
 cudaError_t batch2d_config(int prec, bool fx, int v, int* blocks_per_sm, size_t* smem)
