@@ -53,10 +53,21 @@ struct Run1DSmem {
                                     sizeof(int) * (size_t)NFACE;
 };
 
+// by every thread of the CTA; the aligned forms want a converged warp
+__device__ __forceinline__ void cluster_arrive()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait()
+{
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_barrier()
 {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 
 template <typename T, bool EXACTDET>
@@ -119,7 +130,10 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
         cluster_barrier();
     };
 
-    // the state, and its CFL wave speeds
+    // The state, and its CFL wave speeds.  A CTA may store to another's shared
+    // memory (the first tell) only once that CTA has started: every CTA says so
+    // here, and the loads of the state cover the wait.
+    cluster_arrive();
     if (tid == 0) s_bad = 0;
     __syncthreads();
     {
@@ -133,6 +147,7 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
             if (!cell_speed<T, 1>(u, gamma, inv_dx1, sp)) cbad = true;
             else smax = max_nn(smax, sp);
         }
+        cluster_wait();
         tell(false, cbad, smax);
     }
 
