@@ -304,6 +304,12 @@ weno_status weno_batch_autotune(weno_batch* batch, const void* U_dev, int trial_
  * variant outside 0..2 or a negative blocks_per_sm. */
 weno_status weno_batch_set_config(weno_batch* batch, int variant, int blocks_per_sm, int* blocks);
 
+/* CTAs that a run launches, in place of those that fit the GPU at once (0:
+ * these again).  Any number gives the same results: a run is finished by
+ * whichever of its CTAs are running.  WENO_ERR_INVALID_ARG for a negative
+ * number. */
+weno_status weno_batch_set_launch(weno_batch* batch, int ctas);
+
 /* Number of faces computed with the WENO (non-linear) flux by the batch's
  * runs (autotuner trial runs included) since creation or the last call with
  * reset != 0; a face counts once per RK stage.  Synchronizes. */

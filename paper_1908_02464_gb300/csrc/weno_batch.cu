@@ -75,8 +75,10 @@ struct weno_batch {
     std::vector<int> n_host;      // steps grow with this size: n (1D), max(nx, ny) (2D)
     bool fx = false;              // an FP64 instance takes the integer six-point sums
     int variant = 0;
+    int residency = 0;            // most CTAs per SM, 0 = as many as fit
     int blocks = 0;               // reported: min(count, residency x SMs)
-    int grid = 0;                 // CTAs launched: min(tiles, residency x SMs)
+    int grid = 0;                 // CTAs launched: min(tiles, residency x SMs), or ctas
+    int ctas = 0;                 // weno_batch_set_launch
     cudaGraphExec_t graph = nullptr;
     void* graph_U = nullptr;
     std::string err;
@@ -141,9 +143,10 @@ static weno_status set_variant(weno_batch* bt, int v, int blocks_per_sm_cap)
     if (bps < 1) { bt->err = "batch kernel cannot be resident"; return WENO_ERR_CUDA; }
     if (blocks_per_sm_cap > 0 && bps > blocks_per_sm_cap) bps = blocks_per_sm_cap;
     bt->variant = v;
+    bt->residency = blocks_per_sm_cap;
     const long long resident = (long long)bps * bt->nsm;
     bt->blocks = (int)std::min<long long>(resident, bt->count);
-    bt->grid = (int)std::min<long long>(resident, bt->tiles_of[v]);
+    bt->grid = bt->ctas > 0 ? bt->ctas : (int)std::min<long long>(resident, bt->tiles_of[v]);
     if (bt->graph) cudaGraphExecDestroy(bt->graph);
     bt->graph = nullptr;
     return WENO_OK;
@@ -466,6 +469,17 @@ weno_status weno_batch_set_config(weno_batch* bt, int variant, int blocks_per_sm
     const weno_status st = set_variant(bt, variant, blocks_per_sm);
     if (st == WENO_OK && blocks) *blocks = bt->blocks;
     return st;
+}
+
+weno_status weno_batch_set_launch(weno_batch* bt, int ctas)
+{
+    if (!bt) return WENO_ERR_INVALID_ARG;
+    if (ctas < 0) {
+        bt->err = "set_launch: negative number of CTAs";
+        return WENO_ERR_INVALID_ARG;
+    }
+    bt->ctas = ctas;
+    return set_variant(bt, bt->variant, bt->residency);
 }
 
 weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_steps, int* choice)

@@ -2,15 +2,16 @@
 // weno_batch2d.cu): many independent Euler problems of uneven sizes, each
 // advanced to its own end time with its own CFL step.
 //
-// One launch of resident CTAs works through a queue of tasks.  A task is a
-// run of consecutive tiles of one sweep of one instance.  The CTA that
+// One launch of CTAs works through a queue of tasks.  A task is a run of
+// consecutive tiles of one sweep of one instance.  The CTA that
 // finishes the last run of a sweep goes on with the instance's next sweep,
 // putting parts of it into the queue when other CTAs have nothing to do, and
 // after the last sweep of a step (Sec. 4 of the paper) it also advances the
 // instance's time and takes the next CFL step.  Instances wait
 // only for their own previous sweep.  A CTA without a task polls its place in
-// the queue; it holds nothing that another CTA waits for, so the polls end
-// whichever CTAs are resident.
+// the queue; it holds nothing that another CTA waits for, and a CTA that does
+// not run yet holds nothing at all (instances to prepare come from a counter,
+// tasks from the queue), so the polls end whichever CTAs are resident.
 //
 // What bounds it: the FP64 pipe (FP64), instruction issue and shared-memory
 // loads (FP32).  In the first form of this solver one CTA integrated one
@@ -69,6 +70,7 @@ struct BatchCtrl {
     unsigned long long head;           // places taken by CTAs
     unsigned long long tail;           // tasks put into the queue
     unsigned long long sweeps;         // of all instances so far
+    unsigned int prepared;             // instances taken for preparation
     int finished;                      // instances
     int abort;                         // a wait for a task ran out
 };
@@ -323,8 +325,13 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
         return done == 2;
     };
 
-    // initial states, and their CFL wave speeds
-    for (int k = blockIdx.x; k < b.count; k += gridDim.x) {
+    // Initial states, and their CFL wave speeds.  The instances come from a
+    // counter, so that only a running CTA holds one that is not in the queue yet.
+    for (;;) {
+        if (threadIdx.x == 0) s_inst = (int)atomicAdd(&b.ctrl->prepared, 1u);
+        __syncthreads();
+        const unsigned int k = (unsigned int)s_inst;
+        if (k >= (unsigned int)b.count) break;
         const int inst = b.order[k];
         const BatchInst q = b.inst[inst];
         const long long cells = (long long)q.nx * q.ny;
@@ -346,6 +353,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
         note_cfl(b.state[inst], m, bad);
         next_sweep(inst, true);
     }
+    __syncthreads();   // every thread has read s_inst
 
     int inst = -1, run = 0;
     bool go_on = false;

@@ -94,6 +94,7 @@ SIGNATURES = {
     "weno_batch_results": (ctypes.c_int, [_vp, ctypes.POINTER(_ip), ctypes.POINTER(ctypes.c_longlong), _dp]),
     "weno_batch_weno_face_count": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_ulonglong), _ip]),
     "weno_batch_set_config": (ctypes.c_int, [_vp, _ip, _ip, ctypes.POINTER(ctypes.c_int)]),
+    "weno_batch_set_launch": (ctypes.c_int, [_vp, _ip]),
     "weno_batch_autotune": (ctypes.c_int, [_vp, _vp, _ip, ctypes.POINTER(_ip)]),
     "weno_batch_destroy": (None, [_vp]),
     "weno_batch_last_error": (ctypes.c_char_p, [_vp]),
@@ -543,6 +544,10 @@ class Batch:
         _bcheck(load().weno_batch_set_config(self.handle, int(variant), int(blocks_per_sm), ctypes.byref(b)),
                 self.handle)
         return b.value
+
+    def set_launch(self, ctas: int = 0) -> None:
+        """CTAs of a run (0: as many as the GPU holds at once)."""
+        _bcheck(load().weno_batch_set_launch(self.handle, int(ctas)), self.handle)
 
     def weno_faces(self, reset: bool = False) -> int:
         c = ctypes.c_ulonglong(0)

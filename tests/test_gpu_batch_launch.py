@@ -1,0 +1,76 @@
+"""The batch kernel's waits: launches with fewer and with more CTAs than the
+GPU holds at once (the others start when some have left, as they do beside
+another stream's kernels).  Every instance must carry the single solver's bits
+(no tolerance)."""
+import numpy as np
+import pytest
+
+from paper_1908_02464_gb300 import problems as P
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # pragma: no cover
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from paper_1908_02464_gb300 import weno  # noqa: E402
+
+
+def _line_batch(count, precision="fp64", t_end=0.02):
+    n = [40 + 17 * (i % 60) for i in range(count)]
+    states = [P.riemann_1d(k, (1.0, 0.1, 1.0), (0.3, 0.0, 0.2), t_end) for k in n]
+    b = weno.Batch(n, 0.0, 1.0, [t_end] * count, precision, max_steps=12)
+    return b, [U for _, U in states], states
+
+
+def _run(b, states):
+    D = b.pack(states)
+    b.run(D)
+    st, steps, t = b.results()
+    return D.cpu().numpy(), st, steps, t
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("ctas", [1, 3, 20000])
+def test_lines_with_any_number_of_ctas(ctas, precision):
+    b, states, probs = _line_batch(240, precision)
+    A = _run(b, states)
+    b.set_launch(ctas)
+    B = _run(b, states)
+    b.set_launch(0)
+    C = _run(b, states)
+    for x, y, z in zip(A, B, C):
+        assert np.array_equal(x, y) and np.array_equal(x, z)
+    assert np.all(A[1] == 0) and np.all(A[2] > 0)
+    prob, U = probs[137]
+    s = weno.Solver(prob, precision)
+    s.set_state(U)
+    s.advance(0.02, 12)
+    V, _ = s.get_state()
+    s.close()
+    o = b.offsets
+    assert np.array_equal(B[0][o[137]:o[138]].reshape(3, -1), V)
+    b.close()
+
+
+@pytest.mark.parametrize("ctas", [1, 20000])
+def test_boxes_with_any_number_of_ctas(ctas):
+    nx = [10 + 7 * (i % 9) for i in range(60)]
+    ny = [9 + 5 * (i % 11) for i in range(60)]
+    states = [P.random_state(2, [a, b], 70 + i, "smooth")[1] for i, (a, b) in enumerate(zip(nx, ny))]
+    b = weno.Batch2D(nx, ny, (0.0, 0.0), (1.0, 1.0), [0.02] * 60, "fp64", bc_lo=(2, 2), bc_hi=(2, 2), max_steps=4)
+    A = _run(b, states)
+    b.set_launch(ctas)
+    B = _run(b, states)
+    for x, y in zip(A, B):
+        assert np.array_equal(x, y)
+    assert np.all(A[1] == 0) and np.all(A[2] > 0)
+    b.close()
+
+
+def test_a_negative_number_of_ctas_is_refused():
+    b, _, _ = _line_batch(2)
+    with pytest.raises(weno.WenoError) as e:
+        b.set_launch(-1)
+    assert e.value.status == weno.WENO_ERR_INVALID_ARG
+    b.close()

@@ -36,3 +36,12 @@ def test_one_launch_stepping_waits_for_its_cluster_before_the_first_remote_store
     assert "cluster_barrier()" in before or before.rfind("cluster_wait()") > before.find("cluster_arrive()") >= 0
     # and no CTA leaves while another may still read its shared memory
     assert body.rindex("cluster_barrier()") > body.rindex("tell(")
+
+
+def test_batch_ctas_that_do_not_run_yet_hold_no_instance():
+    """A CTA leaves the batch kernel only when every instance has finished, so
+    no instance may wait for a CTA that is not running: instances are taken
+    from counters, never by the CTA's index."""
+    body = _body(_source("weno_batch.cuh"), "k_batch(BatchArgs b)")
+    assert "blockIdx" not in body and "gridDim" not in body
+    assert re.search(r"atomicAdd\(&b\.ctrl->prepared", body)
