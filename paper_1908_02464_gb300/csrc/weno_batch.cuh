@@ -309,6 +309,9 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             }
             nr = __shfl_sync(0xffffffffu, nr, 0);
             at = __shfl_sync(0xffffffffu, at, 0);
+            // the shuffles order no memory: the tasks that the other lanes
+            // publish come after lane 0's stores, and the stores it acquired
+            __syncwarp();
             if (nr > 0) batch_put(b, inst, first ? 0 : 1, nr, at);
         }
         __syncthreads();

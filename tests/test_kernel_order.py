@@ -45,3 +45,12 @@ def test_batch_ctas_that_do_not_run_yet_hold_no_instance():
     body = _body(_source("weno_batch.cuh"), "k_batch(BatchArgs b)")
     assert "blockIdx" not in body and "gridDim" not in body
     assert re.search(r"atomicAdd\(&b\.ctrl->prepared", body)
+
+
+def test_tasks_are_published_after_the_first_lanes_stores():
+    """Lane 0 acquires the other CTAs' stores and writes the instance's
+    progress, the other lanes of its warp publish tasks too: a barrier that
+    orders memory stands between (a shuffle does not)."""
+    body = _body(_source("weno_batch.cuh"), "k_batch(BatchArgs b)")
+    progress, put = body.index("batch_next_sweep<"), body.index("batch_put(")
+    assert "__syncwarp()" in body[progress:put] or "__syncthreads()" in body[progress:put]
