@@ -310,6 +310,11 @@ weno_status weno_batch_set_config(weno_batch* batch, int variant, int blocks_per
  * number. */
 weno_status weno_batch_set_launch(weno_batch* batch, int ctas);
 
+/* Polls that a CTA without a task makes, while no instance finishes a sweep,
+ * before the run ends with WENO_ERR_TIMEOUT (0: the default, some seconds).
+ * WENO_ERR_INVALID_ARG for a negative number. */
+weno_status weno_batch_set_wait(weno_batch* batch, int polls);
+
 /* Number of faces computed with the WENO (non-linear) flux by the batch's
  * runs (autotuner trial runs included) since creation or the last call with
  * reset != 0; a face counts once per RK stage.  Synchronizes. */

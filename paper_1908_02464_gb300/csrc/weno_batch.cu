@@ -79,6 +79,7 @@ struct weno_batch {
     int blocks = 0;               // reported: min(count, residency x SMs)
     int grid = 0;                 // CTAs launched: min(tiles, residency x SMs), or ctas
     int ctas = 0;                 // weno_batch_set_launch
+    int polls = wis::kTaskPolls;  // weno_batch_set_wait
     cudaGraphExec_t graph = nullptr;
     void* graph_U = nullptr;
     std::string err;
@@ -124,6 +125,7 @@ static BatchArgs batch_args(weno_batch* bt, void* U, int max_steps, int write_ba
     b.status = bt->status; b.steps = bt->steps; b.t_out = bt->t_out;
     b.weno_count = bt->wcount;
     b.max_steps = max_steps;
+    b.polls = bt->polls;
     b.write_back = write_back;
     b.gamma = bt->p.gamma; b.cfl = bt->p.cfl; b.eps = bt->p.eps; b.c_lambda = bt->p.c_lambda;
     b.gamma_f = (float)bt->p.gamma;
@@ -480,6 +482,19 @@ weno_status weno_batch_set_launch(weno_batch* bt, int ctas)
     }
     bt->ctas = ctas;
     return set_variant(bt, bt->variant, bt->residency);
+}
+
+weno_status weno_batch_set_wait(weno_batch* bt, int polls)
+{
+    if (!bt) return WENO_ERR_INVALID_ARG;
+    if (polls < 0) {
+        bt->err = "set_wait: negative number of polls";
+        return WENO_ERR_INVALID_ARG;
+    }
+    bt->polls = polls > 0 ? polls : wis::kTaskPolls;
+    if (bt->graph) cudaGraphExecDestroy(bt->graph);   // it holds the old number
+    bt->graph = nullptr;
+    return WENO_OK;
 }
 
 weno_status weno_batch_autotune(weno_batch* bt, const void* U_dev, int trial_steps, int* choice)

@@ -93,6 +93,7 @@ struct BatchArgs {
     double* t_out;
     unsigned long long* weno_count;
     int max_steps;
+    int polls;                   // of a wait before it runs out (kTaskPolls)
     const int* trial_caps;       // autotuner trial runs: step cap per instance (null otherwise)
     int write_back;              // 0: trial run, the caller's states are not touched
     double gamma, cfl, eps, c_lambda;
@@ -103,7 +104,7 @@ struct BatchArgs {
 
 // polls of a CTA for its next task, while no instance finishes a sweep, before
 // it gives up (about 100 ns each: some seconds, where the longest sweep of a
-// batch takes milliseconds)
+// batch takes milliseconds); weno_batch_set_wait sets another number
 constexpr int kTaskPolls = 1 << 26;
 
 // tiles of nx x ny cells along direction d
@@ -228,10 +229,16 @@ __device__ __forceinline__ void batch_put(const BatchArgs& b, int inst, int r0, 
     for (int r = r0 + (int)(threadIdx.x & 31); r < nr; r += 32) {
         const unsigned long long k = at + (unsigned long long)(r - r0), turn = k / places;
         BatchTask* q = b.queue + (long long)(k - turn * places);
-        for (int w = 0; w < kTaskPolls; ++w) {
+        bool free = false;
+        for (int w = 0; w < b.polls && !free; ++w) {
             unsigned int v;
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&q->taken) : "memory");
-            if (v == (unsigned int)turn || *(volatile int*)&b.ctrl->abort != 0) break;
+            free = v == (unsigned int)turn;
+            if (!free && *(volatile int*)&b.ctrl->abort != 0) return;
+        }
+        if (!free) {   // the place still holds a task that nobody has read
+            atomicExch(&b.ctrl->abort, 1);
+            return;
         }
         q->inst = inst;
         q->run = r;
@@ -254,7 +261,7 @@ __device__ __forceinline__ bool batch_take(const BatchArgs& b, int& inst, int& r
         if (v == (unsigned int)turn + 1u) break;
         if ((k & 7) == 7) {
             if (*(volatile int*)&b.ctrl->finished >= b.count || *(volatile int*)&b.ctrl->abort != 0) return false;
-            if (k >= kTaskPolls) {
+            if (k >= b.polls) {
                 const unsigned long long now = *(volatile unsigned long long*)&b.ctrl->sweeps;
                 if (now == sweeps) {
                     atomicExch(&b.ctrl->abort, 1);

@@ -95,6 +95,7 @@ SIGNATURES = {
     "weno_batch_weno_face_count": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_ulonglong), _ip]),
     "weno_batch_set_config": (ctypes.c_int, [_vp, _ip, _ip, ctypes.POINTER(ctypes.c_int)]),
     "weno_batch_set_launch": (ctypes.c_int, [_vp, _ip]),
+    "weno_batch_set_wait": (ctypes.c_int, [_vp, _ip]),
     "weno_batch_autotune": (ctypes.c_int, [_vp, _vp, _ip, ctypes.POINTER(_ip)]),
     "weno_batch_destroy": (None, [_vp]),
     "weno_batch_last_error": (ctypes.c_char_p, [_vp]),
@@ -548,6 +549,10 @@ class Batch:
     def set_launch(self, ctas: int = 0) -> None:
         """CTAs of a run (0: as many as the GPU holds at once)."""
         _bcheck(load().weno_batch_set_launch(self.handle, int(ctas)), self.handle)
+
+    def set_wait(self, polls: int = 0) -> None:
+        """Polls of a CTA without a task before the run gives up (0: the default)."""
+        _bcheck(load().weno_batch_set_wait(self.handle, int(polls)), self.handle)
 
     def weno_faces(self, reset: bool = False) -> int:
         c = ctypes.c_ulonglong(0)

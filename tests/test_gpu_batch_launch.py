@@ -1,6 +1,6 @@
 """The batch kernel's waits: launches with fewer and with more CTAs than the
 GPU holds at once (the others start when some have left, as they do beside
-another stream's kernels).  Every instance must carry the single solver's bits
+another stream's kernels), and waits that run out.  Every instance must carry the single solver's bits
 (no tolerance)."""
 import numpy as np
 import pytest
@@ -74,3 +74,33 @@ def test_a_negative_number_of_ctas_is_refused():
         b.set_launch(-1)
     assert e.value.status == weno.WENO_ERR_INVALID_ARG
     b.close()
+
+
+@pytest.mark.parametrize("dim", [1, 2])
+def test_a_wait_that_runs_out_is_reported_and_the_next_run_is_good(dim):
+    """One instance of many tiles: one CTA prepares it for hundreds of
+    microseconds while the others give up after a few polls."""
+    if dim == 1:
+        prob, U = P.riemann_1d(20000, (1.0, 0.1, 1.0), (0.3, 0.0, 0.2), 0.02)
+        make = lambda: weno.Batch([20000], 0.0, 1.0, [0.02], "fp64", max_steps=3)
+    else:
+        prob, U = P.random_state(2, [200, 190], 9, "smooth")
+        make = lambda: weno.Batch2D([200], [190], (0.0, 0.0), (1.0, 1.0), [0.02], "fp64", bc_lo=(2, 2), bc_hi=(2, 2),
+                                    max_steps=3)
+    b, fresh = make(), make()
+    good = _run(fresh, [U])
+    assert good[2][0] == 3
+    b.set_wait(1)
+    D = b.pack([U])
+    b.run(D)
+    with pytest.raises(weno.WenoError) as e:
+        b.results()
+    assert e.value.status == weno.WENO_ERR_TIMEOUT
+    b.set_wait(0)
+    for x, y in zip(_run(b, [U]), good):
+        assert np.array_equal(x, y)
+    with pytest.raises(weno.WenoError) as e:
+        b.set_wait(-1)
+    assert e.value.status == weno.WENO_ERR_INVALID_ARG
+    b.close()
+    fresh.close()

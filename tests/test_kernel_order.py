@@ -54,3 +54,12 @@ def test_tasks_are_published_after_the_first_lanes_stores():
     body = _body(_source("weno_batch.cuh"), "k_batch(BatchArgs b)")
     progress, put = body.index("batch_next_sweep<"), body.index("batch_put(")
     assert "__syncwarp()" in body[progress:put] or "__syncthreads()" in body[progress:put]
+
+
+def test_a_place_of_the_queue_is_not_filled_while_its_task_is_unread():
+    """When the wait for a place runs out, the run ends; the task that nobody
+    has read is not overwritten."""
+    body = _body(_source("weno_batch.cuh"), "void batch_put(")
+    out = body.index("atomicExch(&b.ctrl->abort")
+    assert body.index("q->taken") < out < body.index("q->inst = inst")
+    assert "return" in body[out:body.index("q->inst = inst")]
