@@ -310,7 +310,7 @@ weno_status weno_batch_set_config(weno_batch* batch, int variant, int blocks_per
  * number. */
 weno_status weno_batch_set_launch(weno_batch* batch, int ctas);
 
-/* Polls that a CTA without a task makes, while no instance finishes a sweep,
+/* Polls that a CTA without a task makes, while no other makes progress,
  * before the run ends with WENO_ERR_TIMEOUT (0: the default, some seconds).
  * WENO_ERR_INVALID_ARG for a negative number. */
 weno_status weno_batch_set_wait(weno_batch* batch, int polls);

@@ -69,7 +69,7 @@ struct BatchTask {
 struct BatchCtrl {
     unsigned long long head;           // places taken by CTAs
     unsigned long long tail;           // tasks put into the queue
-    unsigned long long sweeps;         // of all instances so far
+    unsigned long long progress;       // sweeps of all instances so far, and parts of long ones
     unsigned int prepared;             // instances taken for preparation
     int finished;                      // instances
     int abort;                         // a wait for a task ran out
@@ -102,10 +102,13 @@ struct BatchArgs {
     int bc_lo[2], bc_hi[2];
 };
 
-// polls of a CTA for its next task, while no instance finishes a sweep, before
-// it gives up (about 100 ns each: some seconds, where the longest sweep of a
-// batch takes milliseconds); weno_batch_set_wait sets another number
+// polls of a CTA for its next task, while no other makes progress, before it
+// gives up (some seconds at 100 ns each); weno_batch_set_wait sets another number
 constexpr int kTaskPolls = 1 << 26;
+// A sweep that is one run (every CTA had work when it began) of an instance of
+// millions of cells can outlast those polls: a run counts as progress every
+// kBeat tiles (about a millisecond), and so do the copies of the states.
+constexpr int kBeat = 32;
 
 // tiles of nx x ny cells along direction d
 template <typename CFG>
@@ -189,7 +192,7 @@ __device__ bool batch_next_sweep(const BatchArgs& b, int inst, bool first, int& 
 {
     BatchState& s = b.state[inst];
     const int nx = b.inst[inst].nx, ny = b.inst[inst].ny;
-    atomicAdd(&b.ctrl->sweeps, 1ull);
+    atomicAdd(&b.ctrl->progress, 1ull);
     if (!first && s.phase + 1 < 3 * DIM) {
         s.phase += 1;
     } else {
@@ -254,7 +257,7 @@ __device__ __forceinline__ bool batch_take(const BatchArgs& b, int& inst, int& r
     const unsigned long long at = atomicAdd(&b.ctrl->head, 1ull);
     const unsigned long long turn = at / (unsigned long long)b.places;
     BatchTask* q = b.queue + (long long)(at - turn * (unsigned long long)b.places);
-    unsigned long long sweeps = 0ull;
+    unsigned long long seen = 0ull;
     for (int k = 0;; ++k) {
         unsigned int v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&q->turn) : "memory");
@@ -262,12 +265,12 @@ __device__ __forceinline__ bool batch_take(const BatchArgs& b, int& inst, int& r
         if ((k & 7) == 7) {
             if (*(volatile int*)&b.ctrl->finished >= b.count || *(volatile int*)&b.ctrl->abort != 0) return false;
             if (k >= b.polls) {
-                const unsigned long long now = *(volatile unsigned long long*)&b.ctrl->sweeps;
-                if (now == sweeps) {
+                const unsigned long long now = *(volatile unsigned long long*)&b.ctrl->progress;
+                if (now == seen) {
                     atomicExch(&b.ctrl->abort, 1);
                     return false;
                 }
-                sweeps = now;
+                seen = now;
                 k = 32;
             }
         }
@@ -295,6 +298,9 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
         const T m = warp_max_nn(smax);
         if (lane == 0 && m > T(0)) atomicMax(&s.smax, (unsigned long long)__double_as_longlong((double)m));
         if (bad) atomicOr(&s.bad, BAD_CFL);
+    };
+    auto beat = [&](long long i, long long every) {
+        if (threadIdx.x == 0 && i % every == every - 1) atomicAdd(&b.ctrl->progress, 1ull);
     };
     // the first warp queues the instance's next sweep; the states of a finished
     // instance go back to the caller.  Every thread calls it; the sweep's (or
@@ -327,7 +333,10 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             if (b.write_back) {
                 const BatchInst q = b.inst[inst];
                 const T* w = W[b.state[inst].cur] + q.off;
-                for (long long c = threadIdx.x; c < (long long)NV * q.nx * q.ny; c += NT) U[q.off + c] = w[c];
+                for (long long c = threadIdx.x; c < (long long)NV * q.nx * q.ny; c += NT) {
+                    U[q.off + c] = w[c];
+                    beat(c / NT, 64 * kBeat);
+                }
             }
             __syncthreads();
             if (threadIdx.x == 0) atomicAdd(&b.ctrl->finished, 1);
@@ -359,6 +368,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             }
             if (!cell_speed<T, DIM>(u, gamma, ih, sp)) bad = true;
             else m = max_nn(m, sp);
+            beat(c / NT, 16 * kBeat);
         }
         note_cfl(b.state[inst], m, bad);
         next_sweep(inst, true);
@@ -407,6 +417,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
                     const int lg = t / ns;
                     sweep_tile<T, DIM, 1, CFG::YL, CFG::YS, NT, EXACTDET, false, FX, true>(a, t - lg * ns, lg * CFG::YL,
                                                                                            0, T(0), smem_raw);
+                    beat(t - t0, kBeat);
                 }
             }
         } else {
@@ -430,9 +441,11 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             if constexpr (DIM == 1) {
                 T u[3];
                 line_load(a, t0 * CFG::XS, u);
-                for (int t = t0; t < t1; ++t)
+                for (int t = t0; t < t1; ++t) {
                     bad |= line_tile<T, NT, EXACTDET, FX>(a, t * CFG::XS, t + 1 < t1 ? (t + 1) * CFG::XS : -1, dt, u,
                                                           smem_raw, cp, wenos);
+                    beat(t - t0, kBeat);
+                }
             } else {
                 a.acc = reinterpret_cast<T*>(b.acc) + q.off;
                 a.acc_scale = q.inv_dx[1] * (1.0 / 60.0);   // the y sweep stores unscaled flux differences
@@ -443,6 +456,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
                     const int lg = t / ns;
                     bad |= sweep_tile<T, DIM, 0, CFG::XL, CFG::XS, NT, EXACTDET, false, FX>(a, t - lg * ns, lg * CFG::XL,
                                                                                             0, dt, smem_raw, cp);
+                    beat(t - t0, kBeat);
                 }
             }
             if (bad) atomicOr(&s.bad, BAD_STAGE);

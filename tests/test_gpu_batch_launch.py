@@ -104,3 +104,22 @@ def test_a_wait_that_runs_out_is_reported_and_the_next_run_is_good(dim):
     assert e.value.status == weno.WENO_ERR_INVALID_ARG
     b.close()
     fresh.close()
+
+
+def test_a_long_sweep_of_one_cta_is_progress():
+    """400000 cells beside thousands of short lines: every CTA has work when
+    the long line's first sweep begins, so one CTA takes it whole (some tens of
+    milliseconds) and the others wait for much longer than their polls."""
+    n = [400000] + [100] * 4000
+    b = weno.Batch(n, 0.0, 1.0, [1e-9] + [0.2] * 4000, "fp64")
+    long_U = P.riemann_1d(400000, (1.0, 0.1, 1.0), (0.3, 0.0, 0.2), 0.2)[1]
+    U = P.riemann_1d(100, (1.0, 0.1, 1.0), (0.3, 0.0, 0.2), 0.2)[1]
+    states = [long_U] + [U] * 4000
+    b.set_wait(10000)
+    A = _run(b, states)
+    assert np.all(A[1] == 0) and A[2][0] == 1 and np.all(A[2][1:] == A[2][1])
+    b.set_wait(0)
+    B = _run(b, states)
+    for x, y in zip(A, B):
+        assert np.array_equal(x, y)
+    b.close()
