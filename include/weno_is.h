@@ -356,8 +356,10 @@ typedef struct {
  * instances back to back, instance i as [4][ny[i]][nx[i]] (rho, rho u, rho v,
  * E; x fastest) starting at element 4 sum_{j<i} nx[j] ny[j] (double for
  * WENO_FP64, float otherwise).  Allocates four work arrays of the batch's
- * size, and in FP64 one of twice that size for the cell primitives.  Errors: WENO_ERR_INVALID_ARG for an empty batch, nx or ny < 3,
- * hi <= lo, negative t_end, other boundary codes, unpaired periodic
+ * size, and in FP64, where that leaves at least as much memory free, one of
+ * twice that size for the cell primitives (the results are the same without
+ * it).  Errors: WENO_ERR_INVALID_ARG for an empty batch, nx or ny < 3, hi <=
+ * lo, negative t_end, other boundary codes, unpaired periodic
  * boundaries or an unknown precision; WENO_ERR_UNSUPPORTED for global
  * Lax-Friedrichs splitting; WENO_ERR_CUDA if allocation fails. */
 weno_status weno_batch2d_create(const weno_batch2d_desc* desc, const weno_params* params, void* stream,

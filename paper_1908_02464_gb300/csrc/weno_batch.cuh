@@ -87,7 +87,8 @@ struct BatchArgs {
     void* U;
     void* work[3];               // two rotating states and the second stage
     void* acc;                   // 2D: divergence of the y sweep
-    void* prim;                  // 2D FP64: cell primitives of the stage's state (PrimLayout records)
+    void* prim;                  // 2D FP64: cell primitives of the stage's state (PrimLayout records);
+                                 // null: both sweeps compute them
     int* status;                 // per instance: 0 ok, WENO_ERR_NONPHYSICAL
     long long* steps;
     double* t_out;
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             a.acc = reinterpret_cast<T*>(b.acc) + q.off;
             // as in a step of the grid solver, the y sweep computes and stores
             // the cell primitives and the x sweep reads them
-            if (sizeof(T) == 8)
+            if (sizeof(T) == 8 && b.prim != nullptr)
                 a.Pout = reinterpret_cast<T*>(b.prim) + q.off / NV * PrimLayout<DIM>::STRIDE;
             const int t1 = min(t0 + len, batch_tiles<CFG>(DIM, q.nx, q.ny, 1)), ns = (q.ny + CFG::YS - 1) / CFG::YS;
             if constexpr (DIM == 2) {
@@ -450,7 +451,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
                 a.acc = reinterpret_cast<T*>(b.acc) + q.off;
                 a.acc_scale = q.inv_dx[1] * (1.0 / 60.0);   // the y sweep stores unscaled flux differences
                 a.acc_scale_f = q.inv_dx60_f[1];
-                if (sizeof(T) == 8) a.P = reinterpret_cast<const T*>(b.prim) + q.off / NV * PrimLayout<DIM>::STRIDE;
+                if (sizeof(T) == 8 && b.prim != nullptr) a.P = reinterpret_cast<const T*>(b.prim) + q.off / NV * PrimLayout<DIM>::STRIDE;
                 const int ns = (q.nx + CFG::XS - 1) / CFG::XS;
                 for (int t = t0; t < t1; ++t) {
                     const int lg = t / ns;

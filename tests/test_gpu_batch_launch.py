@@ -123,3 +123,30 @@ def test_a_long_sweep_of_one_cta_is_progress():
     for x, y in zip(A, B):
         assert np.array_equal(x, y)
     b.close()
+
+
+def test_boxes_fit_without_room_for_their_primitives():
+    """200 FP64 boxes whose work arrays fit the free memory (105 of 150 MB) and
+    whose cell primitives (52 MB) do not."""
+    n = [64] * 200
+    states = [P.random_state(2, [64, 64], 30 + i % 3, "smooth")[1] for i in range(200)]
+    make = lambda: weno.Batch2D(n, n, (0.0, 0.0), (1.0, 1.0), [0.02] * 200, "fp64", bc_lo=(2, 2), bc_hi=(2, 2),
+                                max_steps=3)
+    b = make()
+    A = _run(b, states)                            # also loads the kernel
+    b.close()
+    D = b.pack(states)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    fill = torch.empty(free - (150 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        c = make()
+        c.run(D)
+        st, steps, t = c.results()
+        c.close()
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    for x, y in zip(A, (D.cpu().numpy(), st, steps, t)):
+        assert np.array_equal(x, y)
