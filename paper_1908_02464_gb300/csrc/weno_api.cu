@@ -2,7 +2,8 @@
 // the RK3 step sequence and its CUDA-graph replay.
 //
 // Step sequence (one RK3 step, Sec. 4 of the paper) on three rotating state
-// buffers (cur, x, y) selected by phase = completed steps mod 3:
+// buffers (cur, x, y); phase is the one that holds the state, and every
+// completed step moves it on by one:
 //   stage 1: sweeps(cur)         -> x = cur + dt L(cur)
 //   stage 2: sweeps(x), base cur -> y = 3/4 cur + 1/4 (x + dt L(x))
 //   stage 3: sweeps(y), base cur -> x = 1/3 cur + 2/3 (y + dt L(y)); the last
@@ -66,7 +67,8 @@ struct weno_ctx {
     double* partial = nullptr;
     double* totals_dev = nullptr;
     int tot_blocks = 1;
-    int phase = 0;
+    int phase = 0;              // buffer of the state (DevTime::phase after a look at the time)
+    bool phase_ahead = false;   // steps were enqueued since: they may have stopped short of `phase`
     int tile[3] = {0, 0, 0};    // sweep tile variant per direction
     bool x_first = false;       // sweep order of a stage: x .. last instead of last .. x
     double smax_floor = 0.0;    // CFL wave-speed sum of the fixed boundary states
@@ -283,6 +285,12 @@ static wis::StepArgs step_args(const weno_ctx* c)
 // and dt towards the target time.
 static cudaError_t issue_begin(weno_ctx* c, int ph, cudaStream_t s)
 {
+    if (c->phase_ahead) {
+        const long long n = (long long)(c->buf_elems * c->esz / sizeof(uint4));   // rows are multiples of 32 elements
+        const cudaError_t e = wis::launch_pdl(wis::k_align, dim3(wis::grid_for(n, 256, c->nsm * 8)), dim3(256), 0, s, c->tm,
+                                              (uint4*)c->buf[0], (uint4*)c->buf[1], (uint4*)c->buf[2], n, ph % 3);
+        if (e != cudaSuccess) return e;
+    }
     wis::CflArgs ca;
     std::memset(&ca, 0, sizeof(ca));
     ca.U = c->buf[ph % 3];
@@ -292,7 +300,7 @@ static cudaError_t issue_begin(weno_ctx* c, int ph, cudaStream_t s)
     ca.tm = c->tm;
     cudaError_t e = do_cfl(c, ca, s);
     if (e != cudaSuccess) return e;
-    return wis::launch_pdl(wis::k_begin, dim3(1), dim3(32), 0, s, c->tm, step_args(c));
+    return wis::launch_pdl(wis::k_begin, dim3(1), dim3(32), 0, s, c->tm, step_args(c), ph % 3);
 }
 
 static cudaError_t issue_step(weno_ctx* c, int ph, cudaStream_t s)
@@ -349,7 +357,8 @@ static weno_status read_time(weno_ctx* ctx)
 {
     CK(cudaMemcpyAsync(ctx->tm_host, ctx->tm, sizeof(DevTime), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
-    ctx->phase = (int)(ctx->tm_host->steps % 3);
+    ctx->phase = ctx->tm_host->phase;
+    ctx->phase_ahead = false;
     return WENO_OK;
 }
 
@@ -662,6 +671,7 @@ weno_status weno_set_state(weno_ctx* ctx, const void* U, int on_device, double t
     CK(cudaMemcpyAsync(ctx->tm, ctx->tm_host, sizeof(DevTime), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->phase = 0;
+    ctx->phase_ahead = false;
     return WENO_OK;
 }
 
@@ -940,11 +950,12 @@ weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps)
     CK(cudaGetLastError());
     if (ctx->run1d) {
         if (nsteps > 0) CK(issue_run1d(ctx, nsteps, ctx->stream));
-    } else {
-        if (nsteps > 0) CK(issue_begin(ctx, ctx->phase, ctx->stream));
+    } else if (nsteps > 0) {
+        CK(issue_begin(ctx, ctx->phase, ctx->stream));
         for (int i = 0; i < nsteps; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
+        ctx->phase = (ctx->phase + nsteps % 3) % 3;
+        ctx->phase_ahead = true;
     }
-    ctx->phase = (ctx->phase + nsteps) % 3;
     return WENO_OK;
 }
 

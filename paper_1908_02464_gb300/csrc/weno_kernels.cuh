@@ -63,6 +63,7 @@ struct DevTime {
     int smax_valid;                 // smax_bits holds the current state's
     int cfl_bad;                    // a cell of the current state has no admissible wave speed
     long long steps;                // completed steps
+    int phase;                      // state buffer of the current state
     int status;                     // 0 ok, else WENO_ERR_NONPHYSICAL latched
     int clipped;                    // 1 if dt was clipped to reach t_end
     int go;                         // dt > 0 (float kernels keep off the FP64 pipe)
@@ -1115,11 +1116,29 @@ __device__ __forceinline__ void take_dt(DevTime* tm, const StepArgs& a)
     }
 }
 
-// before the first step of a call, after k_cfl (the target time may be new)
-static __global__ void k_begin(DevTime* tm, StepArgs a)
+// Before steps queued for a state in buffer `want`, if steps queued earlier may
+// have stopped short of the phase that the host counted them to (they do
+// nothing once their end time is reached): moves the state there.  k_begin
+// records it.
+static __global__ void __launch_bounds__(256) k_align(const DevTime* tm, uint4* b0, uint4* b1, uint4* b2, long long n,
+                                                      int want)
+{
+    pdl_enter();
+    const int have = tm->phase;
+    if (have == want) return;
+    const uint4* src = have == 0 ? b0 : (have == 1 ? b1 : b2);
+    uint4* dst = want == 0 ? b0 : (want == 1 ? b1 : b2);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+        dst[i] = src[i];
+}
+
+// before the first step of a call, after k_cfl (the target time may be new);
+// phase: the buffer of the current state
+static __global__ void k_begin(DevTime* tm, StepArgs a, int phase)
 {
     pdl_enter();
     if (threadIdx.x == 0) {
+        tm->phase = phase;
         if (tm->cfl_bad != 0) { tm->status = 1; tm->cfl_bad = 0; }
         tm->smax_valid = tm->status == 0;
         tm->smax_next = 0ull;
@@ -1144,6 +1163,7 @@ static __global__ void k_next(DevTime* tm, StepArgs a)
         if (tm->status == 0 && tm->go != 0) {
             tm->t = tm->clipped ? tm->t_end : tm->t + tm->dt;
             tm->steps += 1;
+            tm->phase = tm->phase == 2 ? 0 : tm->phase + 1;
             tm->smax_bits = tm->smax_next;
         } else {
             if (tm->status == 0 && tm->cfl_bad != 0) tm->status = 1;

@@ -29,7 +29,7 @@ namespace wis {
 
 struct Run1DArgs {
     SweepArgs a;            // constants and boundary conditions
-    void* buf[3];           // state buffers; the state is in steps mod 3
+    void* buf[3];           // state buffers; a step moves the state to the next one
     int nsteps;             // at most
     double cfl, smax_floor;
 };
@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
     const T inv_dx1[1] = {T(a.inv_dx)};
     const T slim = pick<T>(a.slim, a.slim_f);
     const long long steps0 = tm->steps;
+    const int phase0 = tm->phase;
     const double t_end = tm->t_end;
     const bool live = tm->status == 0;
     // time of the current state, kept by the last thread (its staging share is
@@ -137,7 +138,7 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
     if (tid == 0) s_bad = 0;
     __syncthreads();
     {
-        const T* p = reinterpret_cast<const T*>(r.buf[(int)(steps0 % 3)]) + a.off0 + lo;
+        const T* p = reinterpret_cast<const T*>(r.buf[phase0]) + a.off0 + lo;
         T smax = T(0);
         bool cbad = false;
         for (int i = tid; i < m; i += NT) {
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
     }
 
     if (live && done > 0) {
-        T* p = reinterpret_cast<T*>(r.buf[(int)((steps0 + done) % 3)]) + a.off0 + lo;
+        T* p = reinterpret_cast<T*>(r.buf[(phase0 + done) % 3]) + a.off0 + lo;
         for (int i = tid; i < m; i += NT)
 #pragma unroll
             for (int v = 0; v < NV; ++v) p[i + v * a.sv] = ub[(cur * NV + v) * M + i];
@@ -349,6 +350,7 @@ __global__ void __launch_bounds__(kRun1DThreads) k_run1d(Run1DArgs r)
     if (rank == 0 && tid == NT - 1 && live) {
         tm->t = t;
         tm->steps = steps0 + done;
+        tm->phase = (phase0 + done) % 3;
         tm->dt = 0.0;
         tm->clipped = clipped;
         if (status != 0) tm->status = 1;
