@@ -67,8 +67,8 @@ struct weno_ctx {
     double* partial = nullptr;
     double* totals_dev = nullptr;
     int tot_blocks = 1;
-    int phase = 0;              // buffer of the state (DevTime::phase after a look at the time)
-    bool phase_ahead = false;   // steps were enqueued since: they may have stopped short of `phase`
+    int phase = 0;              // buffer of the state; after steps enqueued since the last look at the
+                                // time, the one it is in unless they stopped short
     int tile[3] = {0, 0, 0};    // sweep tile variant per direction
     bool x_first = false;       // sweep order of a stage: x .. last instead of last .. x
     double smax_floor = 0.0;    // CFL wave-speed sum of the fixed boundary states
@@ -280,20 +280,16 @@ static wis::StepArgs step_args(const weno_ctx* c)
     return a;
 }
 
-// Before the first step of a call: the wave speeds of the current state,
-// unless the step that wrote it has left them (k_cfl returns at once then),
-// and dt towards the target time.
+// Before the first step of a call: the state in buffer ph (it is there unless
+// enqueued steps stopped short), its wave speeds, unless the step that wrote
+// it has left them (k_cfl returns at once then), and dt towards the target time.
 static cudaError_t issue_begin(weno_ctx* c, int ph, cudaStream_t s)
 {
-    if (c->phase_ahead) {
-        const long long n = (long long)(c->buf_elems * c->esz / sizeof(uint4));   // rows are multiples of 32 elements
-        const cudaError_t e = wis::launch_pdl(wis::k_align, dim3(wis::grid_for(n, 256, c->nsm * 8)), dim3(256), 0, s, c->tm,
-                                              (uint4*)c->buf[0], (uint4*)c->buf[1], (uint4*)c->buf[2], n, ph % 3);
-        if (e != cudaSuccess) return e;
-    }
     wis::CflArgs ca;
     std::memset(&ca, 0, sizeof(ca));
-    ca.U = c->buf[ph % 3];
+    for (int k = 0; k < 3; ++k) ca.buf[k] = c->buf[k];
+    ca.buf_vec = (long long)(c->buf_elems * c->esz / sizeof(uint4));   // rows are multiples of 32 elements
+    ca.want = ph % 3;
     for (int k = 0; k < 3; ++k) { ca.n[k] = c->n[k]; ca.inv_dx[k] = k < c->dim ? c->inv_dx[k] : 0.0; }
     ca.sy = c->sy; ca.sz = c->sz; ca.sv = c->sv; ca.off0 = c->off0;
     ca.gamma = c->p.gamma;
@@ -358,7 +354,6 @@ static weno_status read_time(weno_ctx* ctx)
     CK(cudaMemcpyAsync(ctx->tm_host, ctx->tm, sizeof(DevTime), cudaMemcpyDeviceToHost, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->phase = ctx->tm_host->phase;
-    ctx->phase_ahead = false;
     return WENO_OK;
 }
 
@@ -671,7 +666,6 @@ weno_status weno_set_state(weno_ctx* ctx, const void* U, int on_device, double t
     CK(cudaMemcpyAsync(ctx->tm, ctx->tm_host, sizeof(DevTime), cudaMemcpyHostToDevice, ctx->stream));
     CK(cudaStreamSynchronize(ctx->stream));
     ctx->phase = 0;
-    ctx->phase_ahead = false;
     return WENO_OK;
 }
 
@@ -954,7 +948,6 @@ weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps)
         CK(issue_begin(ctx, ctx->phase, ctx->stream));
         for (int i = 0; i < nsteps; ++i) CK(cudaGraphLaunch(ctx->graph[(ctx->phase + i) % 3], ctx->stream));
         ctx->phase = (ctx->phase + nsteps % 3) % 3;
-        ctx->phase_ahead = true;
     }
     return WENO_OK;
 }

@@ -972,6 +972,11 @@ struct CflArgs {
     double gamma;
     DevTime* tm;
     int parts;    // k_cfl: x-parts per grid row (rows x parts blocks of work)
+    // k_cfl, which reads the state from its buffer in place of U: the state
+    // buffers, their length in 16 bytes, and the buffer the next step reads
+    void* buf[3];
+    long long buf_vec;
+    int want;
 };
 
 template <typename T, int DIM>
@@ -979,8 +984,19 @@ __global__ void __launch_bounds__(256) k_cfl(CflArgs a)
 {
     pdl_enter();
     constexpr int NV = DIM + 2;
+    // Steps queued earlier may have stopped short of the phase that the host
+    // counted them to (they do nothing once their end time is reached): the
+    // state moves to the buffer that the steps to come start from.
+    const int have = a.tm->phase;
+    if (have != a.want) {
+        const uint4* src = reinterpret_cast<const uint4*>(a.buf[have]);
+        uint4* dst = reinterpret_cast<uint4*>(a.buf[a.want]);
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.buf_vec;
+             i += (long long)gridDim.x * blockDim.x)
+            dst[i] = src[i];
+    }
     if (a.tm->status != 0 || a.tm->smax_valid != 0) return;
-    const T* U = reinterpret_cast<const T*>(a.U);
+    const T* U = reinterpret_cast<const T*>(a.buf[have]);
     const int nx = a.n[0], ny = a.n[1];
     const long long rows = (long long)ny * a.n[2];
     const T gamma = T(a.gamma);
@@ -1114,22 +1130,6 @@ __device__ __forceinline__ void take_dt(DevTime* tm, const StepArgs& a)
             tm->top_line[lane] =
                 cells_below(dmr_shock_x(lane == 0 ? t : (lane == 1 ? t + dt : t + 0.5 * dt)), a.lo0, a.dx0, a.n0);
     }
-}
-
-// Before steps queued for a state in buffer `want`, if steps queued earlier may
-// have stopped short of the phase that the host counted them to (they do
-// nothing once their end time is reached): moves the state there.  k_begin
-// records it.
-static __global__ void __launch_bounds__(256) k_align(const DevTime* tm, uint4* b0, uint4* b1, uint4* b2, long long n,
-                                                      int want)
-{
-    pdl_enter();
-    const int have = tm->phase;
-    if (have == want) return;
-    const uint4* src = have == 0 ? b0 : (have == 1 ? b1 : b2);
-    uint4* dst = want == 0 ? b0 : (want == 1 ? b1 : b2);
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        dst[i] = src[i];
 }
 
 // before the first step of a call, after k_cfl (the target time may be new);
