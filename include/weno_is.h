@@ -199,8 +199,10 @@ weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps);
 
 /* Measurement helper (no counterpart in the paper): times `reps` launches of
  * the sweep kernel of every direction on the current state (ghosts filled at
- * the current time; the sweeps write the RHS accumulator only, the state is
- * not changed), each launch bracketed by CUDA events on the context's stream.
+ * the current time; each sweep does its part of a right-hand side, the state
+ * is not changed), each launch bracketed by CUDA events on the context's
+ * stream.  A 1D line that steps in one launch has no sweep
+ * kernels of its own in a step; the time is then that of weno_rhs.
  * If flush_dev is not NULL, flush_bytes of it are overwritten before every
  * launch (to evict L2).  ms[d] receives the mean launch time of direction d,
  * weno_faces[d] (if not NULL) the number of faces of one launch that took

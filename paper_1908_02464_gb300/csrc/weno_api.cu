@@ -952,8 +952,11 @@ weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps)
     return WENO_OK;
 }
 
-// mean event time of `reps` launches of the direction-d sweep (ACC_SET on the
-// current state at its time); weno faces of one launch to *wf
+// Mean event time of `reps` launches of the direction-d sweep on the current
+// state at its time, as a stage launches it: the first sweep of a stage sets
+// the accumulator, the last one reads it and writes a state (here to a buffer
+// that holds none between steps).  In float the first sweep has its own
+// instantiation.  Weno faces of one launch to *wf.
 static weno_status time_sweep_dir(weno_ctx* ctx, int d, int reps, void* flush_dev, size_t flush_bytes,
                                   cudaEvent_t e0, cudaEvent_t e1, double* ms, unsigned long long* wf)
 {
@@ -966,8 +969,15 @@ static weno_status time_sweep_dir(weno_ctx* ctx, int d, int reps, void* flush_de
         a.U = cur;
         set_time(ctx, a, ctx->tm_host->t);
         a.alpha_g = ctx->alpha_g + 3 * 9 + 3 * d;
-        a.mode = wis::MODE_ACC_SET;
-        a.acc = ctx->dim > 1 ? ctx->acc : ctx->rhs_out;
+        a.acc = ctx->dim > 1 ? ctx->acc : nullptr;
+        a.acc_scale = 0.0;   // a repeated accumulation does not grow
+        a.acc_scale_f = 0.0f;
+        if (d == sweep_dir(ctx, ctx->dim - 1)) {
+            a.mode = wis::MODE_RHS;
+            a.out = ctx->buf[(ctx->phase + 1) % 3];
+        } else {
+            a.mode = d == sweep_dir(ctx, 0) ? wis::MODE_ACC_SET : wis::MODE_ACC_ADD;
+        }
         CK(cudaEventRecord(e0, ctx->stream));
         CK(do_sweep(ctx, d, a, ctx->stream));
         CK(cudaEventRecord(e1, ctx->stream));
@@ -987,7 +997,6 @@ static weno_status prepare_timing(weno_ctx* ctx)
 {
     weno_status st = read_time(ctx);
     if (st != WENO_OK) return st;
-    if (ctx->dim == 1 && (st = ensure_rhs_bufs(ctx)) != WENO_OK) return st;
     void* cur = ctx->buf[ctx->phase];
     if (ctx->p.splitting == wis::SPLIT_LF) CK(issue_lf(ctx, cur, 3, nullptr, ctx->stream));
     if (ctx->use_prims) {
