@@ -428,6 +428,13 @@ weno_status weno_measure_fma_peak(int precision, double* flops, double* seconds)
  * null pointers with n > 0: WENO_ERR_INVALID_ARG.  Synchronizes the device. */
 weno_status weno_arith_selftest(const double* x_dev, long long n, double* out_dev);
 
+/* Diagnostic (no counterpart in the paper): the two six-point sums of the FP64
+ * sweeps in their integer form, for n stencils x_dev[n][6]: out_dev (device,
+ * 2 n doubles, caller-owned) receives [x0 - 5 x1 + 10 x2 - 10 x3 + 5 x4 - x5 |
+ * x0 - 8 x1 + 37 x2 + 37 x3 - 8 x4 + x5].  Errors as weno_arith_selftest.
+ * Synchronizes the device. */
+weno_status weno_sums_selftest(const double* x_dev, long long n, double* out_dev);
+
 #ifdef __cplusplus
 }
 #endif

@@ -1205,3 +1205,26 @@ extern "C" weno_status weno_arith_selftest(const double* x_dev, long long n, dou
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
     return e == cudaSuccess ? WENO_OK : WENO_ERR_CUDA;
 }
+
+__global__ void k_sums_selftest(const double* x, long long n, double* out)
+{
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
+         i += (long long)gridDim.x * blockDim.x) {
+        double v[6];
+        for (int k = 0; k < 6; ++k) v[k] = x[6 * i + k];
+        out[i] = wis::fx_detector(v);
+        out[n + i] = wis::fx_central_flux(v);
+    }
+}
+
+extern "C" weno_status weno_sums_selftest(const double* x_dev, long long n, double* out_dev)
+{
+    if (n < 0 || (n > 0 && (x_dev == nullptr || out_dev == nullptr))) return WENO_ERR_INVALID_ARG;
+    if (n == 0) return WENO_OK;
+    const long long want = (n + 255) / 256;
+    const int blocks = (int)(want < 4096 ? want : 4096);
+    k_sums_selftest<<<blocks, 256>>>(x_dev, n, out_dev);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    return e == cudaSuccess ? WENO_OK : WENO_ERR_CUDA;
+}

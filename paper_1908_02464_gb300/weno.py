@@ -84,6 +84,7 @@ SIGNATURES = {
     "weno_last_error": (ctypes.c_char_p, [_vp]),
     "weno_measure_fma_peak": (ctypes.c_int, [_ip, _dp, _dp]),
     "weno_arith_selftest": (ctypes.c_int, [_vp, ctypes.c_longlong, _vp]),
+    "weno_sums_selftest": (ctypes.c_int, [_vp, ctypes.c_longlong, _vp]),
     "weno_enqueue_steps": (ctypes.c_int, [_vp, ctypes.c_double, _ip]),
     "weno_autotune": (ctypes.c_int, [_vp, _ip, ctypes.POINTER(_ip)]),
     "weno_batch_create": (ctypes.c_int, [ctypes.POINTER(weno_batch_desc), ctypes.POINTER(weno_params), _vp,
@@ -236,6 +237,16 @@ def weno_arith_selftest(x_dev):
     x = x_dev.contiguous()
     out = torch.empty((4, x.numel()), dtype=torch.float64, device=x.device)
     _check(load().weno_arith_selftest(_vp(_ptr(x)), int(x.numel()), _vp(_ptr(out))))
+    return out
+
+
+def weno_sums_selftest(x_dev):
+    """[detector, central flux] six-point sums (integer form) of an (n, 6)
+    float64 CUDA tensor as a (2, n) float64 CUDA tensor."""
+    import torch
+    x = x_dev.contiguous()
+    out = torch.empty((2, x.shape[0]), dtype=torch.float64, device=x.device)
+    _check(load().weno_sums_selftest(_vp(_ptr(x)), int(x.shape[0]), _vp(_ptr(out))))
     return out
 
 
