@@ -197,11 +197,17 @@ weno_status weno_advance(weno_ctx* ctx, double t_end, int max_steps, int* steps_
  * status.  Errors: WENO_ERR_CUDA if capture or a launch fails. */
 weno_status weno_enqueue_steps(weno_ctx* ctx, double t_end, int nsteps);
 
+/* CTAs of the one launch that takes all steps of a short 1D line
+ * (weno_step, weno_advance, weno_enqueue_steps); 0: steps run as kernels per
+ * sweep, as on longer lines, with global Lax-Friedrichs splitting and in more
+ * than one dimension.  0 for NULL. */
+int weno_run1d_ctas(const weno_ctx* ctx);
+
 /* Measurement helper (no counterpart in the paper): times `reps` launches of
  * the sweep kernel of every direction on the current state (ghosts filled at
  * the current time; each sweep does its part of a right-hand side, the state
  * is not changed), each launch bracketed by CUDA events on the context's
- * stream.  A 1D line that steps in one launch has no sweep
+ * stream.  A 1D line that steps in one launch (weno_run1d_ctas) has no sweep
  * kernels of its own in a step; the time is then that of weno_rhs.
  * If flush_dev is not NULL, flush_bytes of it are overwritten before every
  * launch (to evict L2).  ms[d] receives the mean launch time of direction d,

@@ -1014,6 +1014,8 @@ static weno_status prepare_timing(weno_ctx* ctx)
     return WENO_OK;
 }
 
+int weno_run1d_ctas(const weno_ctx* ctx) { return ctx ? ctx->run1d : 0; }
+
 weno_status weno_time_sweeps(weno_ctx* ctx, int reps, void* flush_dev, size_t flush_bytes, double* ms,
                              unsigned long long* weno_faces)
 {

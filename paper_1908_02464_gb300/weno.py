@@ -85,6 +85,7 @@ SIGNATURES = {
     "weno_measure_fma_peak": (ctypes.c_int, [_ip, _dp, _dp]),
     "weno_arith_selftest": (ctypes.c_int, [_vp, ctypes.c_longlong, _vp]),
     "weno_sums_selftest": (ctypes.c_int, [_vp, ctypes.c_longlong, _vp]),
+    "weno_run1d_ctas": (ctypes.c_int, [_vp]),
     "weno_enqueue_steps": (ctypes.c_int, [_vp, ctypes.c_double, _ip]),
     "weno_autotune": (ctypes.c_int, [_vp, _ip, ctypes.POINTER(_ip)]),
     "weno_batch_create": (ctypes.c_int, [ctypes.POINTER(weno_batch_desc), ctypes.POINTER(weno_params), _vp,
@@ -410,6 +411,10 @@ class Solver:
 
     def time(self):
         return weno_get_time(self.ctx)
+
+    def run1d_ctas(self) -> int:
+        """CTAs of the one launch that takes all steps of a short 1D line (0: kernels per step)."""
+        return load().weno_run1d_ctas(_vp(self.ctx))
 
     def enqueue_steps(self, t_end: float, nsteps: int):
         weno_enqueue_steps(self.ctx, t_end, nsteps)
