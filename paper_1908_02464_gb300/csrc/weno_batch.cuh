@@ -48,13 +48,13 @@ struct BatchState {
     unsigned long long smax;     // CFL wave speed of the current state (bits)
     long long steps;
     int left;                    // runs of the current sweep not yet finished
+    int runs;                    // and how many there are
     int run;                     // tiles per run of the current sweep
     int phase;                   // sweep of the step: 1D the stage, 2D 2 stage + (0 y, 1 x)
     int cur;                     // work array (0 or 1) of the current state
     int clipped;                 // the step in progress ends at t_end
     int bad;                     // BAD_STAGE, BAD_CFL
     float dt_f;
-    int pad;
 };
 enum { BAD_STAGE = 1, BAD_CFL = 2 };
 
@@ -71,7 +71,8 @@ struct BatchCtrl {
     unsigned long long tail;           // tasks put into the queue
     unsigned long long progress;       // sweeps of all instances so far, and parts of long ones
     unsigned int prepared;             // instances taken for preparation
-    int finished;                      // instances
+    // polled by CTAs without a task, so not beside the counters they take from
+    alignas(128) int finished;         // instances
     int abort;                         // a wait for a task ran out
 };
 
@@ -185,13 +186,21 @@ __device__ __forceinline__ void batch_next_step(const BatchArgs& b, int inst, bo
     }
 }
 
+// Most tiles of a sweep that is never split: a run that another CTA takes costs
+// some 2 us in the queue and at the sweep's end, as much as a 1D tile in FP32
+// (one line of 200 cells: 136 us in runs of one tile, 113 us in one run).
+template <typename T, int DIM> constexpr int kBatchUnsplit = DIM == 1 && sizeof(T) == 4 ? 2 : 1;
+
 // One thread: moves an instance to its next sweep and reserves its places in
 // the queue: nr runs from place number `at` on.  Returns true when the
 // instance has finished instead.
-template <int DIM, typename CFG>
+template <typename T, int DIM, typename CFG>
 __device__ bool batch_next_sweep(const BatchArgs& b, int inst, bool first, int& nr, unsigned long long& at)
 {
     BatchState& s = b.state[inst];
+    // read beside the instance's progress, not after it
+    const unsigned long long head = *(volatile unsigned long long*)&b.ctrl->head,
+                             tail = *(volatile unsigned long long*)&b.ctrl->tail;
     const int nx = b.inst[inst].nx, ny = b.inst[inst].ny;
     atomicAdd(&b.ctrl->progress, 1ull);
     if (!first && s.phase + 1 < 3 * DIM) {
@@ -211,14 +220,15 @@ __device__ bool batch_next_sweep(const BatchArgs& b, int inst, bool first, int& 
     // FP32 148 ms against 121 ms here, 4096 boxes in FP32 75 against 70 ms, both
     // FP64 batches alike).  When CTAs wait for tasks, it is split for as many of
     // them as there are.
-    const long long idle = (long long)(*(volatile unsigned long long*)&b.ctrl->head -
-                                       *(volatile unsigned long long*)&b.ctrl->tail);
-    const int most = idle <= 0 ? 1 : (idle + 1 < nt ? (int)idle + 1 : nt), run = (nt + most - 1) / most;
+    const long long idle = (long long)(head - tail);
+    const int most = idle <= 0 || nt <= kBatchUnsplit<T, DIM> ? 1 : (idle + 1 < nt ? (int)idle + 1 : nt);
+    const int run = (nt + most - 1) / most;
     nr = (nt + run - 1) / run;
     s.run = run;
+    s.runs = nr;
     s.left = nr;
     // before the first sweep every run goes to the queue, later ones keep run 0
-    at = atomicAdd(&b.ctrl->tail, (unsigned long long)(first ? nr : nr - 1));
+    if (first || nr > 1) at = atomicAdd(&b.ctrl->tail, (unsigned long long)(first ? nr : nr - 1));
     return false;
 }
 
@@ -263,7 +273,7 @@ __device__ __forceinline__ bool batch_take(const BatchArgs& b, int& inst, int& r
         unsigned int v;
         asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&q->turn) : "memory");
         if (v == (unsigned int)turn + 1u) break;
-        if ((k & 7) == 7) {
+        if ((k & 3) == 0) {   // at once, so that a run ends soon after its last instance
             if (*(volatile int*)&b.ctrl->finished >= b.count || *(volatile int*)&b.ctrl->abort != 0) return false;
             if (k >= b.polls) {
                 const unsigned long long now = *(volatile unsigned long long*)&b.ctrl->progress;
@@ -289,6 +299,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
     constexpr int NT = CFG::NT, NV = DIM + 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_inst, s_run, s_done;
+    __shared__ bool s_alone;
     unsigned int wenos = 0;
     const int lane = threadIdx.x & 31;
     const T gamma = pick<T>(b.gamma, b.gamma_f);
@@ -313,11 +324,15 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             int done = 0, nr = 0;   // done: 0 others still work on the sweep, 1 finished, 2 go on
             unsigned long long at = 0ull;
             if (threadIdx.x == 0) {
-                __threadfence();
-                if (first || atomicSub(&b.state[inst].left, 1) == 1) {
-                    __threadfence();
-                    done = batch_next_sweep<DIM, CFG>(b, inst, first, nr, at) ? 1 : 2;
-                    __threadfence();
+                // A sweep of one run has nothing to take over from other CTAs
+                // and, if the next one is too, nothing to publish (2000 lines
+                // of 20 to 60 cells in FP32 127 us with them, 98 us without).
+                const bool alone = !first && s_alone;
+                if (!alone) __threadfence();
+                if (first || alone || atomicSub(&b.state[inst].left, 1) == 1) {
+                    if (!alone) __threadfence();
+                    done = batch_next_sweep<T, DIM, CFG>(b, inst, first, nr, at) ? 1 : 2;
+                    if (first || nr > 1) __threadfence();
                 }
                 s_done = done;
             }
@@ -326,7 +341,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
             // the shuffles order no memory: the tasks that the other lanes
             // publish come after lane 0's stores, and the stores it acquired
             __syncwarp();
-            if (nr > 0) batch_put(b, inst, first ? 0 : 1, nr, at);
+            if (first || nr > 1) batch_put(b, inst, first ? 0 : 1, nr, at);
         }
         __syncthreads();
         const int done = s_done;
@@ -396,6 +411,7 @@ __global__ void __launch_bounds__(CFG::NT, CFG::template min_blocks<T>()) k_batc
         BatchState& s = b.state[inst];
         const BatchInst q = b.inst[inst];
         const int phase = s.phase, cur = s.cur, len = s.run;
+        if (threadIdx.x == 0) s_alone = s.runs == 1;
         const T dt = pick<T>(s.dt, s.dt_f);
         const int t0 = run * len;
         // three stages: x = cur + dt L(cur); y = 3/4 cur + 1/4 (x + dt L(x));
