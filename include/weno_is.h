@@ -226,7 +226,7 @@ weno_status weno_time_sweeps(weno_ctx* ctx, int reps, void* flush_dev, size_t fl
  * and mixed sweeps across x (y, z) by marching warps, one lane per line
  * along a segment of 12 (2D) or 18 (3D) cells with the six-cell stencil
  * in registers (FP32 along x takes 3, FP64 takes 5).  Defaults go
- * by the grid's size: FP64 5, or 2 across x and on lines too short for 5; FP32
+ * by the grid's size: FP64 5, or 2 on many short lines and across x; FP32
  * and mixed 3, 4, 5 or 2 along x, whichever fills its tiles, 1 across, 7
  * across when lines x segments reach four rounds of 16 warps on every SM.
  * variants[3] (if not NULL) receives the choice per direction.

@@ -357,42 +357,64 @@ static weno_status read_time(weno_ctx* ctx)
     return WENO_OK;
 }
 
-// Default tile of direction d (variants of weno_launch.cuh; the times are
-// sweeps on one GB300, us).
+// Default tile of direction d (variants of weno_launch.cuh).  A tile of several
+// short lines fills its CTA, which pays when there are many tiles: a CTA's time
+// is that of its WENO faces, so on a grid of few tiles four lines in one CTA
+// take up to four times as long as one.  Measured on one GB300 as the time of a
+// whole RK3 step (2D) or operator (3D) with 4 x 31 tiles over that with one-line
+// tiles, on a periodic state with discontinuities (mixed) and without (smooth).
 static int default_tile(const weno_ctx* c, int d)
 {
     const int n = c->n[d];
-    const bool f64 = c->prec == WENO_FP64;
-    // lines shorter than a flat tile: the shape with the fewest tiles per
-    // line, between 1 x 127, 4 x 31 and (FP32) 2 x 63
-    auto per_line = [&](int seg, int lines) { return (double)((n + seg - 1) / seg) / lines; };
-    if (!f64) {
+    const long long lines = (long long)c->n[0] * c->n[1] * c->n[2] / n, nsm = c->nsm;
+    if (c->prec != WENO_FP64) {
         if (d > 0) return 1;   // 8 x 15: coalesced rows
-        // Along x the last tile of a line may be nearly empty (256 cells in
-        // 1 x 127 tiles: a third of the work on 2 cells).  1 x 127, or 1 x 95
-        // where that fills better (256^3 x-sweep 486 -> 390), or flat tiles
-        // (128^3: 79 -> 57), or several short lines (55 cells: 13.3 -> 11.3)
+        // Along x.  4 x 31 for lines of one or two such pieces on large grids:
+        // 31 cells 1.01 (mixed) and 1.05 (smooth) at 1600 lines in 2D, 0.80 and
+        // 0.97 in 3D, 0.82 and 0.71 at 6400; 62 cells 1.14 and 0.97 at 1600, 0.95
+        // and 0.87 at 6400; 80 cells 1.02 and 1.01 at 6400.
+        if ((n <= 31 && lines > 8 * nsm) || (n <= 62 && lines > 20 * nsm)) return 2;
+        // The last tile of a longer line may be nearly empty (256 cells in 1 x
+        // 127 tiles: a third of the work on 2 cells): 1 x 95 where it fills
+        // better by a tenth (256 cells 0.91, 190 0.97, 170 0.94 of the 1 x 127
+        // tiles' time; 300, filled alike, 1.01, and 200, filled worse, 1.05),
+        // flat tiles where neither fills to three quarters (130 cells 0.92; at 200
+        // and 400, filled to 0.79 and 0.84, 1.05).
         const double e3 = n / (127.0 * ((n + 126) / 127)), e4 = n / (95.0 * ((n + 94) / 95));
-        if (e3 >= 0.85 && e3 >= e4 - 0.05) return 3;
-        if (e4 >= 0.85) return 4;
-        if (n >= wis::Tile<5>::SEG) return 5;
-        return per_line(31, 4) < per_line(127, 1) ? 2 : 3;
+        if (n >= wis::Tile<5>::SEG && e3 < 0.75 && e4 < 0.75) return 5;
+        // (Lines of one tile: 1 x 95, 0.95 of the 1 x 127 tiles' time at 45 to 80 cells.)
+        return n <= 95 || e4 > e3 + 0.1 ? 4 : 3;
     }
-    if (d == 0) return n >= wis::Tile<5>::SEG || per_line(31, 4) >= per_line(127, 1) ? 5 : 2;
-    // Across x, 4 x 31: four x-adjacent lines share the 32-byte sectors of the
-    // strided loads (256^3: y 3524 -> 3130, z 4046 -> 3933).
-    if (c->dim == 3) return 2;
-    // In 2D the flat tiles of long lines win or tie (RK3 steps of 2048 x 512
-    // 1707 against 1732, 1000 x 250 540 against 590); 4 x 31 wins on shorter
-    // ones (637 x 159: 290 against 306, 1651 x 135: y-sweep 76 against 85)
-    // unless the grid has fewer such tiles than the chip holds CTAs, where the
-    // time of one tile counts (512 x 128: 304 against 283); and on lines that
-    // leave most of a one-line tile empty (700 x 45: 119 against 171) unless
-    // even the one-line tiles are too few (177 x 70: 168 against 134).
-    const long long tiles = (long long)((c->n[0] + 3) / 4) * ((n + 30) / 31);
-    if (n < wis::Tile<5>::SEG) return c->n[0] > 2 * c->nsm && per_line(31, 4) < 0.8 ? 2 : 5;
-    if (n >= 192) return 5;
-    return tiles > 5LL * c->nsm ? 2 : 5;
+    const bool lf = c->p.splitting == wis::SPLIT_LF;   // its speeds' kernel before every sweep hides nothing of a tile's time
+    // Very short lines of a 3D grid whose 4 x 31 tiles are about one per SM: 24
+    // cells 0.85 at 400 lines, 0.80 at 576 along x and z, 1.16 at 1024; 31 cells
+    // 1.11 at 400.
+    if (c->dim == 3 && n <= 24 && lines > 2 * nsm && lines <= 4 * nsm) return 2;
+    if (d == 0) {
+        // 4 x 31 along x: 31 cells 1.16 at 1024 lines of a 3D grid, 1.00 and 0.85
+        // at 1920; in 2D 1.00 and 0.85 at 700 lines, 0.95 and 0.83 at 1500, with
+        // global Lax-Friedrichs 1.12 at 1500 and 0.94 at 4000.  45 and 62 cells:
+        // 1.15 and 0.97 at 1500 lines in 2D, 1.00 and 0.94 at 1920 in 3D.
+        const bool many = lines > (lf ? 25 : 10) * nsm;
+        return many && n <= (c->dim == 3 ? 62 : 31) ? 2 : 5;
+    }
+    // Across x four x-adjacent lines share the 32-byte sectors of the strided
+    // loads (256^3: y sweep 3524 -> 3130 us, z 4046 -> 3933).
+    // z: 31 cells 1.21 at 1024 lines, 0.98 at 1920; 62 cells 1.30 at 400, 1.05
+    // at 1024, 1.00 and 0.94 at 1920; 121 cells 1.00 at 1920.
+    if (c->dim == 3) return d == 1 || lines > 10 * nsm ? 2 : 5;
+    // y in 2D, lines short of a flat tile: 45 cells 1.24 and 1.05 at 304 lines,
+    // 1.16 and 1.01 at 500, 0.91 and 0.73 at 700, 0.97 and 0.97 at 1500 (at 1000
+    // lines 1.19 and 0.99); 80 cells 1.23 at 304, 1.10 at 700, 0.99 at 1000; 100
+    // cells 1.08 at 700, 0.94 at 1000.  With global Lax-Friedrichs 45 cells 1.21 at
+    // 700, 1.35 at 1000, 1.06 at 1500, 0.94 (40 cells) at 2000 and at 4000.
+    if (n < wis::Tile<5>::SEG) return n <= 93 && lines > (lf ? 12 : 4) * nsm ? 2 : 5;
+    // Longer ones: 4 x 31 where they are up to six full pieces and the tiles
+    // number more than the CTAs that the chip holds (637 x 159: y sweep 46.6 ->
+    // 39.1 us, 512 x 128 step 283 us with flat tiles and 304 with these; 170 cells
+    // 0.96 at 700 lines, 191 cells, seven pieces, 1.03).
+    const long long tiles = ((c->n[0] + 3) / 4) * (long long)((n + 30) / 31);
+    return n <= 6 * 31 && tiles > 5 * nsm ? 2 : 5;
 }
 
 // ----------------------------------------------------------- ABI
