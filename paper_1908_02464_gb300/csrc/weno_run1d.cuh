@@ -35,10 +35,13 @@ struct Run1DArgs {
 };
 
 constexpr int kRun1DThreads = 128;
-// Cells of one CTA.  FP32 lines of 8000 cells step in 16 us against 24 us with
-// kernels per step; FP64 ones of 4000 in 64 against 72 us, of 8000 in 97
-// against 83 us, so FP64 segments end at 256 cells.
-template <typename T> constexpr int run1d_cells() { return sizeof(T) == 8 ? 256 : 512; }
+// Cells of one CTA, which end where the kernels per step are as fast.  FP64, one
+// round of faces: 40 steps of a line of 2000 cells 54 us each against 67 (27
+// against 35 on a smooth state), of 2500, which took a second round, 66 against
+// 66 (38 against 35), of 4000 70 against 57.  FP32, four rounds: 14 us against 19
+// at 4000 cells, 18 against 19 at 8000 (calls of one step 51 against 46 there,
+// 42 against 46 at 4000).
+template <typename T> constexpr int run1d_cells() { return sizeof(T) == 8 ? 128 : 512; }
 // the fewest cells worth a CTA of its own
 constexpr int kRun1DMinCells = 12;
 constexpr int kRun1DMaxCluster = 16;
