@@ -675,15 +675,20 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
     const int mode = FIRST ? MODE_ACC_SET : a.mode;
     T ea[NV], en[NV];
     if constexpr (EARLY) {
-        long long g = 0;
-        int l = 0, fl = 0, fr_ = 0, cpos = 0;
-        const bool read = mode != MODE_ACC_SET && out_cell(g, l, fl, fr_, cpos);
-        const T* accr = reinterpret_cast<const T*>(a.acc);
-        const T* Unr = reinterpret_cast<const T*>(a.Un);
+        // 1D has no accumulator, and only a combination that takes a base state
+        // loads one (operator on a million cells 61.3 -> 58.6 us; 58.2 without
+        // early loads, which then cost a step of 20000 cells 24.2 us against 23.2)
+        if (DIM > 1 || (mode == MODE_COMBINE && rka != T(0))) {
+            long long g = 0;
+            int l = 0, fl = 0, fr_ = 0, cpos = 0;
+            const bool read = mode != MODE_ACC_SET && out_cell(g, l, fl, fr_, cpos);
+            const T* accr = reinterpret_cast<const T*>(a.acc);
+            const T* Unr = reinterpret_cast<const T*>(a.Un);
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            ea[v] = read && accr != nullptr ? accr[g + v * a.sv] : T(0);
-            en[v] = read && mode == MODE_COMBINE && rka != T(0) ? Unr[g + v * a.sv] : T(0);
+            for (int v = 0; v < NV; ++v) {
+                if constexpr (DIM > 1) ea[v] = read && accr != nullptr ? accr[g + v * a.sv] : T(0);
+                en[v] = read && mode == MODE_COMBINE && rka != T(0) ? Unr[g + v * a.sv] : T(0);
+            }
         }
     }
 
@@ -873,7 +878,7 @@ __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int 
 #pragma unroll
             for (int v = 0; v < NV; ++v) {
                 tot[v] = (fh[v * NFACE + fl] - fh[v * NFACE + fr_]) * inv_dx;
-                if (accp) tot[v] = fmaT(EARLY ? ea[v] : accp[g + v * a.sv], acs, tot[v]);
+                if (DIM > 1 && accp) tot[v] = fmaT(EARLY ? ea[v] : accp[g + v * a.sv], acs, tot[v]);
             }
             if (mode != MODE_COMBINE) {
                 T* o = mode == MODE_ACC_ADD ? accp : outp;
