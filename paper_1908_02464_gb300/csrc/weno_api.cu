@@ -11,9 +11,9 @@
 //   k_next (t += dt, steps += 1 unless a stage failed; the next dt, and the
 //            boundary times t, t+dt, t+dt/2)
 // A call begins with k_cfl(cur), which does nothing when the last step has
-// left its wave speeds, and k_begin (dt towards the call's target time).  CFL,
-// dt and bookkeeping kernels in every step took 13 of 206 us on the 2048 x 512
-// grid in mixed precision and 14 of 300 us on 512 x 128 in FP64.
+// left its wave speeds, and k_begin (dt towards the call's target time).
+// Separate CFL, dt and bookkeeping kernels took 18 of 225 us of kernel time per
+// step on the 2048 x 512 grid in mixed precision.
 // The sweeps take the ghost cells from the boundary conditions at the
 // stage's time while staging their tiles; no ghost-cell kernel runs.
 // The new state is x, i.e. buffer (phase + 1) mod 3.  A failed admissibility

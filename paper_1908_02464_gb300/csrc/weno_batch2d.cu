@@ -14,8 +14,10 @@ namespace wis {
 // their loads are row pieces.  1024 explosions in FP64: 59, 57 and 60 ms (one
 // CTA per instance: 103, 106 and 150 ms); with the primitives shared between
 // the sweeps the first takes 55 ms.  4096 boxes of 16 to 64 cells a side in
-// FP32: 70, 72 and 94 ms with 16 warps per SM (64 registers a thread; 112 to 124
-// registers and half as many warps took half as long again).
+// FP32: 70, 72 and 94 ms with 32 warps per SM (64 registers a thread; 112 to 124
+// registers and half as many warps took half as long again).  2000 boxes of 8
+// to 20 cells, one or two tiles a sweep, are the other way round: 2.9 ms, 2.2 ms
+// with one CTA per instance and the larger number of registers.
 template <int V> struct Batch2Shape;
 template <> struct Batch2Shape<0> { static constexpr int NT = 128, XL = 4, XS = 31, YL = 8, YS = 15; };
 template <> struct Batch2Shape<1> { static constexpr int NT = 128, XL = 2, XS = 63, YL = 4, YS = 31; };

@@ -142,13 +142,15 @@ struct SweepArgs {
 };
 
 // FP64 problems of at least this many cells form their six-point sums on the
-// integer pipes (fx_detector, fx_central_flux), in the grid solver and in the
-// batches alike, so that both give the same bits.  There the FP64 pipe bounds
-// the sweeps: double Mach 2048 x 512 RK3 step 2.21 -> 1.72 ms, 512 x 128 (the
-// next smaller size measured) 0.346 -> 0.304 ms.  A few thousand cells do not
-// fill the pipe, the longer integer sequence gains little (Sod, 200 cells:
-// 5%), and the whole runs of thousands of such instances in one batch keep
-// the FP64 form.
+// integer pipes (fx_detector, fx_central_flux).  RK3 step with integer over FP64
+// sums on a grid with discontinuities (mixed) and without (smooth): 64 x 64 132
+// over 129 us and 64 over 62, 128 x 128 167 over 164 and 76 over 73, 182 x 180
+// 223 over 233 and 93 over 103, 256 x 256 385 over 427 and 150 over 189.  Smaller
+// grids do not fill the FP64 pipe, and the longer integer sequence adds to a
+// tile's time.  Batches follow the same rule per instance, so that an instance
+// has the grid solver's bits; most of their instances are below it, although a
+// batch does fill the pipe (1024 Riemann problems 52 over 63 ms, 1024 explosions
+// 51 over 56).
 constexpr long long kFxMinCells = 32768;
 __host__ __device__ inline bool use_fx(long long cells) { return cells >= kFxMinCells; }
 
@@ -458,24 +460,7 @@ __device__ __forceinline__ void weno_queue(const SweepArgs& a, int nq, const T* 
     }
 }
 
-// One tile of the sweep: stage, faces, WENO queue, divergence and output.
-// EXACTDET: detector difference by nested differences (mixed precision);
-// otherwise the direct six-term combination.  dt is the RK step (COMBINE
-// mode only).  Returns true in every thread whose cells failed the
-// admissibility check.  Ends with a barrier, so tiles can be chained by one
-// CTA (the batched solver) reusing the same shared memory.
-//
-// Regular tiles hold LINES lines of SEG cells starting at cell seg_blk * SEG.
-// A flat tile (LINES = 1, lines of at least SEG cells) holds SEG + 1
-// consecutive faces of the sequence of all lines' faces (line after line,
-// nd + 1 faces each), starting at face seg_blk * SEG: every tile computes a
-// full set of faces, and a tile that reaches the end of a line continues on
-// the next one, each piece with its own halo.  line0 and pb are unused then.
-// FX: a.fx may ask for the integer six-point sums (FP64).
-// FIRST: a.mode is MODE_ACC_SET, known when compiled (the first sweep of a
-// float stage then holds no registers for the accumulator and base state).
-// cfl (COMBINE mode, may be null): the CFL wave speeds of the cells written
-// (cell_speed), for the step that follows.
+// the CFL wave speeds of the cells that a tile writes
 template <typename T, int DIM>
 struct TileCfl {
     T inv_dx[DIM];   // 1 / dx per direction
@@ -497,6 +482,25 @@ struct TileCfl {
         if (bad) atomicOr(&tm->cfl_bad, 1);
     }
 };
+
+// One tile of the sweep: stage, faces, WENO queue, divergence and output.
+// EXACTDET: detector difference by nested differences (mixed precision);
+// otherwise the direct six-term combination.  dt is the RK step (COMBINE
+// mode only).  Returns true in every thread whose cells failed the
+// admissibility check.  Ends with a barrier, so tiles can be chained by one
+// CTA (the batched solver) reusing the same shared memory.
+//
+// Regular tiles hold LINES lines of SEG cells starting at cell seg_blk * SEG.
+// A flat tile (LINES = 1, lines of at least SEG cells) holds SEG + 1
+// consecutive faces of the sequence of all lines' faces (line after line,
+// nd + 1 faces each), starting at face seg_blk * SEG: every tile computes a
+// full set of faces, and a tile that reaches the end of a line continues on
+// the next one, each piece with its own halo.  line0 and pb are unused then.
+// FX: a.fx may ask for the integer six-point sums (FP64).
+// FIRST: a.mode is MODE_ACC_SET, known when compiled (the first sweep of a
+// float stage then holds no registers for the accumulator and base state).
+// cfl (COMBINE mode, may be null): the CFL wave speeds of the cells written
+// (cell_speed), for the step that follows.
 template <typename T, int DIM, int DIR, int LINES, int SEG, int NT, bool EXACTDET, bool FLAT = false,
           bool FX = sizeof(T) == 8, bool FIRST = false>
 __device__ __forceinline__ bool sweep_tile(const SweepArgs& a, int seg_blk, int line0, int pb, T dt,

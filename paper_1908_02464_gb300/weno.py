@@ -556,7 +556,8 @@ class Batch:
         return weno_batch_autotune(self.handle, U_dev, trial_steps)
 
     def set_config(self, variant: int, blocks_per_sm: int = 0) -> int:
-        """Fix the tile variant and residency without timing; returns the CTAs a run launches."""
+        """Fix the tile variant and residency without timing; returns min(instances, residency x SMs), the
+        instances that can have a task in work at once (a run launches min(tiles, residency x SMs) CTAs)."""
         b = ctypes.c_int(0)
         _bcheck(load().weno_batch_set_config(self.handle, int(variant), int(blocks_per_sm), ctypes.byref(b)),
                 self.handle)
