@@ -502,7 +502,7 @@ weno_status weno_batch_set_wait(weno_batch* bt, int polls)
         bt->err = "set_wait: negative number of polls";
         return WENO_ERR_INVALID_ARG;
     }
-    bt->polls = polls > 0 ? polls : wis::kTaskPolls;
+    bt->polls = polls > 0 ? std::min(polls, 1 << 30) : wis::kTaskPolls;   // the counter of polls stays an int
     if (bt->graph) cudaGraphExecDestroy(bt->graph);   // it holds the old number
     bt->graph = nullptr;
     return WENO_OK;

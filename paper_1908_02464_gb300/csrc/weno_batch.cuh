@@ -158,7 +158,9 @@ __device__ __forceinline__ void batch_next_step(const BatchArgs& b, int inst, bo
     double t = s.t, dt = 0.0;
     long long steps = s.steps;
     int clipped = s.clipped;
-    const int bad = s.bad;
+    // what the sweep's warps noted by atomics, past this SM's L1
+    const int bad = *(volatile int*)&s.bad;
+    const unsigned long long smax = *(volatile unsigned long long*)&s.smax;
     if (!first) {
         if (bad & BAD_STAGE) {
             status = WENO_ERR_NONPHYSICAL;   // the state before the step stays
@@ -170,7 +172,7 @@ __device__ __forceinline__ void batch_next_step(const BatchArgs& b, int inst, bo
     }
     if (status == 0 && steps < max_steps) {
         if (bad & BAD_CFL) status = WENO_ERR_NONPHYSICAL;
-        else dt = cfl_step(b.cfl, __longlong_as_double((long long)s.smax), t, t_end, &clipped);
+        else dt = cfl_step(b.cfl, __longlong_as_double((long long)smax), t, t_end, &clipped);
     }
     s.t = t;
     s.steps = steps;
